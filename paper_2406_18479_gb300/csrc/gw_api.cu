@@ -129,6 +129,13 @@ struct gw_ctx {
   long long *tab_kkpq = nullptr, *tab_kpqk = nullptr, *tab_gkpq = nullptr;
   long long *tab_kkmq = nullptr, *tab_kmqk = nullptr, *tab_gkmq = nullptr;
   double2* work = nullptr;                // contraction intermediates, nt * 2 * nk * pair
+  // Digit workspaces of the tensor-core FP64 products. Those of the transforms and of the products
+  // outside the contractions lie in a P array that is not in use (oz_buf): P~ during a transform to
+  // Matsubara, P0(tau) during one to tau, P(i Omega) otherwise; digits of up to kOz64L2Bytes stay in
+  // the 129 MB L2 between the packing and the GEMM. The FP64 contractions have their own (oz_mem).
+  unsigned char *oz_mem = nullptr, *oz_small = nullptr, *oz_count = nullptr;
+  size_t oz_bytes = 0;
+  Oz64Ws oz_fwd, oz_back, oz_w, oz;
   double2 *P0t = nullptr, *Pw = nullptr, *Pt = nullptr;
   double2* dyson_ws = nullptr;            // nk * nwf * nao2
   std::vector<int> mq;                    // index of -q for every q
@@ -215,7 +222,7 @@ void free_ctx(gw_ctx* c) {
   mixed_destroy(c->mixed);
   void* ptrs[] = {c->Fb, c->Bb, c->Ff, c->Bf, c->wf, c->tabs, c->mq_dev, c->wlist, c->wlist_q, c->work, c->P0t, c->Pw,
                   c->Pt, c->dyson_ws, c->status, c->maxdiff, c->nonfinite, c->wbeta, c->gamma, c->rho,
-                  c->xinf, c->scal, c->gw_w, c->heff, c->gf2_ws, c->Vfull, c->cw_tmp};
+                  c->xinf, c->scal, c->gw_w, c->heff, c->gf2_ws, c->Vfull, c->cw_tmp, c->oz_mem, c->oz_small, c->oz_count};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete c;
@@ -251,6 +258,33 @@ int canonical_end(const gw_ctx* c, int q, int T, int q0, int q1) {
   return (c->mq[q] < q0 || c->mq[q] >= q1) ? T : canonical_end(c, q, T);
 }
 
+// The V.G products of nt tau nodes from t0, for the nk blocks of V at vtab, out [t][k][pair]:
+//   plain      out[Q][i][b] = sum_a V_ia(Q) G_ab(t0 + t)            (G of k at gtab, or k gstep)
+//   mirrored   out[Q'][d][b] = sum_c V_bc(Q') G_cd(beta - (t0 + t))
+// as one product per k over the joined rows of all nodes, so that row tiles fill whatever nao is.
+int vg_fp64(gw_ctx* c, const long long* vtab, const double2* G, const long long* gtab, long long gstep, int t0, int nt,
+            bool mirrored, double2* out) {
+  const int nk = c->nk, nao = c->nao, naux = c->naux;
+  const long long nao2 = c->nao2, pair = c->pair;
+  ZGemm g;
+  g.K = nao; g.nbatch = nk; g.slot = SLOT_VG_FP64; g.ws = &c->oz; g.C = out; g.bc.bs_in = pair;
+  g.unit = (double)naux * nao * nao * nao;
+  if (!mirrored) {   // rows (t, b) of G^T, columns (Q, i) of V
+    g.M = nt * nao; g.N = naux * nao;
+    g.A = G + (long long)t0 * nao2; g.va.rin = nao; g.va.rs_in = 1; g.va.rs_out = nao2; g.va.ks_in = nao;
+    g.ba.tab = gtab; g.ba.bs_in = gstep;
+    g.B = c->V; g.vb.rs_in = nao; g.vb.ks_in = 1; g.bb.tab = vtab;
+    g.vc.rin = nao; g.vc.rs_in = 1; g.vc.rs_out = (long long)nk * pair; g.vc.ks_in = nao;
+  } else {           // rows (Q', b) of V, columns (t, d) of G at the mirrored node
+    g.M = naux * nao; g.N = nt * nao;
+    g.A = c->V; g.va.rs_in = nao; g.va.ks_in = 1; g.ba.tab = vtab;
+    g.B = G + (long long)(c->ntau - 1 - t0) * nao2; g.vb.rin = nao; g.vb.rs_in = 1; g.vb.rs_out = -nao2; g.vb.ks_in = nao;
+    g.bb.tab = gtab; g.bb.bs_in = gstep;
+    g.vc.rin = nao; g.vc.rs_in = 1; g.vc.rs_out = nao2; g.vc.kin = nao; g.vc.ks_in = nao; g.vc.ks_out = (long long)nk * pair;
+  }
+  return zgemm_fp64(g, c->stream);
+}
+
 int polarization_fp64(gw_ctx* c, const double2* G, double2* P0t, int q0, int q1) {
   const int nk = c->nk, nao = c->nao, naux = c->naux, ntau = c->ntau;
   const long long nao2 = c->nao2, pair = c->pair;
@@ -260,27 +294,10 @@ int polarization_fp64(gw_ctx* c, const double2* G, double2* P0t, int q0, int q1)
       const int nt = std::min(c->nt, tend - t0);
       double2* Abuf = c->work;
       double2* Bbuf = c->work + (long long)c->nt * nk * pair;
-      {  // A^Q_{db}(k,t) = sum_a V^{k,k+q}_da(Q) G^{k+q}_ab(t)
-        ZGemm g;
-        g.M = naux * nao; g.N = nao; g.K = nao; g.nbatch = nt * nk; g.bin = nk;
-        g.A = c->V; g.va.rs_in = nao; g.va.ks_in = 1; g.ba.tab = c->tab_kkpq + (long long)q * nk;
-        g.B = G + (long long)t0 * nao2; g.vb.rs_in = 1; g.vb.ks_in = nao;
-        g.bb.tab = c->tab_gkpq + (long long)q * nk; g.bb.bs_out = nao2;
-        g.C = Abuf; g.vc.rs_in = nao; g.vc.ks_in = 1; g.bc.bs_in = pair; g.bc.bs_out = (long long)nk * pair;
-        g.slot = SLOT_VG_FP64;
-        GW_TRY(zgemm_fp64(g, c->stream));
-      }
-      {  // B^{Q'}_{bd}(k,t) = sum_c V^{k+q,k}_bc(Q') G^k_cd(beta - t), stored as [Q'][d][b]
-        ZGemm g;
-        g.M = naux * nao; g.N = nao; g.K = nao; g.nbatch = nt * nk; g.bin = nk;
-        g.A = c->V; g.va.rs_in = nao; g.va.ks_in = 1; g.ba.tab = c->tab_kpqk + (long long)q * nk;
-        g.B = G + (long long)(ntau - 1 - t0) * nao2; g.vb.rs_in = 1; g.vb.ks_in = nao;
-        g.bb.bs_in = (long long)ntau * nao2; g.bb.bs_out = -nao2;
-        g.C = Bbuf; g.vc.rin = nao; g.vc.rs_in = 1; g.vc.rs_out = nao2; g.vc.ks_in = nao;
-        g.bc.bs_in = pair; g.bc.bs_out = (long long)nk * pair;
-        g.slot = SLOT_VG_FP64;
-        GW_TRY(zgemm_fp64(g, c->stream));
-      }
+      // A^Q_{db}(k,t) = sum_a V^{k,k+q}_da(Q) G^{k+q}_ab(t), stored [Q][d][b]
+      GW_TRY(vg_fp64(c, c->tab_kkpq + (long long)q * nk, G, c->tab_gkpq + (long long)q * nk, 0, t0, nt, false, Abuf));
+      // B^{Q'}_{bd}(k,t) = sum_c V^{k+q,k}_bc(Q') G^k_cd(beta - t), stored [Q'][d][b]
+      GW_TRY(vg_fp64(c, c->tab_kpqk + (long long)q * nk, G, nullptr, (long long)ntau * nao2, t0, nt, true, Bbuf));
       {  // P0^q_QQ'(t) = -(s/N_k) sum_{k,d,b} A^Q_{db} B^{Q'}_{bd}
         ZGemm g;
         g.M = naux; g.N = naux; g.K = nk * (int)nao2; g.nbatch = nt;
@@ -291,6 +308,7 @@ int polarization_fp64(gw_ctx* c, const double2* G, double2* P0t, int q0, int q1)
         g.bc.bs_in = c->naux2;
         g.alpha = -c->cfg.spin_factor / nk;
         g.slot = SLOT_P0_FP64;
+        g.ws = &c->oz;
         GW_TRY(zgemm_fp64(g, c->stream));
       }
     }
@@ -316,18 +334,11 @@ int self_energy_fp64(gw_ctx* c, const double2* G, const double2* Pt, double2* Si
         g.B = c->V; g.vb.rs_in = 1; g.vb.ks_in = nao2; g.bb.tab = c->tab_kmqk + (long long)q * nk;
         g.C = Rbuf; g.vc.rs_in = nao2; g.vc.ks_in = 1; g.bc.bs_in = pair; g.bc.bs_out = (long long)nk * pair;
         g.slot = SLOT_R_FP64;
+        g.ws = &c->oz;
         GW_TRY(zgemm_fp64(g, c->stream));
       }
-      {  // Z^Q_{ib}(k,t) = sum_a V^{k,k-q}_ia(Q) G^{k-q}_ab(t)
-        ZGemm g;
-        g.M = naux * nao; g.N = nao; g.K = nao; g.nbatch = nt * nk; g.bin = nk;
-        g.A = c->V; g.va.rs_in = nao; g.va.ks_in = 1; g.ba.tab = c->tab_kkmq + (long long)q * nk;
-        g.B = G + (long long)t0 * nao2; g.vb.rs_in = 1; g.vb.ks_in = nao;
-        g.bb.tab = c->tab_gkmq + (long long)q * nk; g.bb.bs_out = nao2;
-        g.C = Zbuf; g.vc.rs_in = nao; g.vc.ks_in = 1; g.bc.bs_in = pair; g.bc.bs_out = (long long)nk * pair;
-        g.slot = SLOT_VG_FP64;
-        GW_TRY(zgemm_fp64(g, c->stream));
-      }
+      // Z^Q_{ib}(k,t) = sum_a V^{k,k-q}_ia(Q) G^{k-q}_ab(t), stored [Q][i][b]
+      GW_TRY(vg_fp64(c, c->tab_kkmq + (long long)q * nk, G, c->tab_gkmq + (long long)q * nk, 0, t0, nt, false, Zbuf));
       {  // Sigma^k_ij(t) += -(1/N_k) sum_{Q,b} Z^Q_{ib} R^Q_{bj}
         ZGemm g;
         g.M = nao; g.N = nao; g.K = naux * nao; g.nbatch = nt * nk; g.bin = nk;
@@ -340,6 +351,7 @@ int self_energy_fp64(gw_ctx* c, const double2* G, const double2* Pt, double2* Si
         g.alpha = -1.0 / nk;
         g.accumulate = 1;
         g.slot = SLOT_SIGMA_FP64;
+        g.ws = &c->oz;
         GW_TRY(zgemm_fp64(g, c->stream));
       }
     }
@@ -361,6 +373,7 @@ int transform(gw_ctx* c, int stat, bool forward, const double2* in, double2* out
     g.B = in + (long long)b0 * nin * nelem; g.vb.rs_in = 1; g.vb.ks_in = nelem; g.bb.bs_in = nin * nelem;
     g.C = out + (long long)b0 * nout * nelem; g.vc.rs_in = nelem; g.vc.ks_in = 1; g.bc.bs_in = nout * nelem;
     g.slot = SLOT_TRANSFORM_FP64;
+    g.ws = stat == 0 ? (forward ? &c->oz_fwd : &c->oz_back) : &c->oz_w;
     GW_TRY(zgemm_fp64(g, c->stream));
   }
   return GW_OK;
@@ -379,6 +392,7 @@ int transform_q(gw_ctx* c, int stat, bool forward, const double2* in, double2* o
   g.B = in + (long long)q * nin * nelem; g.vb.rs_in = 1; g.vb.ks_in = nelem;
   g.C = out + ((long long)q * nout + row0) * nelem; g.vc.rs_in = nelem; g.vc.ks_in = 1;
   g.slot = SLOT_TRANSFORM_FP64;
+  g.ws = stat == 0 ? (forward ? &c->oz_fwd : &c->oz_back) : &c->oz_w;
   return zgemm_fp64(g, c->stream);
 }
 
@@ -572,6 +586,14 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
     int nt = cfg->tau_chunk > 0 ? cfg->tau_chunk : (int)std::max(1.0, std::floor(4294967296.0 / per_t));
     c->nt = std::min(nt, c->ntau);
     if (cfg->precision == GW_FP64) {
+      // The digits of the contractions take three times their intermediates. An automatic tau batch
+      // shares its memory between both, so that a context needs no more than its intermediates alone
+      // would at the full batch (64 MiB where that is less); a given one gets digits for as much memory
+      // again. More digits than fit are made in pieces, with the same result.
+      const double dig_t = (double)oz64_bytes(c->naux, c->naux, nk * (int)c->nao2);
+      const double budget = std::max(c->nt * per_t, 67108864.0);
+      if (cfg->tau_chunk <= 0) c->nt = std::max(1, std::min(c->nt, (int)(budget / (per_t + dig_t))));
+      c->oz_bytes = (size_t)std::min(c->nt * dig_t, cfg->tau_chunk > 0 ? budget : std::max(budget - c->nt * per_t, 0.0));
       if ((rc = dev_alloc(c, &c->work, (size_t)c->nt * 2 * nk * c->pair)) != GW_OK) break;
       if (cfg->v_packed && (rc = dev_alloc(c, &c->Vfull, (size_t)nk * nk * c->pair)) != GW_OK) break;
     }
@@ -602,6 +624,31 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
       weights_at_beta(tau.data(), c->ntau, cfg->beta, w);
       if ((rc = dev_alloc(c, &c->wbeta, (size_t)c->ntau)) != GW_OK) break;
       upload(c, c->wbeta, w.data(), w.size() * sizeof(double));
+    }
+    {
+      if ((rc = dev_alloc(c, &c->oz_small, kOz64SmallBytes)) != GW_OK) break;
+      if ((rc = dev_alloc(c, &c->oz_count, oz64_counter_bytes())) != GW_OK) break;
+      if (!c->dry) cudaMemset(c->oz_count, 0, oz64_counter_bytes());
+      // a P array where it is larger than the small buffer
+      auto ws = [&](void* p, size_t n) {
+        Oz64Ws w;
+        const bool big = n > kOz64SmallBytes;
+        w.mem = big ? p : c->oz_small;
+        w.bytes = big ? std::min(n, kOz64L2Bytes) : kOz64SmallBytes;
+        w.counters = c->oz_count;
+        w.status = c->status;
+        return w;
+      };
+      const size_t nt_bytes = (size_t)nk * c->ntau * c->naux2 * sizeof(double2);
+      c->oz_fwd = ws(c->Pt, nt_bytes);
+      c->oz_back = ws(c->P0t, nt_bytes);
+      c->oz_w = ws(c->Pw, (size_t)nk * c->nwb * c->naux2 * sizeof(double2));
+      c->oz = c->oz_w;
+      if (c->oz_bytes > c->oz.bytes) {
+        if ((rc = dev_alloc(c, &c->oz_mem, c->oz_bytes)) != GW_OK) break;
+        c->oz.mem = c->oz_mem;
+        c->oz.bytes = c->oz_bytes;
+      }
     }
     if (!c->dry) cudaMemset(c->status, 0, 4 * sizeof(int));
     if (cfg->precision != GW_FP64) {
@@ -851,12 +898,13 @@ int gw_sigma_eval_q(gw_ctx* ctx, const gw_c128* G_dev, gw_c128* Sig_dev, int q_b
   else
     GW_TRY(polarization_fp64(ctx, G, ctx->P0t, q_begin, q_end));
   GW_TRY(mirror_fill(ctx->P0t, ctx->nk, ctx->ntau, ctx->naux, ctx->mq_dev, ctx->stream, q_begin, q_end));
-  GW_TRY(screened_sym(ctx, ctx->P0t, ctx->Pt, q_begin, q_end));
-  // the range's blocks, for a caller that checks the stages
+  // the range's blocks, for a caller that checks the stages (P0 first: its buffer serves as workspace
+  // of the transform back)
   const size_t blk = (size_t)(q_end - q_begin) * ctx->ntau * ctx->naux2 * sizeof(double2);
   const size_t off = (size_t)q_begin * ctx->ntau * ctx->naux2;
   if (P0t_dev && blk && cudaMemcpyAsync(P0t_dev, ctx->P0t + off, blk, cudaMemcpyDeviceToDevice, ctx->stream) != cudaSuccess)
     return cuda_check("gw_sigma_eval_q: P0 copy");
+  GW_TRY(screened_sym(ctx, ctx->P0t, ctx->Pt, q_begin, q_end));
   if (Pt_dev && blk && cudaMemcpyAsync(Pt_dev, ctx->Pt + off, blk, cudaMemcpyDeviceToDevice, ctx->stream) != cudaSuccess)
     return cuda_check("gw_sigma_eval_q: P~ copy");
   if (ctx->mixed) return mixed_self_energy(ctx->mixed, G, ctx->Pt, S, q_begin, q_end);
@@ -926,6 +974,7 @@ int gw_sigma_inf(gw_ctx* ctx, const gw_c128* G_dev, gw_c128* SigInf_dev) {
     a.vc.rs_in = nao;
     a.vc.ks_in = 1;
     a.slot = SLOT_STATIC_FP64;
+    a.ws = &ctx->oz_w;
     return zgemm_fp64(a, ctx->stream);
   };
   auto second = [&](const double2* X, const double2* Vb, int k) {
@@ -949,6 +998,7 @@ int gw_sigma_inf(gw_ctx* ctx, const gw_c128* G_dev, gw_c128* SigInf_dev) {
     b.alpha = -1.0 / nk;
     b.accumulate = 1;
     b.slot = SLOT_STATIC_FP64;
+    b.ws = &ctx->oz_w;
     return zgemm_fp64(b, ctx->stream);
   };
   if (packed) {
@@ -1017,6 +1067,7 @@ int gw_commutator_residual(gw_ctx* ctx, const gw_c128* H_dev, const gw_c128* Sig
     g.alpha = alpha;
     g.accumulate = acc;
     g.slot = SLOT_STATIC_FP64;
+    g.ws = &ctx->oz_w;
     return zgemm_fp64(g, ctx->stream);
   };
   if (!ctx->S) {
@@ -1122,6 +1173,7 @@ static int gf2_exchange(gw_ctx* c, const double2* G, double2* S, double alpha) {
     g.vc.ks_in = 1;
     g.bc.bs_in = pair;
     g.slot = SLOT_GF2_FP64;
+    g.ws = &c->oz;
     return zgemm_fp64(g, c->stream);
   };
   // out[t][(a b)][(c d)] = sum_Q X[t][Q][a][b] Z[t][Q][c][d]   (Z's batch stride may be 0)
@@ -1144,6 +1196,7 @@ static int gf2_exchange(gw_ctx* c, const double2* G, double2* S, double alpha) {
     g.vc.ks_in = 1;
     g.bc.bs_in = n4;
     g.slot = SLOT_GF2_FP64;
+    g.ws = &c->oz;
     return zgemm_fp64(g, c->stream);
   };
   for (int k = 0; k < nk; ++k)
@@ -1200,6 +1253,7 @@ static int gf2_exchange(gw_ctx* c, const double2* G, double2* S, double alpha) {
             g.bc.bs_in = n2;
             g.bc.bs_out = n3;
             g.slot = SLOT_GF2_FP64;
+            g.ws = &c->oz;
             GW_TRY(zgemm_fp64(g, c->stream));
           }
           GW_TRY(reduce_partials_fp64(part, S + ((long long)k * T + t0) * n2, m, (int)n2, nao, alpha, c->stream));
@@ -1363,6 +1417,7 @@ int gw_synchronize(gw_ctx* ctx) {
   cudaMemcpy(st, ctx->status, sizeof(st), cudaMemcpyDeviceToHost);
   if (st[0] || st[1] || st[2] || st[3]) {
     cudaMemset(ctx->status, 0, sizeof(st));
+    cudaMemset(ctx->oz_count, 0, oz64_counter_bytes());   // a kernel that gave up may have left arrivals behind
     if (st[1]) return fail(GW_EDEVTIMEOUT, "a device-side wait gave up (code %d)", st[1]);
     if (st[0]) return fail(GW_EINVAL, "a Dyson matrix was singular");
     return fail(GW_ECUDA, "device status %d %d", st[2], st[3]);

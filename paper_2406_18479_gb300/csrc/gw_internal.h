@@ -70,25 +70,49 @@ struct ZView {
 };
 
 // Batch index b -> (bo, bi) = (b / bin, b % bin); the operand's offset is
-//   (tab ? tab[bi] : bi * bs_in) + bo * bs_out.
+//   (tab ? tab[bi] : (list ? list[bi] : bi) * bs_in) + bo * bs_out.
 struct ZBatch {
   const long long* tab = nullptr;
+  const int* list = nullptr;
   long long bs_in = 0, bs_out = 0;
 };
+
+// Device workspace of the digit tiles of zgemm_oz64 (owned by a context, used in its stream's order).
+// counters (optional): oz64_counter_bytes(), zero before first use and between launches, for products
+// that share a tile's K among CTAs. status[1] receives a device-side wait that gave up.
+struct Oz64Ws {
+  void* mem = nullptr;
+  size_t bytes = 0;
+  void* counters = nullptr;
+  int* status = nullptr;
+};
+
+constexpr size_t kOz64L2Bytes = 96ull << 20, kOz64SmallBytes = 4ull << 20;
 
 struct ZGemm {
   int M = 0, N = 0, K = 0, nbatch = 1, bin = 1 << 30;
   const double2* A = nullptr;    // A(m, k)
   const double2* B = nullptr;    // B(n, k)
-  double2* C = nullptr;          // C(m, n): rows per C.rs_*, columns with stride C.ks_in
+  double2* C = nullptr;          // C(m, n): row m and column n as r and k of vc
   ZView va, vb, vc;
   ZBatch ba, bb, bc;
   double alpha = 1.0;            // C = alpha * sum_k A(m,k) B(n,k) (+ C if accumulate)
   int accumulate = 0;
   int slot = SLOT_VG_FP64;       // profiling slot of this launch
+  const Oz64Ws* ws = nullptr;    // digit workspace: with one, products that pay run on the tensor cores
+  double unit = 0.0;             // complex multiply-adds of one (k, tau) matrix where a product joins several
 };
 
+// C = alpha A B^T (+ C) to FP64 accuracy: on the tensor cores through exact digits (k_oz64.cu) where
+// g.ws is given and oz64_takes(g), else on the FP64 pipe.
 int zgemm_fp64(const ZGemm& g, void* stream);
+bool oz64_takes(const ZGemm& g);
+// *done = false: the workspace cannot hold one pair of row tiles (nothing was launched)
+int zgemm_oz64(const ZGemm& g, void* stream, bool* done);
+// workspace bytes for all digits of operands of p_rows (the side whose output index is contiguous)
+// and q_rows rows over K complex k
+size_t oz64_bytes(long long p_rows, long long q_rows, int K);
+size_t oz64_counter_bytes();
 
 // In-place Gauss-Jordan inversion with partial pivoting of nbatch n x n matrices
 // (matrix b at base + b * stride). diag_shift: before inverting, M <- diag_sign*M + shift(b)*I

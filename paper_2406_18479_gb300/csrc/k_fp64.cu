@@ -38,7 +38,7 @@ __device__ __forceinline__ long long view_k(const ZView& v, int k) {
 }
 
 __device__ __forceinline__ long long batch_off(const ZBatch& b, int bo, int bi) {
-  return (b.tab ? b.tab[bi] : (long long)bi * b.bs_in) + (long long)bo * b.bs_out;
+  return (b.tab ? b.tab[bi] : (long long)(b.list ? b.list[bi] : bi) * b.bs_in) + (long long)bo * b.bs_out;
 }
 
 __global__ void __launch_bounds__(256) zgemm_fp64_kernel(const ZGemm g) {
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256) zgemm_fp64_kernel(const ZGemm g) {
     for (int j = 0; j < 2; ++j) {
       const int n = n0 + 2 * tx + j;
       if (n >= g.N) continue;
-      double2* c = C + ro + (long long)n * g.vc.ks_in;
+      double2* c = C + ro + view_k(g.vc, n);
       double2 v = make_double2(g.alpha * acc[i][j].x, g.alpha * acc[i][j].y);
       if (g.accumulate) {
         const double2 old = *c;
@@ -779,6 +779,11 @@ inline int grid_for(long long total, int block) {
 
 int zgemm_fp64(const ZGemm& g, void* stream) {
   if (g.M <= 0 || g.N <= 0 || g.nbatch <= 0) return GW_OK;
+  if (oz64_takes(g)) {
+    bool done = false;
+    const int rc = zgemm_oz64(g, stream, &done);
+    if (rc != GW_OK || done) return rc;
+  }
   if (g.nbatch > 65535) return fail(GW_EINVAL, "zgemm_fp64: batch %d too large", g.nbatch);
   dim3 grid((g.N + TN - 1) / TN, (g.M + TM - 1) / TM, g.nbatch);
   if (grid.y > 65535) return fail(GW_EINVAL, "zgemm_fp64: M=%d too large", g.M);

@@ -1,0 +1,763 @@
+// FP64-accurate complex GEMM on tcgen05 tensor cores through exact integer digits.
+//
+// GB300 issues 2 FP64 FMAs per clock and SM (1.25 TFLOP/s), 1/900 of its bf16 tensor rate, so an
+// FP64 product is cheaper as a sum of exact bf16 products (the error-free splitting of Ozaki et
+// al.). C(m, n) = alpha sum_k A(m, k) B(n, k) over complex k is taken as a real GEMM: one operand
+// (P) is embedded as two real rows (re, -im), (im, re) per complex row over 2 K real k, the other
+// (Q) as its plain real row (re, im); the product of the two gives (Re C, Im C) in adjacent rows,
+// which is the memory order of a complex output.
+//
+// Each row is scaled by one power of two 2^E above its largest |re|, |im| and rounded to
+//   N = round(x 2^(62 - E)) = sum_i d_i 256^(7 - i),   d_i in [-128, 127], i = 0..7
+// (residual 2^-63 of the row's scale, 2^10 finer than FP64's own rounding of its largest
+// element). Digits are exact in bf16. Products of order o = i + j are summed in their own FP32
+// accumulator over at most 128 real k: |sum| <= 8 * 128 * 2^14 = 2^24, exact whatever order the
+// tensor core adds in. The 8 accumulators (o = 0..7; higher orders are below 2^-59) are joined
+// into a 96-bit integer, summed over the chunks of 128 k without rounding, and only the final
+// value is rounded to FP64. The result does not depend on tiling or batching, and its error is
+// below that of a running FP64 sum.
+//
+// Bound: the tensor cores and the L2 reads of the digit tiles (48 KB per k-step of a 128 x 64 tile),
+// about 23 TFLOP/s of complex products at long K (R of a molecule, nao = 45) and 13 where the output is
+// as large as the work (transforms), against 0.7..1.1 on the FP64 pipe. P0 of a 2x2x2 solid (nao = 26,
+// naux = 104, 80 nodes): 313 -> 31.3 ms; Sigma of a molecule (nao = 45): 76.9 -> 5.8 ms; the two
+// transforms of a 3x3x3 solid (naux = 200, 100 nodes): 198 -> 21 ms. Error against 64-bit references
+// on these: 2e-16 and 4e-16 (FP64 pipe: 3e-15 and 6e-15).
+//
+// Rows with a non-finite element, or whose scale lies outside 2^+-480 (where the scaled product
+// could over- or underflow), carry a NaN scale; outputs that meet one are computed by a plain
+// FP64 loop in the epilogue, so infinities, NaN and extreme ranges behave as in zgemm_fp64.
+//
+// Kernels
+//   oz64_pack_kernel  FP64 views -> digit tiles, in the order the tensor core reads shared memory
+//                     (8-row x 16-byte core matrices, no swizzle): a k-step of a tile is one
+//                     contiguous block, moved by one bulk copy, no tensor map
+//   oz64_gemm_kernel  persistent GEMM, 128 real rows of P x NT rows of Q per tile. The 8 digit
+//                     tiles of Q lie behind one another in N, and the accumulator of order o in
+//                     TMEM columns [o NT, (o + 1) NT): one MMA of digit i of P against the digits
+//                     0..7-i of Q (N = (8 - i) NT, split at 256) adds every product of row i to its
+//                     order at once: 8 to 12 wide MMAs per 16 k instead of 36 narrow ones.
+#include <algorithm>
+#include <cmath>
+
+#include "gw_internal.h"
+#include "tc_ptx.cuh"
+
+namespace gwi {
+
+namespace {
+
+constexpr int kDigits = 8;
+constexpr int kK = 16;              // real k per MMA
+constexpr int kChunkSteps = 8;      // k-steps per exact chunk (128 real k)
+constexpr int kPTile = 64;          // complex rows of P per tile (128 TMEM lanes)
+constexpr int kScaleMax = 480;      // |E| beyond this takes the plain FP64 loop
+constexpr int kSegSteps = 8;        // least k-steps of a packing segment
+constexpr int kMaxSegs = 32;
+constexpr int kSplitUnits = 152;    // tiles x splits of a split-K launch, at most (one wave)
+
+// x / d for x < 2^31: multiply-high (see FastDiv in k_mixed.cu)
+struct Div {
+  unsigned long long m = 1ull << 31;
+  int sh = 31, d = 1 << 30;
+};
+Div make_div(int d) {
+  Div f;
+  int l = 0;
+  while ((1ll << l) < d) ++l;
+  f.d = d;
+  f.sh = 31 + l;
+  f.m = ((1ull << f.sh) + (unsigned long long)d - 1) / (unsigned long long)d;
+  return f;
+}
+__device__ __forceinline__ int div_by(int x, const Div& f) {
+  return (int)(((unsigned long long)(unsigned)x * f.m) >> f.sh);
+}
+
+// one operand: element (r, k) of batch (bo, bi) as in ZGemm, and where its digit tiles go
+struct Side {
+  const double2* src = nullptr;
+  ZBatch b;
+  long long rs_in = 0, rs_out = 0, ks_in = 0, ks_out = 0;
+  Div rdiv, kdiv;
+  int row0 = 0, rows = 0, tiles = 0;    // rows [row0, row0 + rows) of this launch
+  int dep_o = 0, dep_i = 0;             // whether the operand varies with the outer / inner batch index
+  int no = 1, ni = 1;                   // packed batches
+  unsigned char* dst = nullptr;
+  double* scale = nullptr;              // per packed row: 2^(E - 34), NaN: plain FP64 loop
+  unsigned long long* pmax = nullptr;   // segs > 1: largest |value| bits of each row and K segment
+};
+
+struct Job {
+  Side p, q;
+  int K = 0, nks = 0;                   // complex k; k-steps of 16 real k
+  int segs = 1, seg_steps = 0;          // packing: K segments per row tile, k-steps of one
+  int o0 = 0, i0 = 0, no = 1, ni = 1;   // batch range of this launch: bo in [o0, o0 + no), bi likewise
+  double2* C = nullptr;
+  ZBatch bc;
+  // output element of P row a, Q row b: cp(a) + cq(b)
+  long long cp_in = 0, cp_out = 0, cq_in = 0, cq_out = 0;
+  Div cp_div, cq_div;
+  double alpha = 1.0;
+  int accumulate = 0;
+  // split K: ksplit CTAs share a tile, each summing split_chunks chunks; their 96-bit integers meet in
+  // part ([tile][split][column][128 lanes], hi and lo apart), and the last to arrive (a counter per
+  // tile and epilogue warp) adds them, exactly, and writes the output
+  int ksplit = 1, split_chunks = 0;
+  long long* part_hi = nullptr;
+  uint32_t* part_lo = nullptr;
+  unsigned int* counter = nullptr;
+  int* status = nullptr;
+};
+
+__device__ __forceinline__ long long side_row(const Side& s, int r) {
+  const int rq = div_by(r, s.rdiv);
+  return (long long)rq * s.rs_out + (long long)(r - rq * s.rdiv.d) * s.rs_in;
+}
+__device__ __forceinline__ long long side_k(const Side& s, int k) {
+  const int kq = div_by(k, s.kdiv);
+  return (long long)kq * s.ks_out + (long long)(k - kq * s.kdiv.d) * s.ks_in;
+}
+__device__ __forceinline__ long long batch_in(const ZBatch& b, int bi) {
+  return b.tab ? b.tab[bi] : (long long)(b.list ? b.list[bi] : bi) * b.bs_in;
+}
+__device__ __forceinline__ const double2* side_base(const Side& s, int bo, int bi) {
+  return s.src + batch_in(s.b, bi) + (long long)bo * s.b.bs_out;
+}
+
+// round(x 2^(62 - E)) + 0x80..80 for |x| < 2^E: byte 7 - i of the result is digit i plus 128
+__device__ __forceinline__ unsigned long long digits_of(double x, int E) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((bits >> 52) & 0x7FF);
+  const unsigned long long m = ex ? ((bits & 0xFFFFFFFFFFFFFull) | (1ull << 52)) : 0ull;
+  const int sh = E + 1013 - ex;                  // x = m 2^(ex - 1075): right shift, >= -9
+  unsigned long long n;
+  if (sh <= 0) n = m << -sh;
+  else n = sh > 54 ? 0ull : (m + (1ull << (sh - 1))) >> sh;
+  const unsigned long long neg = (unsigned long long)((long long)bits >> 63);
+  return ((n ^ neg) - neg) + 0x8080808080808080ull;
+}
+
+// digit j (0: leading) of four words as two bf16 pairs
+__device__ __forceinline__ float digit_f(unsigned long long u, int j) {
+  const uint32_t w = j < 4 ? (uint32_t)(u >> 32) : (uint32_t)u;
+  const uint32_t b = (w >> (24 - 8 * (j & 3))) & 0xFFu;
+  return __fsub_rn(__uint_as_float(0x4B000000u | b), 8388736.0f);     // 2^23 + b - (2^23 + 128)
+}
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {   // both exact in bf16
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+
+// One block per row tile, packed batch and K segment. A thread owns one row and every
+// (256 / RT)-th group of four complex k (8 real k: one 16-byte piece of a core-matrix row per digit).
+// The row's scale needs a pass over the row first: within the block where it covers all of K, by
+// oz64_scale_kernel (a maximum per segment) where long rows are split so that few row tiles still
+// fill the GPU. Bound: memory (16 bytes read twice, 64 (P) or 32 (Q) written per complex element);
+// neighbouring lanes hold neighbouring rows, so that a digit's 8 rows make one 128-byte line.
+template <int kRows>
+struct PackPos {
+  int tile, pb, seg, row, grp, k0, k1;   // this block's tile, batch and segment; this thread's row and group
+  long long prow;
+  bool row_ok;
+  const double2* src;
+  __device__ PackPos(const Side& s, const Job& j, long long t) {
+    seg = (int)(t % j.segs);
+    t /= j.segs;
+    tile = (int)(t % s.tiles);
+    pb = (int)(t / s.tiles);
+    row = threadIdx.x % kRows;
+    grp = threadIdx.x / kRows;
+    const int r = tile * kRows + row;
+    row_ok = r < s.rows;
+    src = side_base(s, j.o0 + pb / s.ni, j.i0 + pb % s.ni) + (row_ok ? side_row(s, s.row0 + r) : 0);
+    prow = ((long long)pb * s.tiles + tile) * kRows + row;
+    k0 = seg * j.seg_steps;              // k-steps [k0, k1) of the segment
+    k1 = min(j.nks, k0 + j.seg_steps);
+  }
+};
+
+template <int kRows>
+__device__ __forceinline__ unsigned long long row_max(const Side& s, const Job& j, const PackPos<kRows>& p) {
+  constexpr int kGroups = 256 / kRows;
+  unsigned long long mx = 0;
+  if (p.row_ok) {
+    const int kend = min(j.K, 8 * p.k1);
+    for (int k = 8 * p.k0 + p.grp * 4; k < kend; k += kGroups * 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (k + u >= kend) break;
+        const double2 x = p.src[side_k(s, k + u)];
+        mx = max(mx, max((unsigned long long)__double_as_longlong(x.x) & 0x7FFFFFFFFFFFFFFFull,
+                         (unsigned long long)__double_as_longlong(x.y) & 0x7FFFFFFFFFFFFFFFull));
+      }
+    }
+  }
+  __shared__ unsigned long long red[256];
+  red[threadIdx.x] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int g = 0; g < kGroups; ++g) mx = max(mx, red[g * kRows + p.row]);
+  return mx;
+}
+
+template <int kRows>
+__device__ void scale_tile(const Side& s, const Job& j, long long t) {
+  const PackPos<kRows> p(s, j, t);
+  const unsigned long long mx = row_max<kRows>(s, j, p);
+  if (p.grp == 0) s.pmax[p.prow * j.segs + p.seg] = mx;
+}
+
+template <int RT, bool PSIDE>
+__device__ void pack_tile(const Side& s, const Job& j, long long t) {
+  constexpr int kRows = PSIDE ? kPTile : RT;      // complex rows of the tile
+  constexpr int kReal = PSIDE ? 2 * kPTile : RT;  // real rows of the tile
+  constexpr int kGroups = 256 / kRows;
+  const PackPos<kRows> p(s, j, t);
+  unsigned long long mx = 0;
+  if (j.segs == 1) {
+    mx = row_max<kRows>(s, j, p);
+  } else {
+    for (int g = 0; g < j.segs; ++g) mx = max(mx, s.pmax[p.prow * j.segs + g]);
+  }
+  const int ex = (int)(mx >> 52);
+  int E = ex - 1022;
+  const bool plain = mx != 0 && (ex == 0x7FF || E > kScaleMax || E < -kScaleMax);
+  const bool zero = mx == 0 || plain;
+  if (zero) E = 0;
+  if (p.grp == 0 && p.seg == 0)
+    s.scale[p.prow] = plain ? __longlong_as_double(0x7FF8000000000000ll)
+                            : __longlong_as_double((long long)(E - 34 + 1023) << 52);
+  unsigned char* base = s.dst + ((long long)p.pb * s.tiles + p.tile) * j.nks * (long long)(kDigits * kReal * 32);
+  const int rr = PSIDE ? 2 * p.row : p.row;
+  for (int g = 2 * p.k0 + p.grp; g < 2 * p.k1; g += kGroups) {
+    unsigned long long u[8];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int k = 4 * g + c;
+      double2 x = make_double2(0.0, 0.0);
+      if (p.row_ok && !zero && k < j.K) x = p.src[side_k(s, k)];
+      u[2 * c] = digits_of(x.x, E);
+      u[2 * c + 1] = digits_of(x.y, E);
+    }
+    unsigned char* d = base + (long long)(g >> 1) * (kDigits * kReal * 32) + (rr >> 3) * 256 + (g & 1) * 128 +
+                       (rr & 7) * 16;
+#pragma unroll
+    for (int q = 0; q < kDigits; ++q) {
+      uint32_t w[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) w[c] = bf16_pair(digit_f(u[2 * c], q), digit_f(u[2 * c + 1], q));
+      uint4* o = reinterpret_cast<uint4*>(d + q * (kReal * 32));
+      if (PSIDE) {   // rows (re, -im) and (im, re)
+        o[0] = make_uint4(w[0] ^ 0x80000000u, w[1] ^ 0x80000000u, w[2] ^ 0x80000000u, w[3] ^ 0x80000000u);
+        o[1] = make_uint4(__funnelshift_l(w[0], w[0], 16), __funnelshift_l(w[1], w[1], 16),
+                          __funnelshift_l(w[2], w[2], 16), __funnelshift_l(w[3], w[3], 16));
+      } else {
+        o[0] = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    }
+  }
+}
+
+template <int NT>
+__global__ void __launch_bounds__(256) oz64_scale_kernel(const __grid_constant__ Job j) {
+  const long long np = (long long)j.p.tiles * j.p.no * j.p.ni * j.segs;
+  if (blockIdx.x < np) scale_tile<kPTile>(j.p, j, blockIdx.x);
+  else scale_tile<NT>(j.q, j, blockIdx.x - np);
+}
+
+template <int NT>
+__global__ void __launch_bounds__(256) oz64_pack_kernel(const __grid_constant__ Job j) {
+  const long long np = (long long)j.p.tiles * j.p.no * j.p.ni * j.segs;
+  if (blockIdx.x < np) pack_tile<2 * kPTile, true>(j.p, j, blockIdx.x);
+  else pack_tile<NT, false>(j.q, j, blockIdx.x - np);
+}
+
+// the plain FP64 loop of one real output (part 0: re, 1: im), for rows without a digit form
+__device__ __noinline__ double plain_dot(const Job& j, int bo, int bi, int pr, int qr, int part) {
+  const double2* a = side_base(j.p, bo, bi) + side_row(j.p, pr);
+  const double2* b = side_base(j.q, bo, bi) + side_row(j.q, qr);
+  double s = 0.0;
+  for (int k = 0; k < j.K; ++k) {
+    const double2 x = a[side_k(j.p, k)], y = b[side_k(j.q, k)];
+    s = part ? fma(x.y, y.x, fma(x.x, y.y, s)) : fma(-x.y, y.y, fma(x.x, y.x, s));
+  }
+  return s;
+}
+
+template <int NT>
+struct Oz64Shape {
+  static constexpr int kABytes = kDigits * 128 * 32;            // one k-step of a P tile
+  static constexpr int kBBytes = kDigits * NT * 32;             // and of a Q tile
+  static constexpr int kStageBytes = kABytes + kBBytes;
+  static constexpr int kStages = NT == 64 ? 4 : 5;
+  static constexpr int kBufCols = kDigits * NT;
+  static constexpr int kBufs = 512 / kBufCols;                  // accumulator sets in TMEM
+  static constexpr int kThreads = 320;                          // producer, MMA, 8 epilogue warps
+  static constexpr size_t kSmem = 128 + (size_t)kStages * kStageBytes + 256;
+  static_assert(kSmem <= 232448, "stages exceed shared memory");
+};
+
+// K-major operand without swizzle: 8 x 16-byte core matrices, 128 bytes between the two k halves
+// (leading offset), 256 bytes between 8-row groups (stride offset)
+__device__ __forceinline__ uint64_t core_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+  d |= (uint64_t)(128 >> 4) << 16;
+  d |= (uint64_t)(256 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+
+// hi 2^32 + lo += sum_o a_o 256^(7 - o), a_o the exact integer accumulators of one chunk
+__device__ __forceinline__ void join_orders(const float (&v)[kDigits][4], int u, long long& hi, uint32_t& lo) {
+  int a[kDigits];
+#pragma unroll
+  for (int o = 0; o < kDigits; ++o) a[o] = __float2int_rn(v[o][u]);
+  // leading digits are within 64, so |a0| <= 2^19, |a1| <= 2^21, |a2| <= 2^22: no overflow in 32 bits
+  const int h0 = a[0] * 256 + a[1], h1 = a[2] * 256 + a[3];
+  hi += (long long)h0 * 65536 + h1;
+  const long long l = (long long)a[4] * 16777216 + (long long)a[5] * 65536 + (long long)a[6] * 256 + a[7] +
+                      (long long)(unsigned long long)lo;
+  hi += l >> 32;
+  lo = (uint32_t)l;
+}
+
+// (hi 2^32 + lo) 2^e rounded to FP64, in integer arithmetic: int64 -> FP64 conversions and scalings run
+// on the FP64 pipe (2 a clock and SM), which five of them per output would make the bound of short
+// products (a rank-16 update: 12k clocks a tile, against 1.2k of MMAs)
+__device__ __forceinline__ double to_fp64(long long hi, uint32_t lo, int e) {
+  const long long neg = hi >> 63;
+  unsigned long long H = (unsigned long long)(hi ^ neg);
+  uint32_t L = lo ^ (uint32_t)neg;
+  if (neg) {                                   // two's complement of the 96 bits
+    L += 1u;
+    H += L == 0u;
+  }
+  if (H == 0) {
+    if (L == 0) return 0.0;
+    H = (unsigned long long)L << 32;
+    L = 0;
+    e -= 64;
+  }
+  const int lz = __clzll((long long)H);
+  H = (H << lz) | (((unsigned long long)L << 32) >> 1 >> (63 - lz));
+  const unsigned long long m = (H >> 11) + ((H >> 10) & 1ull);      // 53 bits, rounded half up
+  const int E = 52 + 43 - lz + e + 1023;
+  if (E < 1 || E > 2045) {                     // beyond the normal range: rare
+    const double x = scalbn((double)m, 43 - lz + e);
+    return neg ? -x : x;
+  }
+  return __longlong_as_double((long long)((((unsigned long long)(E - 1) << 52) + m) | ((unsigned long long)neg & (1ull << 63))));
+}
+
+template <int NT, bool MULTI>
+__global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant__ Job j) {
+  using S = Oz64Shape<NT>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S::kStages * S::kStageBytes);
+  uint64_t* empty = full + S::kStages;
+  uint64_t* acc_full = empty + S::kStages;      // [kBufs]
+  uint64_t* acc_empty = acc_full + 2;
+  uint64_t* drain_bar = acc_full + 4;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 5);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < S::kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < S::kBufs; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], 8);
+    }
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(512));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int per_batch = j.p.tiles * j.q.tiles;
+  const int ksplit = MULTI ? j.ksplit : 1;
+  const int total = per_batch * j.no * j.ni * ksplit;
+  // work unit -> batch, P tile, Q tile (Q fastest: neighbouring CTAs share the larger P tile in L2),
+  // and its k-steps [s0, s1)
+  auto split = [&](int unit, int& o, int& i, int& pt, int& qt, int& s0, int& s1) {
+    const int tile = MULTI ? unit / ksplit : unit;
+    s0 = 0;
+    s1 = j.nks;
+    if (MULTI && ksplit > 1) {
+      s0 = (unit - tile * ksplit) * j.split_chunks * kChunkSteps;
+      s1 = min(j.nks, s0 + j.split_chunks * kChunkSteps);
+    }
+    const int b = tile / per_batch, w = tile - b * per_batch;
+    o = b / j.ni;
+    i = b - o * j.ni;
+    pt = w / j.q.tiles;
+    qt = w - pt * j.q.tiles;
+  };
+  auto packed = [](const Side& s, int o, int i) { return (s.dep_o ? o : 0) * s.ni + (s.dep_i ? i : 0); };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t step = 0;
+      for (int tile = blockIdx.x; tile < total && !*abort_flag; tile += gridDim.x) {
+        int o, i, pt, qt, s0, s1;
+        split(tile, o, i, pt, qt, s0, s1);
+        const unsigned char* a = j.p.dst + ((long long)packed(j.p, o, i) * j.p.tiles + pt) * j.nks * (long long)S::kABytes;
+        const unsigned char* b = j.q.dst + ((long long)packed(j.q, o, i) * j.q.tiles + qt) * j.nks * (long long)S::kBBytes;
+        for (int s = s0; s < s1; ++s, ++step) {
+          const int st = step % S::kStages;
+          if (!mbar_wait(&empty[st], ((step / S::kStages) & 1) ^ 1, abort_flag, j.status, 21)) break;
+          mbar_expect_tx(&full[st], S::kStageBytes);
+          uint8_t* sa = smem + (size_t)st * S::kStageBytes;
+          bulk_load(sa, a + (long long)s * S::kABytes, S::kABytes, &full[st]);
+          bulk_load(sa + S::kABytes, b + (long long)s * S::kBBytes, S::kBBytes, &full[st]);
+        }
+      }
+      if (*abort_flag) {   // let every issued copy land before the CTA exits (bounded)
+        const uint64_t t0 = globaltimer();
+        for (int k = 0; k < S::kStages && step > (uint32_t)k; ++k) {
+          const uint32_t s2 = step - 1 - k;
+          while (!mbar_try(&full[s2 % S::kStages], (s2 / S::kStages) & 1) && globaltimer() - t0 < kWaitLimitNs) {
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      uint32_t step = 0, chunk = 0;
+      const uint64_t desc0 = core_desc(smem_u32(smem));
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
+        int o, i, pt, qt, s0, s1;
+        split(tile, o, i, pt, qt, s0, s1);
+        for (int s = s0; s < s1 && ok; ++s, ++step) {
+          const bool start = (s % kChunkSteps) == 0;
+          const uint32_t buf = chunk % S::kBufs;
+          if (start) {
+            if (!mbar_wait(&acc_empty[buf], ((chunk / S::kBufs) & 1) ^ 1, abort_flag, j.status, 22)) { ok = false; break; }
+            tc_fence_after();
+          }
+          const int st = step % S::kStages;
+          if (!mbar_wait(&full[st], (step / S::kStages) & 1, abort_flag, j.status, 23)) { ok = false; break; }
+          tc_fence_after();
+          const uint64_t sa = desc0 + (uint64_t)((st * S::kStageBytes) >> 4);
+          const uint64_t sb = sa + (uint64_t)(S::kABytes >> 4);
+          const uint32_t d = tmem + buf * S::kBufCols;
+#pragma unroll
+          for (int i = 0; i < kDigits; ++i) {
+            // digits 0..7-i of Q, at most 256 columns per MMA; digit 0 of P opens every order
+            constexpr int kPer = 256 / NT;
+#pragma unroll
+            for (int q = 0; q < kDigits - i; q += kPer) {
+              const int nq = kDigits - i - q < kPer ? kDigits - i - q : kPer;
+              mma_bf16(d + (uint32_t)((i + q) * NT), sa + (uint64_t)(i * 128 * 32 >> 4),
+                       sb + (uint64_t)(q * NT * 32 >> 4), idesc_bf16(nq * NT, false), start && i == 0 ? 0u : 1u);
+            }
+          }
+          mma_commit(&empty[st]);
+          if ((s % kChunkSteps) == kChunkSteps - 1 || s == s1 - 1) {
+            mma_commit(&acc_full[buf]);
+            ++chunk;
+          }
+        }
+      }
+      mma_commit(drain_bar);   // the last MMAs end before TMEM is released
+      const uint64_t t0 = globaltimer();
+      while (!mbar_try(drain_bar, 0) && globaltimer() - t0 < kWaitLimitNs) {
+      }
+    }
+  } else {
+    // epilogue: TMEM lane quarter warp % 4, columns [half NT/2, half NT/2 + NT/2)
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    constexpr int kCols = NT / 2;
+    const int lrow = quarter * 32 + lane;
+    const int part = lrow & 1;
+    uint32_t chunk = 0;
+    for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
+      int o, i, pt, qt, s0, s1;
+      split(tile, o, i, pt, qt, s0, s1);
+      const int nchunks = (s1 - s0 + kChunkSteps - 1) / kChunkSteps;
+      const int bo = j.o0 + o, bi = j.i0 + i;
+      const int pr = pt * kPTile + (lrow >> 1);
+      const bool p_ok = pr < j.p.rows;
+      // biased exponents of the scales (0x7FF: a row for the plain loop)
+      const int ep = __double2hiint(j.p.scale[((long long)packed(j.p, o, i) * j.p.tiles + pt) * kPTile + (lrow >> 1)]) >> 20;
+      const double* sq = j.q.scale + ((long long)packed(j.q, o, i) * j.q.tiles + qt) * NT;
+      const int ap = j.p.row0 + (p_ok ? pr : 0), apq = div_by(ap, j.cp_div);
+      double* C = reinterpret_cast<double*>(j.C + batch_in(j.bc, bi) + (long long)bo * j.bc.bs_out + (long long)apq * j.cp_out +
+                                            (long long)(ap - apq * j.cp_div.d) * j.cp_in) + part;
+      auto put = [&](int col, long long hi, uint32_t lo) {
+        const int qr = qt * NT + col;
+        if (!p_ok || qr >= j.q.rows) return;
+        const int eq = __double2hiint(sq[col]) >> 20;
+        double x = ep == 0x7FF || eq == 0x7FF ? plain_dot(j, bo, bi, ap, j.q.row0 + qr, part)
+                                              : to_fp64(hi, lo, ep + eq - 2046);
+        if (j.alpha != 1.0) x *= j.alpha;
+        const int aq = j.q.row0 + qr, aqq = div_by(aq, j.cq_div);
+        double* c = C + 2 * ((long long)aqq * j.cq_out + (long long)(aq - aqq * j.cq_div.d) * j.cq_in);
+        *c = j.accumulate ? *c + x : x;
+      };
+      long long hi[MULTI ? kCols : 1];
+      uint32_t lo[MULTI ? kCols : 1];
+      bool ok = true;
+      for (int c = 0; c < nchunks; ++c, ++chunk) {
+        const uint32_t buf = chunk % S::kBufs;
+        if (!mbar_wait(&acc_full[buf], (chunk / S::kBufs) & 1, abort_flag, j.status, 24)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + buf * S::kBufCols + half * kCols;
+#pragma unroll(MULTI ? kCols / 4 : 1)
+        for (int g = 0; g < kCols / 4; ++g) {
+          float v[kDigits][4];
+#pragma unroll
+          for (int d = 0; d < kDigits; ++d) tmem_ld4(tb + d * NT + 4 * g, v[d]);
+          tmem_wait_ld();
+          if (g == kCols / 4 - 1) {       // this warp's columns are in registers: release TMEM
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if constexpr (MULTI) {
+              if (c == 0) hi[4 * g + u] = 0, lo[4 * g + u] = 0;
+              join_orders(v, u, hi[4 * g + u], lo[4 * g + u]);
+            } else {
+              long long h = 0;
+              uint32_t l = 0;
+              join_orders(v, u, h, l);
+              put(half * kCols + 4 * g + u, h, l);
+            }
+          }
+        }
+      }
+      if (!ok) break;
+      if constexpr (MULTI) {
+        if (ksplit > 1) {
+          const int t = tile / ksplit, me = tile - t * ksplit;
+          const long long at = ((long long)t * ksplit + me) * NT * 128 + (long long)half * kCols * 128 + lrow;
+#pragma unroll
+          for (int u = 0; u < kCols; ++u) {
+            j.part_hi[at + u * 128] = hi[u];
+            j.part_lo[at + u * 128] = lo[u];
+          }
+          // every warp meets its counterparts of the other splits on a counter of its own: no wait
+          __threadfence();
+          __syncwarp();
+          unsigned int n = 0;
+          if (lane == 0) {
+            n = atomicAdd(&j.counter[t * 8 + warp - 2], 1u);
+            if (n == (unsigned)ksplit - 1) j.counter[t * 8 + warp - 2] = 0;   // ready for the next launch
+          }
+          if (__shfl_sync(0xffffffffu, n, 0) != (unsigned)ksplit - 1) continue;
+          __threadfence();
+          for (int m = 0; m < ksplit; ++m) {
+            if (m == me) continue;
+            const long long from = ((long long)t * ksplit + m) * NT * 128 + (long long)half * kCols * 128 + lrow;
+#pragma unroll
+            for (int u = 0; u < kCols; ++u) {
+              const unsigned long long l = (unsigned long long)lo[u] + __ldcg(&j.part_lo[from + u * 128]);
+              hi[u] += __ldcg(&j.part_hi[from + u * 128]) + (long long)(l >> 32);
+              lo[u] = (uint32_t)l;
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kCols; ++u) put(half * kCols + u, hi[u], lo[u]);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(v, 1);
+  }();
+  return n;
+}
+
+template <int NT, bool MULTI>
+int launch_gemm(const Job& j, int slot, cudaStream_t st) {
+  using S = Oz64Shape<NT>;
+  static const bool attr = cudaFuncSetAttribute(oz64_gemm_kernel<NT, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)S::kSmem) == cudaSuccess;
+  if (!attr) return fail(GW_ECUDA, "oz64_gemm: shared memory attribute refused");
+  const long long total = (long long)j.p.tiles * j.q.tiles * j.no * j.ni * j.ksplit;
+  const long long np = (long long)j.p.tiles * j.p.no * j.p.ni, nq = (long long)j.q.tiles * j.q.no * j.q.ni;
+  if (total > 2147483647LL || (np + nq) * j.segs > 2147483647LL) return fail(GW_EINVAL, "oz64_gemm: too many tiles");
+  if (j.segs > 1) {
+    prof_begin(SLOT_LIMBS, st);
+    oz64_scale_kernel<NT><<<(unsigned)((np + nq) * j.segs), 256, 0, st>>>(j);
+    prof_end(SLOT_LIMBS, st, 0.0, ((double)np * kPTile + (double)nq * NT) * 16.0 * j.K);
+  }
+  prof_begin(SLOT_LIMBS, st);
+  oz64_pack_kernel<NT><<<(unsigned)((np + nq) * j.segs), 256, 0, st>>>(j);
+  prof_end(SLOT_LIMBS, st, 0.0, ((double)np * kPTile * (32.0 + 64.0) + (double)nq * NT * (32.0 + 32.0)) * 8.0 * j.nks);
+  prof_begin(slot, st);
+  oz64_gemm_kernel<NT, MULTI><<<(int)std::min<long long>(total, sm_count()), S::kThreads, S::kSmem, st>>>(j);
+  // algorithmic flops: 8 per complex multiply-add
+  prof_end(slot, st, 8.0 * j.p.rows * (double)j.q.rows * j.K * j.no * j.ni,
+           (double)total / j.ksplit * j.nks * S::kStageBytes);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "oz64_gemm launch: %s", cudaGetErrorString(e));
+}
+
+Side make_side(const double2* src, const ZView& v, const ZBatch& b, int no, int ni) {
+  Side s;
+  s.src = src;
+  s.b = b;
+  s.rs_in = v.rs_in;
+  s.rs_out = v.rs_out;
+  s.ks_in = v.ks_in;
+  s.ks_out = v.ks_out;
+  s.rdiv = make_div(v.rin);
+  s.kdiv = make_div(v.kin);
+  s.dep_o = no > 1 && b.bs_out != 0;
+  s.dep_i = ni > 1 && (b.tab || b.bs_in != 0);
+  return s;
+}
+
+inline long long up(long long x, long long m) { return (x + m - 1) / m * m; }
+
+}  // namespace
+
+size_t oz64_counter_bytes() { return (size_t)kSplitUnits * 8 * sizeof(unsigned int); }
+
+size_t oz64_bytes(long long p_rows, long long q_rows, int K) {
+  const long long nks = (K + 7) / 8;
+  // digit tiles (64-row Q tiles bound the padding) and scales
+  const long long extra = 8 + (nks >= 2 * kSegSteps ? 8 * kMaxSegs : 0);
+  return (size_t)(up(p_rows, kPTile) * (nks * 512 + extra) + up(q_rows, 64) * (nks * 256 + extra) + 1024);
+}
+
+// Where digits pay: below 8 complex k most of a k-step is padding, and tiny products (under 2^13
+// complex multiply-adds per matrix) stay on the FP64 pipe for their single launch. The rule looks
+// at one matrix only (g.unit where several share a product), so that batch sizes and tau batches
+// never change a result.
+bool oz64_takes(const ZGemm& g) {
+  return g.ws && g.ws->mem && g.K >= 8 && (g.unit > 0.0 ? g.unit : (double)g.M * g.N * g.K) >= 8192.0;
+}
+
+int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
+  *done = false;
+  cudaStream_t st = (cudaStream_t)stream;
+  const int ni = std::min(g.bin, g.nbatch), no = (g.nbatch + ni - 1) / ni;
+  if (no * (long long)ni != g.nbatch) return GW_OK;
+  // P, the embedded side, is the one whose output index is contiguous in memory
+  const bool p_is_b = g.vc.ks_in == 1 || g.vc.rs_in != 1;
+  Job j;
+  j.p = p_is_b ? make_side(g.B, g.vb, g.bb, no, ni) : make_side(g.A, g.va, g.ba, no, ni);
+  j.q = p_is_b ? make_side(g.A, g.va, g.ba, no, ni) : make_side(g.B, g.vb, g.bb, no, ni);
+  const int pr = p_is_b ? g.N : g.M, qr = p_is_b ? g.M : g.N;
+  j.K = g.K;
+  j.nks = (g.K + 7) / 8;
+  j.C = g.C;
+  j.bc = g.bc;
+  j.alpha = g.alpha;
+  j.accumulate = g.accumulate;
+  j.status = g.ws->status;
+  const Div rd = make_div(g.vc.rin), kd = make_div(g.vc.kin);
+  j.cp_div = p_is_b ? kd : rd;
+  j.cp_in = p_is_b ? g.vc.ks_in : g.vc.rs_in;
+  j.cp_out = p_is_b ? g.vc.ks_out : g.vc.rs_out;
+  j.cq_div = p_is_b ? rd : kd;
+  j.cq_in = p_is_b ? g.vc.rs_in : g.vc.ks_in;
+  j.cq_out = p_is_b ? g.vc.rs_out : g.vc.ks_out;
+  // 64-column Q tiles halve the operand traffic per product; 32 where K fits one or two chunks (two
+  // accumulator sets: the next tile's MMAs run under this one's epilogue) or 64 would pad more
+  const int nt = (j.nks > 2 * kChunkSteps && up(qr, 64) == up(qr, 32)) ? 64 : 32;
+  // bytes per packed row: digits, scale, and the segment maxima of long rows
+  const long long row_extra = 8 + (j.nks >= 2 * kSegSteps ? 8 * kMaxSegs : 0);
+  const long long pb = (long long)j.nks * 512 + row_extra, qb = (long long)j.nks * 256 + row_extra;
+  const long long W = (long long)g.ws->bytes - 1024;
+  auto need = [&](long long prow, long long qrow, long long o, long long i) {
+    return up(prow, kPTile) * pb * (j.p.dep_o ? o : 1) * (j.p.dep_i ? i : 1) +
+           up(qrow, nt) * qb * (j.q.dep_o ? o : 1) * (j.q.dep_i ? i : 1);
+  };
+  long long go = no, gi = ni, prc = pr, qrc = qr;
+  while (go > 1 && need(pr, qr, go, gi) > W) go = (go + 1) / 2;
+  while (gi > 1 && need(pr, qr, go, gi) > W) gi = (gi + 1) / 2;
+  if (need(pr, qr, go, gi) > W) {
+    qrc = std::min<long long>(qr, (W / 2) / qb / nt * nt);
+    if (qrc <= 0) return GW_OK;
+    prc = std::min<long long>(pr, (W - up(qrc, nt) * qb) / pb / kPTile * kPTile);
+    if (prc <= 0) return GW_OK;
+  }
+  *done = true;
+  for (long long o0 = 0; o0 < no; o0 += go)
+    for (long long i0 = 0; i0 < ni; i0 += gi)
+      for (long long q0 = 0; q0 < qr; q0 += qrc)
+        for (long long p0 = 0; p0 < pr; p0 += prc) {
+          j.o0 = (int)o0;
+          j.i0 = (int)i0;
+          j.no = (int)std::min(go, no - o0);
+          j.ni = (int)std::min(gi, ni - i0);
+          for (Side* s : {&j.p, &j.q}) {
+            s->no = s->dep_o ? j.no : 1;
+            s->ni = s->dep_i ? j.ni : 1;
+          }
+          j.p.row0 = (int)p0;
+          j.p.rows = (int)std::min(prc, pr - p0);
+          j.p.tiles = (j.p.rows + kPTile - 1) / kPTile;
+          j.q.row0 = (int)q0;
+          j.q.rows = (int)std::min(qrc, qr - q0);
+          j.q.tiles = (j.q.rows + nt - 1) / nt;
+          const long long pn = (long long)j.p.no * j.p.ni * j.p.tiles * kPTile;
+          const long long qn = (long long)j.q.no * j.q.ni * j.q.tiles * nt;
+          unsigned char* m = (unsigned char*)g.ws->mem;
+          j.p.dst = m;
+          j.q.dst = m + pn * j.nks * 512;
+          j.p.scale = reinterpret_cast<double*>(j.q.dst + qn * j.nks * 256);
+          j.q.scale = j.p.scale + pn;
+          // few tiles, long K: share a tile's chunks among CTAs so that every SM has work (the partial
+          // sums take what the digits leave of the workspace)
+          const long long tiles = (long long)j.p.tiles * j.q.tiles * j.no * j.ni;
+          const int nchunks = (j.nks + kChunkSteps - 1) / kChunkSteps;
+          j.ksplit = 1;
+          // long rows are packed in segments where the row tiles alone leave SMs idle (4 blocks an SM)
+          const long long blocks = (long long)j.p.no * j.p.ni * j.p.tiles + (long long)j.q.no * j.q.ni * j.q.tiles;
+          const int segs = (int)std::min<long long>(std::min(j.nks / kSegSteps, kMaxSegs), (8LL * sm_count() + blocks - 1) / blocks);
+          j.seg_steps = (j.nks + std::max(segs, 1) - 1) / std::max(segs, 1);
+          j.segs = (j.nks + j.seg_steps - 1) / j.seg_steps;
+          j.p.pmax = reinterpret_cast<unsigned long long*>(j.q.scale + qn);
+          j.q.pmax = j.p.pmax + (j.segs > 1 ? pn * j.segs : 0);
+          j.part_hi = reinterpret_cast<long long*>(j.q.pmax + (j.segs > 1 ? qn * j.segs : 0));
+          const long long room = (m + g.ws->bytes - reinterpret_cast<unsigned char*>(j.part_hi)) / (128 * nt * 12);
+          if (g.ws->counters && nchunks > 1 && 2 * tiles <= std::min<long long>(kSplitUnits, room)) {
+            const int ks = (int)std::min<long long>(std::min<long long>(kSplitUnits, room) / tiles, nchunks);
+            j.split_chunks = (nchunks + ks - 1) / ks;
+            j.ksplit = (nchunks + j.split_chunks - 1) / j.split_chunks;
+            j.counter = reinterpret_cast<unsigned int*>(g.ws->counters);
+            j.part_lo = reinterpret_cast<uint32_t*>(j.part_hi + tiles * j.ksplit * 128 * nt);
+          }
+          int rc;
+          if (j.nks <= kChunkSteps)
+            rc = nt == 64 ? launch_gemm<64, false>(j, g.slot, st) : launch_gemm<32, false>(j, g.slot, st);
+          else
+            rc = nt == 64 ? launch_gemm<64, true>(j, g.slot, st) : launch_gemm<32, true>(j, g.slot, st);
+          if (rc != GW_OK) return rc;
+        }
+  return GW_OK;
+}
+
+}  // namespace gwi
