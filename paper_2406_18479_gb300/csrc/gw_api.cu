@@ -135,14 +135,13 @@ struct gw_ctx {
   // the 129 MB L2 between the packing and the GEMM. The FP64 contractions have their own (oz_mem).
   unsigned char *oz_mem = nullptr, *oz_small = nullptr, *oz_count = nullptr;
   size_t oz_bytes = 0;
-  Oz64Ws oz_fwd, oz_back, oz_w, oz;
+  Oz64Ws oz_fwd, oz_back, oz_w, oz_inv, oz;
   double2 *P0t = nullptr, *Pw = nullptr, *Pt = nullptr;
   double2* dyson_ws = nullptr;            // nk * nwf * nao2
   std::vector<int> mq;                    // index of -q for every q
   int* mq_dev = nullptr;
   int* wlist = nullptr;                   // canonical (q, n) matrices of P~(i Omega), as q * nwb + n
   int* wlist_q = nullptr;                 // (q, n) matrices of a q range (gw_sigma_eval_q)
-  std::vector<int> wlist_host;            // host copy of wlist (the items of a grouped inversion)
   int nwlist = 0;
   int* status = nullptr;                  // device flags: [0] singular matrix
   double* maxdiff = nullptr;
@@ -404,7 +403,7 @@ int aux_dyson(gw_ctx* c, const double2* P0w, double2* Pw) {
           cudaSuccess)
     return cuda_check("aux_dyson copy");
   GW_TRY(add_identity_fp64(Pw, c->naux, n2, nb, -1.0, 1.0, c->stream));   // I - P0
-  GW_TRY(batched_inverse_fp64(Pw, c->naux, n2, nb, c->status, c->stream));
+  GW_TRY(batched_inverse_fp64(Pw, c->naux, n2, nb, c->status, c->stream, nullptr, &c->oz_inv));
   GW_TRY(add_identity_fp64(Pw, c->naux, n2, nb, 1.0, -1.0, c->stream));   // (I - P0)^-1 - I
   return GW_OK;
 }
@@ -463,7 +462,7 @@ int screened_sym(gw_ctx* c, const double2* P0t, double2* Pt, int q0 = 0, int q1 
   const int* list = nullptr;
   int nlist = 0;
   GW_TRY(screened_sym_pre(c, P0t, q0, q1, &list, &nlist));
-  if (nlist > 0) GW_TRY(batched_inverse_fp64(c->Pw, c->naux, c->naux2, nlist, c->status, c->stream, list));
+  if (nlist > 0) GW_TRY(batched_inverse_fp64(c->Pw, c->naux, c->naux2, nlist, c->status, c->stream, list, &c->oz_inv));
   return screened_sym_post(c, Pt, q0, q1, list, nlist);
 }
 
@@ -575,7 +574,6 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
       for (int q = 0; q < nk; ++q)
         for (int n = 0; n < canonical_end(c, q, c->nwb); ++n) wl.push_back(q * c->nwb + n);
       c->nwlist = (int)wl.size();
-      c->wlist_host = wl;
       if ((rc = dev_alloc(c, &c->wlist, wl.size())) != GW_OK) break;
       upload(c, c->wlist, wl.data(), wl.size() * sizeof(int));
       // the (q, n) list of a q range (gw_sigma_eval_q): at most every (q, n)
@@ -643,6 +641,8 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
       c->oz_fwd = ws(c->Pt, nt_bytes);
       c->oz_back = ws(c->P0t, nt_bytes);
       c->oz_w = ws(c->Pw, (size_t)nk * c->nwb * c->naux2 * sizeof(double2));
+      c->oz_inv = c->oz_fwd;   // P~ while the matrices of P(i Omega) are inverted
+      if (nt_bytes > c->oz_inv.bytes) c->oz_inv.bytes = std::min(nt_bytes, kOz64InvBytes);
       c->oz = c->oz_w;
       if (c->oz_bytes > c->oz.bytes) {
         if ((rc = dev_alloc(c, &c->oz_mem, c->oz_bytes)) != GW_OK) break;
@@ -867,16 +867,17 @@ int sigma_eval_part(gw_ctx* ctx, const double2* G, double2* Sig, int part) {
     int nlist = 0;
     return screened_sym_pre(ctx, ctx->P0t, 0, ctx->nk, &list, &nlist);
   }
+  if (part == 1) {
+    ProfScope _ps(&ctx->prof);
+    return batched_inverse_fp64(ctx->Pw, ctx->naux, ctx->naux2, ctx->nwlist, ctx->status, ctx->stream, ctx->wlist,
+                                &ctx->oz_inv);
+  }
   {
     ProfScope _ps(&ctx->prof);
     GW_TRY(screened_sym_post(ctx, ctx->Pt, 0, ctx->nk, ctx->wlist, ctx->nwlist));
   }
   return gw_self_energy(ctx, reinterpret_cast<const gw_c128*>(G), reinterpret_cast<const gw_c128*>(ctx->Pt),
                         reinterpret_cast<gw_c128*>(Sig));
-}
-
-void inverse_items(gw_ctx* ctx, std::vector<GjItem>* items) {
-  for (int w : ctx->wlist_host) items->push_back(GjItem{ctx->Pw + (long long)w * ctx->naux2, ctx->naux, ctx->status});
 }
 
 }  // namespace gwi
@@ -921,7 +922,8 @@ int gw_dyson_G(gw_ctx* ctx, const gw_c128* H_dev, const gw_c128* Sig_dev, gw_c12
   GW_TRY(transform(ctx, 1, true, S, ctx->dyson_ws, ctx->nk, ctx->nao2));
   GW_TRY(build_g_dyson_fp64(ctx->dyson_ws, H, ctx->S, ctx->wf, ctx->cfg.mu, ctx->nk, ctx->nwf, ctx->nao,
                             ctx->stream));
-  GW_TRY(batched_inverse_fp64(ctx->dyson_ws, ctx->nao, ctx->nao2, ctx->nk * ctx->nwf, ctx->status, ctx->stream));
+  GW_TRY(batched_inverse_fp64(ctx->dyson_ws, ctx->nao, ctx->nao2, ctx->nk * ctx->nwf, ctx->status, ctx->stream, nullptr,
+                              &ctx->oz_w));
   GW_TRY(transform(ctx, 1, false, ctx->dyson_ws, G, ctx->nk, ctx->nao2));
   return GW_OK;
 }

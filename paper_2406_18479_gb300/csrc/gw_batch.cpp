@@ -3,13 +3,9 @@
 // few CUDA streams by predicted cost (longest first onto the least-loaded
 // stream), and the whole batch captured once into a CUDA graph whose branches
 // run concurrently; later evaluations are one graph launch. In the grouped
-// modes the aux Dyson inversions of all systems (the FP64 stage whose one
-// launch per system fills few SMs: one block per canonical frequency) run as
-// one launch over the ragged list of every system's matrices (one block per
-// matrix, largest first), between the two halves of each system's
-// evaluation; a system whose aux basis exceeds the blocked kernel's limit
-// (800) keeps its own inversion and runs whole in the first half. A
-// per-system serial loop and eager concurrent streams are kept for comparison.
+// modes the aux Dyson inversions of all systems run side by side, after every
+// system's first and before any system's last stages. A per-system serial
+// loop and eager concurrent streams are kept for comparison.
 //
 // Each system computes exactly what a lone gw_sigma_eval computes: the
 // branches share no memory and no kernel depends on timing.
@@ -46,12 +42,6 @@ struct gw_batch {
   std::vector<const gw_c128*> gG;
   std::vector<gw_c128*> gS;
   int graph_grouped = 0;                 // the captured graph is of the grouped flow
-  // grouped inversion: items of every system, split by panel class (n <= 430, n > 430) so that each
-  // matrix gets the panel width of its lone inversion, largest first; in device memory
-  GjItem* items_dev[2] = {nullptr, nullptr};
-  int items_n[2] = {0, 0}, items_maxn[2] = {0, 0};
-  double items_flops[2] = {0.0, 0.0};
-  std::vector<char> whole;               // systems evaluated whole in the grouped flow (naux > 800)
 };
 
 namespace {
@@ -119,47 +109,6 @@ void fit_tau_batches(gw_batch* b, size_t budget) {
   }
 }
 
-void drop_items(gw_batch* b) {
-  for (int c = 0; c < 2; ++c) {
-    if (b->items_dev[c]) cudaFree(b->items_dev[c]);
-    b->items_dev[c] = nullptr;
-    b->items_n[c] = b->items_maxn[c] = 0;
-    b->items_flops[c] = 0.0;
-  }
-}
-
-// the inversion items of every context, by panel class and largest first
-int build_items(gw_batch* b) {
-  drop_items(b);
-  std::vector<GjItem> all;
-  b->whole.assign(b->n, 0);
-  for (int i = 0; i < b->n; ++i) {
-    if (b->cfg[i].naux > kGjBlockedMaxN8)
-      b->whole[i] = 1;
-    else
-      inverse_items(b->ctx[i], &all);
-  }
-  std::stable_sort(all.begin(), all.end(), [](const GjItem& x, const GjItem& y) { return x.n > y.n; });
-  std::vector<GjItem> cls[2];
-  for (const GjItem& it : all) cls[it.n > kGjBlockedMaxN16 ? 1 : 0].push_back(it);
-  for (int c = 0; c < 2; ++c) {
-    if (cls[c].empty()) continue;
-    if (cudaMalloc(reinterpret_cast<void**>(&b->items_dev[c]), cls[c].size() * sizeof(GjItem)) != cudaSuccess ||
-        cudaMemcpy(b->items_dev[c], cls[c].data(), cls[c].size() * sizeof(GjItem), cudaMemcpyHostToDevice) !=
-            cudaSuccess) {
-      cudaGetLastError();
-      drop_items(b);
-      return fail(GW_ENOMEM, "gw_batch: inversion item list");
-    }
-    b->items_n[c] = (int)cls[c].size();
-    for (const GjItem& it : cls[c]) {
-      b->items_maxn[c] = std::max(b->items_maxn[c], it.n);
-      b->items_flops[c] += 8.0 * (double)it.n * it.n * it.n;
-    }
-  }
-  return GW_OK;
-}
-
 void drop_graph(gw_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   b->exec = nullptr;
@@ -175,7 +124,7 @@ int create_contexts(gw_batch* b) {
     if (b->V[i]) GW_TRY_BATCH(gw_set_coulomb(b->ctx[i], b->V[i]));
   }
   drop_graph(b);
-  return build_items(b);
+  return GW_OK;
 }
 
 // every system on its stream, eager; the streams fork from and join into main
@@ -207,24 +156,17 @@ int join_lanes(gw_batch* b) {
   return GW_OK;
 }
 
-// every system's first half on its stream; all aux Dyson inversions as one launch per panel class
-// on main; every system's second half on its stream
+// every system's evaluation up to the aux Dyson equation on its stream; then every system's inversions;
+// then the rest
 int enqueue_grouped(gw_batch* b, const gw_c128* const* G, gw_c128* const* S) {
-  GW_TRY_BATCH(fork_lanes(b));
   const std::vector<int> order = by_cost(b);
-  for (int i : order)
-    GW_TRY_BATCH(b->whole[i] ? gw_sigma_eval(b->ctx[i], G[i], S[i])
-                             : sigma_eval_part(b->ctx[i], reinterpret_cast<const double2*>(G[i]),
-                                               reinterpret_cast<double2*>(S[i]), 0));
-  GW_TRY_BATCH(join_lanes(b));
-  for (int c = 0; c < 2; ++c)
-    GW_TRY_BATCH(batched_inverse_group_fp64(b->items_dev[c], b->items_n[c], b->items_maxn[c], b->items_flops[c],
-                                            b->main));
-  GW_TRY_BATCH(fork_lanes(b));
-  for (int i : order)
-    if (!b->whole[i])
-      GW_TRY_BATCH(sigma_eval_part(b->ctx[i], reinterpret_cast<const double2*>(G[i]), reinterpret_cast<double2*>(S[i]), 1));
-  return join_lanes(b);
+  for (int part = 0; part < 3; ++part) {
+    GW_TRY_BATCH(fork_lanes(b));
+    for (int i : order)
+      GW_TRY_BATCH(sigma_eval_part(b->ctx[i], reinterpret_cast<const double2*>(G[i]), reinterpret_cast<double2*>(S[i]), part));
+    GW_TRY_BATCH(join_lanes(b));
+  }
+  return GW_OK;
 }
 
 // one system after another, each waiting for the previous one
@@ -353,7 +295,6 @@ int gw_batch_destroy(gw_batch* b) {
     if (s) cudaStreamSynchronize(s);
   if (b->main) cudaStreamSynchronize(b->main);
   drop_graph(b);
-  drop_items(b);
   for (gw_ctx* c : b->ctx)
     if (c) gw_destroy(c);
   for (cudaEvent_t e : b->ev)

@@ -87,7 +87,8 @@ struct Oz64Ws {
   int* status = nullptr;
 };
 
-constexpr size_t kOz64L2Bytes = 96ull << 20, kOz64SmallBytes = 4ull << 20;
+constexpr size_t kOz64L2Bytes = 96ull << 20, kOz64SmallBytes = 4ull << 20,
+                 kOz64InvBytes = 1ull << 30;   // groups of matrices large enough to fill the GPU four blocks an SM
 
 struct ZGemm {
   int M = 0, N = 0, K = 0, nbatch = 1, bin = 1 << 30;
@@ -114,29 +115,17 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done);
 size_t oz64_bytes(long long p_rows, long long q_rows, int K);
 size_t oz64_counter_bytes();
 
-// In-place Gauss-Jordan inversion with partial pivoting of nbatch n x n matrices
-// (matrix b at base + b * stride). diag_shift: before inverting, M <- diag_sign*M + shift(b)*I
-// is applied by the callers' build kernels instead; here only the inversion.
-// list (optional, device): the matrix indices to process, nbatch of them.
+// In-place Gauss-Jordan inversion with partial pivoting of nbatch n x n matrices (matrix b at
+// base + b * stride). list (optional, device): the matrix indices to process, nbatch of them.
+// From kGjPanelMinN on, with a digit workspace of at least one matrix's digits, pivot rows and swaps,
+// the rank-B updates of the panels run on the tensor cores to FP64 accuracy; below it the whole
+// inversion is one block per matrix on the FP64 pipe; above kGjPanelMaxN8 (or without a workspace)
+// it goes column by column. The route follows n and the workspace's size, never the batch.
 int batched_inverse_fp64(double2* base, int n, long long stride, int nbatch, int* status_dev,
-                         void* stream, const int* list = nullptr);
-
-// One matrix of a grouped inversion: its pointer (n x n, row-major), size and status word.
-// largest matrix the blocked Gauss-Jordan inversion takes with a 16-column panel and with an
-// 8-column panel (its shared-memory footprint); larger ones take the unblocked kernel
-constexpr int kGjBlockedMaxN16 = 430;
-constexpr int kGjBlockedMaxN8 = 800;
-struct GjItem {
-  double2* M;
-  int n;
-  int* status;
-};
-// Gauss-Jordan inversion of a ragged list of matrices (items in device memory, count of them,
-// the largest n at most 800) in one launch, one block per item in list order; flops for the
-// profile. The panel width follows max_n (16 up to 430, else 8), as batched_inverse_fp64's does
-// for one n, so a matrix gets bit for bit what a lone inversion of its size gives when both
-// take the same panel width.
-int batched_inverse_group_fp64(const GjItem* items_dev, int count, int max_n, double flops, void* stream);
+                         void* stream, const int* list = nullptr, const Oz64Ws* ws = nullptr);
+// panels of 16 columns up to kGjPanelMaxN16, of 8 up to kGjPanelMaxN8 (a panel and its pivot column in
+// shared memory: n (B + 1) 16 bytes)
+constexpr int kGjPanelMinN = 64, kGjPanelMaxN16 = 800, kGjPanelMaxN8 = 1536;
 
 // Aux Dyson pieces: M <- I - M; and after inversion M <- M - I.
 int add_identity_fp64(double2* base, int n, long long stride, int nbatch, double scale_m,
@@ -189,13 +178,11 @@ int add_fp64(const double2* a, const double2* b, double2* c, long long n, void* 
 int dot_re_fp64(const double2* x, const double2* y, long long n, double* partial_dev, double* out_dev, void* stream);
 int lincomb_fp64(const double2* const* v, const double* c, int m, double2* out, long long n, void* stream);
 
-// gw_sigma_eval in two parts around the aux Dyson inversions (for batches that invert the
-// matrices of many systems in one launch): part 0 is P0, the forward transforms and I - P0 of
-// the canonical (q, n); then the caller inverts the matrices inverse_items lists (in place, as
-// batched_inverse_fp64 does); part 1 is (I - P0)^{-1} - I, the mirror fills, the back transforms
-// and Sigma. Together they issue exactly the launches of gw_sigma_eval, in its order.
+// gw_sigma_eval in three parts (for batches whose systems run their aux Dyson inversions together): part 0
+// is P0, the forward transforms and I - P0 of
+// the canonical (q, n); part 1 inverts those matrices; part 2 is (I - P0)^{-1} - I, the mirror fills,
+// the back transforms and Sigma. Together they issue exactly the launches of gw_sigma_eval, in its order.
 int sigma_eval_part(gw_ctx* ctx, const double2* G, double2* Sig, int part);
-void inverse_items(gw_ctx* ctx, std::vector<GjItem>* items);
 
 // sizes, stream and mu of a context (for host code outside the file that defines gw_ctx)
 struct CtxInfo {

@@ -214,43 +214,29 @@ __global__ void __launch_bounds__(256) gj_inverse_kernel(double2* base, int n, l
   }
 }
 
-// Blocked form of the same inversion (same pivots, same result up to rounding order), for
-// n <= kGjBlockedMaxN[B]. Columns are taken in panels of B (16, or 8 for larger n, where two
-// 16-column panels no longer fit in shared memory): the panel (n x B) is
+// Blocked form of the same inversion (same pivots, same result up to rounding order), one block per
+// matrix, for small n (below kGjPanelMinN). Columns are taken in panels of B: the panel (n x B) is
 // eliminated in shared memory with partial pivoting (explicit row swaps), written back, the
 // panel's row swaps are applied to the other columns, and those columns receive the panel's
 // effect as one rank-B update,
 //   A[i][c] <- (i in the panel's pivot rows ? 0 : A[i][c]) + sum_t P[i][t] A_old[k0 + t][c],
 // so the matrix is read and written once per panel instead of once per column. The column
 // swaps that undo the row interchanges are applied at the end through one permutation.
-// The size limits (kGjBlockedMaxN16, kGjBlockedMaxN8) keep the dynamic shared memory,
-// n * (2 * B * 16 + 16 + 8) bytes, plus the kernel's static shared memory within 227 KB.
-
 template <int B>
 size_t gj_blocked_smem(int n) {
   return (size_t)n * (2 * B * sizeof(double2) + sizeof(double2) + 2 * sizeof(int));
 }
 
-// One matrix per block: matrix blockIdx.x of base (through list when given), or, with items,
-// the item blockIdx.x (its own pointer, size and status word: a ragged list of matrices from
-// several systems in one launch; the dynamic shared memory is sized for the largest).
+// One matrix per block: matrix blockIdx.x of base (through list when given).
 template <int B>
 __global__ void __launch_bounds__(256) gj_inverse_blocked_kernel(double2* base, int n, long long stride,
-                                                                 const int* list, int* status,
-                                                                 const GjItem* items) {
+                                                                 const int* list, int* status) {
   extern __shared__ double2 sm[];
   __shared__ double red_v[8];
   __shared__ int red_i[8];
   __shared__ int s_p, s_bad;
   __shared__ double2 rowc[B];
-  double2* M;
-  if (items) {
-    M = items[blockIdx.x].M;
-    n = items[blockIdx.x].n;
-    status = items[blockIdx.x].status;
-  } else {
-    M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
-  }
+  double2* M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
   double2* P = sm;                         // [n][B]  panel
   double2* AK = P + (size_t)n * B;         // [B][n]  pivot rows at the panel start; staging at the end
   double2* fcol = AK + (size_t)n * B;      // [n]     pivot column of one step
@@ -395,6 +381,186 @@ __global__ void __launch_bounds__(256) gj_inverse_blocked_kernel(double2* base, 
     for (int e = tid; e < rb * n; e += blockDim.x) {
       const int t = e / n, y = e % n;
       M[(long long)(r0 + t) * n + y] = AK[t * n + pi[y]];
+    }
+    __syncthreads();
+  }
+}
+
+// The same elimination for larger n, its rank-B updates on the tensor cores (zgemm_oz64): per panel
+// of B columns, this kernel (one block per matrix) eliminates the panel in shared memory, writes it
+// back, moves the rows its pivots interchanged, leaves the old pivot rows in ak ([B][n], zero in the
+// panel's columns) and zeros in their place, so that the update is A += P ak over the whole matrix.
+// What stays on the FP64 pipe is n B complex multiply-adds per column instead of n^2. Bound: that
+// (B = 16, n = 200: 6.4k clocks a column; two matrices an SM take 15 us) and the block-wide steps of
+// a column (pivot search, elimination). Against the whole inversion on the FP64 pipe: 2727 matrices of
+// 200 x 200 209 -> 68 ms, 81 of 480 x 480 120 -> 18 ms (one block per matrix left half the SMs idle
+// there; the updates use all). swp[c]: the row swapped with row c at step c.
+template <int B>
+size_t gj_panel_smem(int n) {
+  return (size_t)n * (B + 1) * sizeof(double2);
+}
+template <int B>
+__global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, long long stride, const int* list, int k0,
+                                                       double2* ak_all, int* swp_all, int* status) {
+  extern __shared__ double2 sm[];
+  __shared__ double red_v[8];
+  __shared__ int red_i[8];
+  __shared__ int s_p, s_bad, s_cnt;
+  __shared__ int s_swp[B], s_row[2 * B], s_src[2 * B];
+  __shared__ double2 rowc[B];
+  double2* M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
+  double2* ak = ak_all + (long long)blockIdx.x * B * n;
+  int* swp = swp_all + (long long)blockIdx.x * n;
+  double2* P = sm;                         // [n][B]  panel
+  double2* fcol = P + (size_t)n * B;       // [n]     pivot column of one step
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int kb = min(B, n - k0);
+  if (tid == 0) s_bad = 0;
+  for (int e = tid; e < n * B; e += blockDim.x) {
+    const int i = e / B, j = e % B;
+    P[e] = j < kb ? M[(long long)i * n + k0 + j] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  for (int j = 0; j < kb; ++j) {
+    const int c = k0 + j;
+    double best = -1.0;
+    int bi = c;
+    for (int i = c + tid; i < n; i += blockDim.x) {
+      const double2 v = P[i * B + j];
+      const double a = v.x * v.x + v.y * v.y;
+      if (a > best) { best = a; bi = i; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ob = __shfl_down_sync(0xffffffffu, best, o);
+      const int oi = __shfl_down_sync(0xffffffffu, bi, o);
+      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    if (lane == 0) { red_v[warp] = best; red_i[warp] = bi; }
+    __syncthreads();
+    if (tid == 0) {
+      double bb = red_v[0];
+      int ii = red_i[0];
+      for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+        if (red_v[w] > bb || (red_v[w] == bb && red_i[w] < ii)) { bb = red_v[w]; ii = red_i[w]; }
+      s_p = ii;
+      s_swp[j] = ii;
+      if (!(bb > 0.0)) s_bad = 1;
+    }
+    __syncthreads();
+    if (s_bad) break;
+    const int p = s_p;
+    // rows p and c change places as they are read: row c's elimination writes what row p held
+    const double2 pv = P[p * B + j];
+    const double den = pv.x * pv.x + pv.y * pv.y;
+    const double2 inv = make_double2(pv.x / den, -pv.y / den);
+    for (int i = tid; i < n; i += blockDim.x) fcol[i] = P[(i == p ? c : i) * B + j];
+    double2 keep = make_double2(0.0, 0.0);
+    if (tid < B) {
+      keep = P[c * B + tid];
+      rowc[tid] = (tid == j) ? inv : cmul(P[p * B + tid], inv);
+    }
+    __syncthreads();
+    if (tid < B && p != c) P[p * B + tid] = keep;
+    __syncthreads();
+    for (int e = tid; e < n * B; e += blockDim.x) {
+      const int i = e / B, jj = e % B;
+      if (jj >= kb) continue;
+      if (i == c) {
+        P[e] = rowc[jj];
+      } else {
+        const double2 f = fcol[i], r = rowc[jj];
+        double2 v = jj == j ? make_double2(0.0, 0.0) : P[e];
+        v.x = fma(-f.x, r.x, v.x);
+        v.x = fma(f.y, r.y, v.x);
+        v.y = fma(-f.x, r.y, v.y);
+        v.y = fma(-f.y, r.x, v.y);
+        P[e] = v;
+      }
+    }
+    __syncthreads();
+  }
+  if (s_bad) {
+    if (tid == 0) atomicExch(status, 1);
+    for (int t = tid; t < kb; t += blockDim.x) swp[k0 + t] = k0 + t;
+    return;
+  }
+  for (int e = tid; e < n * B; e += blockDim.x) {
+    const int i = e / B, j = e % B;
+    if (j < kb) M[(long long)i * n + k0 + j] = P[e];
+  }
+  if (tid < kb) swp[k0 + tid] = s_swp[tid];
+  if (tid == 0) {   // the swaps as one move: row s_row[t] takes what row s_src[t] held
+    int cnt = kb;
+    for (int t = 0; t < kb; ++t) s_row[t] = s_src[t] = k0 + t;
+    for (int j = 0; j < kb; ++j) {
+      const int p = s_swp[j];
+      int at = -1;
+      for (int t = 0; t < cnt; ++t)
+        if (s_row[t] == p) at = t;
+      if (at < 0) {
+        at = cnt++;
+        s_row[at] = s_src[at] = p;
+      }
+      const int x = s_src[j];
+      s_src[j] = s_src[at];
+      s_src[at] = x;
+    }
+    s_cnt = cnt;
+  }
+  __syncthreads();
+  const int cnt = s_cnt;
+  for (int col = tid; col < n; col += blockDim.x) {
+    if (col >= k0 && col < k0 + kb) {
+      for (int t = 0; t < B; ++t) ak[(long long)t * n + col] = make_double2(0.0, 0.0);
+      continue;
+    }
+    double2 v[2 * B];
+#pragma unroll
+    for (int t = 0; t < 2 * B; ++t)
+      if (t < cnt) v[t] = M[(long long)s_src[t] * n + col];
+#pragma unroll
+    for (int t = 0; t < 2 * B; ++t)
+      if (t < cnt) {
+        if (t < kb) ak[(long long)t * n + col] = v[t];
+        M[(long long)s_row[t] * n + col] = t < kb ? make_double2(0.0, 0.0) : v[t];
+      }
+  }
+}
+
+// Undoes the row interchanges as column swaps in reverse order, composed into one permutation; a
+// block takes every gridDim.y-th group of kPermRows rows of its matrix.
+constexpr int kPermRows = 4;
+inline size_t gj_permute_smem(int n) { return (size_t)n * (kPermRows * sizeof(double2) + 2 * sizeof(int)); }
+__global__ void __launch_bounds__(256) gj_permute_kernel(double2* base, int n, long long stride, const int* list,
+                                                         const int* swp_all) {
+  extern __shared__ double2 sm[];
+  int* pi = reinterpret_cast<int*>(sm + (size_t)kPermRows * n);
+  int* sw = pi + n;
+  double2* M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
+  const int* swp = swp_all + (long long)blockIdx.x * n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    pi[i] = i;
+    sw[i] = swp[i];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int c = n - 1; c >= 0; --c) {
+      const int r = sw[c];
+      if (r != c) {
+        const int t = pi[c];
+        pi[c] = pi[r];
+        pi[r] = t;
+      }
+    }
+  __syncthreads();
+  for (int r0 = blockIdx.y * kPermRows; r0 < n; r0 += gridDim.y * kPermRows) {
+    const int rb = min(kPermRows, n - r0);
+    for (int e = threadIdx.x; e < rb * n; e += blockDim.x) sm[e] = M[(long long)r0 * n + e];
+    __syncthreads();
+    for (int e = threadIdx.x; e < rb * n; e += blockDim.x) {
+      const int t = e / n, y = e % n;
+      M[(long long)(r0 + t) * n + y] = sm[t * n + pi[y]];
     }
     __syncthreads();
   }
@@ -796,40 +962,96 @@ int zgemm_fp64(const ZGemm& g, void* stream) {
 }
 
 namespace {
+
+// one-time setup; function-local statics initialise once even when contexts run on several threads
 template <int B>
-bool gj_blocked_attr() {
-  static const bool ok = [] {
-    const int maxn = B == 16 ? kGjBlockedMaxN16 : kGjBlockedMaxN8;
-    const bool r = cudaFuncSetAttribute(gj_inverse_blocked_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)gj_blocked_smem<B>(maxn)) == cudaSuccess;
-    cudaGetLastError();
-    return r;
-  }();
+bool gj_panel_attr() {
+  static const bool ok = cudaFuncSetAttribute(gj_panel_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)gj_panel_smem<B>(B == 16 ? kGjPanelMaxN16 : kGjPanelMaxN8)) == cudaSuccess &&
+                         cudaFuncSetAttribute(gj_permute_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)gj_permute_smem(kGjPanelMaxN8)) == cudaSuccess;
   return ok;
 }
 
+size_t gj_group_bytes(int n, int B) { return oz64_bytes(n, n, B) + (size_t)n * (B * sizeof(double2) + sizeof(int)); }
+
+// Panels and tensor-core updates of groups of matrices whose digits, pivot rows and swaps fit ws
 template <int B>
-int launch_gj_blocked(double2* base, int n, long long stride, int nblocks, int* status_dev, cudaStream_t st,
-                      const int* list, const GjItem* items, double flops, double bytes) {
-  if (!gj_blocked_attr<B>()) return fail(GW_ECUDA, "gj_inverse_blocked: shared memory attribute refused");
-  prof_begin(SLOT_INVERSE_FP64, st);
-  gj_inverse_blocked_kernel<B><<<nblocks, 256, gj_blocked_smem<B>(n), st>>>(base, n, stride, list, status_dev, items);
-  prof_end(SLOT_INVERSE_FP64, st, flops, bytes);
+int inverse_panels(double2* base, int n, long long stride, int nbatch, int* status, cudaStream_t st, const int* list,
+                   const Oz64Ws& ws) {
+  if (!gj_panel_attr<B>()) return fail(GW_ECUDA, "gj_panel: shared memory attribute refused");
+  const int group = (int)std::min<size_t>(nbatch, std::max<size_t>(1, ws.bytes / gj_group_bytes(n, B)));
+  const int ngroups = (nbatch + group - 1) / group;
+  for (int g = 0; g < ngroups; ++g) {
+    const int m0 = (int)((long long)nbatch * g / ngroups), m1 = (int)((long long)nbatch * (g + 1) / ngroups), m = m1 - m0;
+    double2* b0 = list ? base : base + (long long)m0 * stride;
+    const int* l0 = list ? list + m0 : nullptr;
+    double2* ak = reinterpret_cast<double2*>(ws.mem);
+    int* swp = reinterpret_cast<int*>(ak + (size_t)m * B * n);
+    const size_t head = ((size_t)m * n * (B * sizeof(double2) + sizeof(int)) + 255) / 256 * 256;
+    Oz64Ws rest = ws;
+    rest.mem = (unsigned char*)ws.mem + head;
+    rest.bytes = ws.bytes - head;
+    for (int k0 = 0; k0 < n; k0 += B) {
+      const int kb = std::min(B, n - k0);
+      prof_begin(SLOT_INVERSE_FP64, st);
+      gj_panel_kernel<B><<<m, 256, gj_panel_smem<B>(n), st>>>(b0, n, stride, l0, k0, ak, swp, status);
+      prof_end(SLOT_INVERSE_FP64, st, 8.0 * m * (double)n * kb * kb, 32.0 * m * (double)n * (2 * kb));
+      ZGemm z;                               // A += P ak
+      z.M = n;
+      z.N = n;
+      z.K = kb;
+      z.nbatch = m;
+      z.A = b0 + k0;
+      z.va.rs_in = n;
+      z.va.ks_in = 1;
+      z.ba.list = l0;
+      z.ba.bs_in = stride;
+      z.B = ak;
+      z.vb.rs_in = 1;
+      z.vb.ks_in = n;
+      z.bb.bs_in = (long long)B * n;
+      z.C = b0;
+      z.vc.rs_in = n;
+      z.vc.ks_in = 1;
+      z.bc = z.ba;
+      z.accumulate = 1;
+      z.slot = SLOT_INVERSE_FP64;
+      z.ws = &rest;
+      bool done = false;
+      const int rc = zgemm_oz64(z, st, &done);
+      if (rc != GW_OK) return rc;
+      if (!done) return fail(GW_ENOMEM, "batched_inverse: digit workspace of %zu bytes too small for n=%d", ws.bytes, n);
+    }
+    const int rows = std::max(1, std::min((n + kPermRows - 1) / kPermRows, (1216 + m - 1) / m));
+    prof_begin(SLOT_INVERSE_FP64, st);
+    gj_permute_kernel<<<dim3(m, rows), 256, gj_permute_smem(n), st>>>(b0, n, stride, l0, swp);
+    prof_end(SLOT_INVERSE_FP64, st, 0.0, 32.0 * m * (double)n * n);
+  }
   const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "gj_inverse_blocked launch: %s", cudaGetErrorString(e));
+  return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "gj_panel launch: %s", cudaGetErrorString(e));
 }
+
 }  // namespace
 
 int batched_inverse_fp64(double2* base, int n, long long stride, int nbatch, int* status_dev,
-                         void* stream, const int* list) {
+                         void* stream, const int* list, const Oz64Ws* ws) {
   if (nbatch <= 0) return GW_OK;
+  cudaStream_t st = (cudaStream_t)stream;
+  if (n >= kGjPanelMinN && n <= kGjPanelMaxN8 && ws && ws->mem) {
+    if (n <= kGjPanelMaxN16 && ws->bytes >= gj_group_bytes(n, 16))
+      return inverse_panels<16>(base, n, stride, nbatch, status_dev, st, list, *ws);
+    if (n > kGjPanelMaxN16 && ws->bytes >= gj_group_bytes(n, 8))
+      return inverse_panels<8>(base, n, stride, nbatch, status_dev, st, list, *ws);
+  }
   const double flops = 8.0 * (double)n * n * n * nbatch, bytes = 32.0 * (double)n * n * nbatch;
-  if (n <= kGjBlockedMaxN16)
-    return launch_gj_blocked<16>(base, n, stride, nbatch, status_dev, (cudaStream_t)stream, list, nullptr, flops,
-                                 bytes);
-  if (n <= kGjBlockedMaxN8)
-    return launch_gj_blocked<8>(base, n, stride, nbatch, status_dev, (cudaStream_t)stream, list, nullptr, flops,
-                                bytes);
+  if (n < kGjPanelMinN) {
+    prof_begin(SLOT_INVERSE_FP64, st);
+    gj_inverse_blocked_kernel<16><<<nbatch, 256, gj_blocked_smem<16>(n), st>>>(base, n, stride, list, status_dev);
+    prof_end(SLOT_INVERSE_FP64, st, flops, bytes);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "gj_inverse_blocked launch: %s", cudaGetErrorString(e));
+  }
   const size_t smem = 2 * (size_t)n * sizeof(double2) + (size_t)n * sizeof(int);
   if (smem > 200 * 1024) return fail(GW_EINVAL, "batched_inverse_fp64: n=%d too large", n);
   static const bool attr_set = [] {   // once, also when several threads launch
@@ -837,10 +1059,9 @@ int batched_inverse_fp64(double2* base, int n, long long stride, int nbatch, int
     return true;
   }();
   (void)attr_set;
-  prof_begin(SLOT_INVERSE_FP64, (cudaStream_t)stream);
-  gj_inverse_kernel<<<nbatch, 256, smem, (cudaStream_t)stream>>>(base, n, stride, list, status_dev);
-  prof_end(SLOT_INVERSE_FP64, (cudaStream_t)stream, 8.0 * (double)n * n * n * nbatch,
-           32.0 * (double)n * n * nbatch);
+  prof_begin(SLOT_INVERSE_FP64, st);
+  gj_inverse_kernel<<<nbatch, 256, smem, st>>>(base, n, stride, list, status_dev);
+  prof_end(SLOT_INVERSE_FP64, st, flops, bytes);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "gj_inverse launch: %s", cudaGetErrorString(e));
 }
@@ -1036,21 +1257,6 @@ int lincomb_fp64(const double2* const* v, const double* c, int m, double2* out, 
   prof_end(SLOT_ELEMENTWISE, (cudaStream_t)stream, 4.0 * n * m, 16.0 * n * (m + 1));
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "lincomb launch: %s", cudaGetErrorString(e));
-}
-
-}  // namespace gwi
-
-namespace gwi {
-
-int batched_inverse_group_fp64(const GjItem* items_dev, int count, int max_n, double flops, void* stream) {
-  if (count <= 0) return GW_OK;
-  if (max_n > kGjBlockedMaxN8) return fail(GW_EINVAL, "batched_inverse_group_fp64: n = %d above %d", max_n, kGjBlockedMaxN8);
-  const double bytes = 32.0 * (double)max_n * max_n * count;
-  if (max_n <= kGjBlockedMaxN16)
-    return launch_gj_blocked<16>(nullptr, max_n, 0, count, nullptr, (cudaStream_t)stream, nullptr, items_dev, flops,
-                                 bytes);
-  return launch_gj_blocked<8>(nullptr, max_n, 0, count, nullptr, (cudaStream_t)stream, nullptr, items_dev, flops,
-                              bytes);
 }
 
 }  // namespace gwi

@@ -52,6 +52,7 @@ constexpr int kK = 16;              // real k per MMA
 constexpr int kChunkSteps = 8;      // k-steps per exact chunk (128 real k)
 constexpr int kPTile = 64;          // complex rows of P per tile (128 TMEM lanes)
 constexpr int kScaleMax = 480;      // |E| beyond this takes the plain FP64 loop
+constexpr int kEpiWarps = 16;
 constexpr int kSegSteps = 8;        // least k-steps of a packing segment
 constexpr int kMaxSegs = 32;
 constexpr int kSplitUnits = 152;    // tiles x splits of a split-K launch, at most (one wave)
@@ -294,7 +295,7 @@ struct Oz64Shape {
   static constexpr int kStages = NT == 64 ? 4 : 5;
   static constexpr int kBufCols = kDigits * NT;
   static constexpr int kBufs = 512 / kBufCols;                  // accumulator sets in TMEM
-  static constexpr int kThreads = 320;                          // producer, MMA, 8 epilogue warps
+  static constexpr int kThreads = 64 + 32 * kEpiWarps;          // producer, MMA, epilogue warps
   static constexpr size_t kSmem = 128 + (size_t)kStages * kStageBytes + 256;
   static_assert(kSmem <= 232448, "stages exceed shared memory");
 };
@@ -310,23 +311,38 @@ __device__ __forceinline__ uint64_t core_desc(uint32_t saddr) {
   return d;
 }
 
-// hi 2^32 + lo += sum_o a_o 256^(7 - o), a_o the exact integer accumulators of one chunk
-__device__ __forceinline__ void join_orders(const float (&v)[kDigits][4], int u, long long& hi, uint32_t& lo) {
+// old + alpha 2^e (hi 2^32 + lo) for |hi|, |lo| < 2^51: the integers become FP64 by an addition to the bits
+// of 1.5 2^52 (scaled by 2^e) and that is taken off again, exactly; no branch and three FP64 operations,
+// so that a thread's outputs overlap (the general form, to_fp64, is 200 instructions in a row)
+__device__ __forceinline__ double finish(long long hi, long long lo, int e, double alpha, double old) {
+  const long long es = (long long)e << 52;
+  const double h = __longlong_as_double(0x4338000000000000ll + hi + es);
+  const double l = __longlong_as_double(0x4338000000000000ll + lo + es);
+  const double k = __longlong_as_double(0x4538000000180000ll + es);      // 2^e (1.5 2^84 + 1.5 2^52)
+  return fma(fma(h, 4294967296.0, -k) + l, alpha, old);
+}
+constexpr int kFinishSteps = 64 * kChunkSteps;     // k-steps up to which hi stays below 2^51
+
+// the exact integer accumulators a_o of one chunk as hi 2^32 + lo = sum_o a_o 256^(7 - o)
+__device__ __forceinline__ void join_chunk(const float (&v)[kDigits][4], int u, long long& hi, long long& lo) {
   int a[kDigits];
 #pragma unroll
   for (int o = 0; o < kDigits; ++o) a[o] = __float2int_rn(v[o][u]);
   // leading digits are within 64, so |a0| <= 2^19, |a1| <= 2^21, |a2| <= 2^22: no overflow in 32 bits
-  const int h0 = a[0] * 256 + a[1], h1 = a[2] * 256 + a[3];
-  hi += (long long)h0 * 65536 + h1;
-  const long long l = (long long)a[4] * 16777216 + (long long)a[5] * 65536 + (long long)a[6] * 256 + a[7] +
-                      (long long)(unsigned long long)lo;
-  hi += l >> 32;
+  hi = (long long)(a[0] * 256 + a[1]) * 65536 + (a[2] * 256 + a[3]);
+  lo = (long long)a[4] * 16777216 + (long long)a[5] * 65536 + (long long)a[6] * 256 + a[7];
+}
+
+// the same, added to a running hi 2^32 + lo with 0 <= lo < 2^32
+__device__ __forceinline__ void join_orders(const float (&v)[kDigits][4], int u, long long& hi, uint32_t& lo) {
+  long long h, l;
+  join_chunk(v, u, h, l);
+  l += (long long)(unsigned long long)lo;
+  hi += h + (l >> 32);
   lo = (uint32_t)l;
 }
 
-// (hi 2^32 + lo) 2^e rounded to FP64, in integer arithmetic: int64 -> FP64 conversions and scalings run
-// on the FP64 pipe (2 a clock and SM), which five of them per output would make the bound of short
-// products (a rank-16 update: 12k clocks a tile, against 1.2k of MMAs)
+// (hi 2^32 + lo) 2^e rounded to FP64, in integer arithmetic, for sums of any length
 __device__ __forceinline__ double to_fp64(long long hi, uint32_t lo, int e) {
   const long long neg = hi >> 63;
   unsigned long long H = (unsigned long long)(hi ^ neg);
@@ -353,7 +369,7 @@ __device__ __forceinline__ double to_fp64(long long hi, uint32_t lo, int e) {
 }
 
 template <int NT, bool MULTI>
-__global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant__ Job j) {
+__global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const __grid_constant__ Job j) {
   using S = Oz64Shape<NT>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -373,7 +389,7 @@ __global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant
     }
     for (int b = 0; b < S::kBufs; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 8);
+      mbar_init(&acc_empty[b], kEpiWarps);
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
@@ -481,9 +497,11 @@ __global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant
       }
     }
   } else {
-    // epilogue: TMEM lane quarter warp % 4, columns [half NT/2, half NT/2 + NT/2)
+    // epilogue: TMEM lane quarter warp % 4, columns [half kCols, (half + 1) kCols). 16 warps: each output
+    // is a long chain (8 conversions, the joins, three FP64 operations), and two warps a scheduler
+    // left it idle three clocks in four
     const int quarter = warp & 3, half = (warp - 2) >> 2;
-    constexpr int kCols = NT / 2;
+    constexpr int kCols = NT * 4 / kEpiWarps;
     const int lrow = quarter * 32 + lane;
     const int part = lrow & 1;
     uint32_t chunk = 0;
@@ -500,17 +518,34 @@ __global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant
       const int ap = j.p.row0 + (p_ok ? pr : 0), apq = div_by(ap, j.cp_div);
       double* C = reinterpret_cast<double*>(j.C + batch_in(j.bc, bi) + (long long)bo * j.bc.bs_out + (long long)apq * j.cp_out +
                                             (long long)(ap - apq * j.cp_div.d) * j.cp_in) + part;
-      auto put = [&](int col, long long hi, uint32_t lo) {
-        const int qr = qt * NT + col;
-        if (!p_ok || qr >= j.q.rows) return;
-        const int eq = __double2hiint(sq[col]) >> 20;
-        double x = ep == 0x7FF || eq == 0x7FF ? plain_dot(j, bo, bi, ap, j.q.row0 + qr, part)
-                                              : to_fp64(hi, lo, ep + eq - 2046);
-        if (j.alpha != 1.0) x *= j.alpha;
-        const int aq = j.q.row0 + qr, aqq = div_by(aq, j.cq_div);
-        double* c = C + 2 * ((long long)aqq * j.cq_out + (long long)(aq - aqq * j.cq_div.d) * j.cq_in);
-        *c = j.accumulate ? *c + x : x;
+      // output element of tile column col (P row fixed per thread)
+      auto at = [&](int col) {
+        const int aq = j.q.row0 + qt * NT + col, aqq = div_by(aq, j.cq_div);
+        return C + 2 * ((long long)aqq * j.cq_out + (long long)(aq - aqq * j.cq_div.d) * j.cq_in);
       };
+      auto col_ok = [&](int col) { return p_ok && qt * NT + col < j.q.rows; };
+      bool special = false;           // some output needs the plain loop (done after the others)
+      const bool quick = j.nks <= kFinishSteps;
+      auto put = [&](int col, long long hi, long long lo, double old) {
+        const int eq = col_ok(col) ? __double2hiint(sq[col]) >> 20 : 1023;
+        const bool plain = ep == 0x7FF || eq == 0x7FF;
+        const int e = plain ? 0 : ep + eq - 2046;
+        const double x = !MULTI || quick ? finish(hi, lo, e, j.alpha, old)
+                                         : fma(to_fp64(hi, (uint32_t)lo, e), j.alpha, old);
+        if (col_ok(col) && !plain) *at(col) = x;
+        special |= plain && col_ok(col);
+      };
+      // outputs that are added to are read ahead of the wait for the accumulators (a load behind every
+      // store would put 16 memory latencies in a row: 24k clocks a tile instead of 5k)
+      constexpr int kAhead = MULTI ? 1 : kCols;
+      double old[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) old[u] = 0.0;
+      if (!MULTI && j.accumulate) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+          if (col_ok(half * kCols + u)) old[u] = *at(half * kCols + u);
+      }
       long long hi[MULTI ? kCols : 1];
       uint32_t lo[MULTI ? kCols : 1];
       bool ok = true;
@@ -519,7 +554,7 @@ __global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant
         if (!mbar_wait(&acc_full[buf], (chunk / S::kBufs) & 1, abort_flag, j.status, 24)) { ok = false; break; }
         tc_fence_after();
         const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + buf * S::kBufCols + half * kCols;
-#pragma unroll(MULTI ? kCols / 4 : 1)
+#pragma unroll
         for (int g = 0; g < kCols / 4; ++g) {
           float v[kDigits][4];
 #pragma unroll
@@ -536,10 +571,9 @@ __global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant
               if (c == 0) hi[4 * g + u] = 0, lo[4 * g + u] = 0;
               join_orders(v, u, hi[4 * g + u], lo[4 * g + u]);
             } else {
-              long long h = 0;
-              uint32_t l = 0;
-              join_orders(v, u, h, l);
-              put(half * kCols + 4 * g + u, h, l);
+              long long h, l;
+              join_chunk(v, u, h, l);
+              put(half * kCols + 4 * g + u, h, l, old[4 * g + u]);
             }
           }
         }
@@ -559,8 +593,8 @@ __global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant
           __syncwarp();
           unsigned int n = 0;
           if (lane == 0) {
-            n = atomicAdd(&j.counter[t * 8 + warp - 2], 1u);
-            if (n == (unsigned)ksplit - 1) j.counter[t * 8 + warp - 2] = 0;   // ready for the next launch
+            n = atomicAdd(&j.counter[t * kEpiWarps + warp - 2], 1u);
+            if (n == (unsigned)ksplit - 1) j.counter[t * kEpiWarps + warp - 2] = 0;   // ready for the next launch
           }
           if (__shfl_sync(0xffffffffu, n, 0) != (unsigned)ksplit - 1) continue;
           __threadfence();
@@ -576,7 +610,25 @@ __global__ void __launch_bounds__(320, 1) oz64_gemm_kernel(const __grid_constant
           }
         }
 #pragma unroll
-        for (int u = 0; u < kCols; ++u) put(half * kCols + u, hi[u], lo[u]);
+        for (int u0 = 0; u0 < kCols; u0 += 4) {
+          double o4[4] = {0.0, 0.0, 0.0, 0.0};
+          if (j.accumulate) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (col_ok(half * kCols + u0 + u)) o4[u] = *at(half * kCols + u0 + u);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) put(half * kCols + u0 + u, hi[u0 + u], lo[u0 + u], o4[u]);
+        }
+      }
+      if (special) {
+#pragma unroll 1
+        for (int col = half * kCols; col < half * kCols + kCols; ++col) {
+          if (!col_ok(col) || (ep != 0x7FF && __double2hiint(sq[col]) >> 20 != 0x7FF)) continue;
+          const double x = j.alpha * plain_dot(j, bo, bi, ap, j.q.row0 + qt * NT + col, part);
+          double* c = at(col);
+          *c = j.accumulate ? *c + x : x;
+        }
       }
     }
   }
@@ -641,7 +693,7 @@ inline long long up(long long x, long long m) { return (x + m - 1) / m * m; }
 
 }  // namespace
 
-size_t oz64_counter_bytes() { return (size_t)kSplitUnits * 8 * sizeof(unsigned int); }
+size_t oz64_counter_bytes() { return (size_t)kSplitUnits * kEpiWarps * sizeof(unsigned int); }
 
 size_t oz64_bytes(long long p_rows, long long q_rows, int K) {
   const long long nks = (K + 7) / 8;
