@@ -135,7 +135,7 @@ struct gw_ctx {
   // the 129 MB L2 between the packing and the GEMM. The FP64 contractions have their own (oz_mem).
   unsigned char *oz_mem = nullptr, *oz_small = nullptr, *oz_count = nullptr;
   size_t oz_bytes = 0;
-  Oz64Ws oz_fwd, oz_back, oz_w, oz_inv, oz;
+  Oz64Ws oz_fwd, oz_back, oz_w, oz_x, oz_inv, oz;
   double2 *P0t = nullptr, *Pw = nullptr, *Pt = nullptr;
   double2* dyson_ws = nullptr;            // nk * nwf * nao2
   std::vector<int> mq;                    // index of -q for every q
@@ -643,6 +643,9 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
       c->oz_w = ws(c->Pw, (size_t)nk * c->nwb * c->naux2 * sizeof(double2));
       c->oz_inv = c->oz_fwd;   // P~ while the matrices of P(i Omega) are inverted
       if (nt_bytes > c->oz_inv.bytes) c->oz_inv.bytes = std::min(nt_bytes, kOz64InvBytes);
+      c->oz_x = c->oz_w;       // P(i Omega) for the exchange: its long rows fill the GPU in large pieces only
+      const size_t nw_bytes = (size_t)nk * c->nwb * c->naux2 * sizeof(double2);
+      if (nw_bytes > c->oz_x.bytes) c->oz_x.bytes = std::min(nw_bytes, kOz64InvBytes);
       c->oz = c->oz_w;
       if (c->oz_bytes > c->oz.bytes) {
         if ((rc = dev_alloc(c, &c->oz_mem, c->oz_bytes)) != GW_OK) break;
@@ -936,6 +939,69 @@ int gw_density(gw_ctx* ctx, const gw_c128* G_dev, gw_c128* gamma_dev) {
                       ctx->nk, ctx->ntau, ctx->nao, ctx->stream);
 }
 
+}  // extern "C"
+
+namespace {
+
+// The exchange term as two digit products over all (k, k') of a group of k: X = V^{kk'} gamma^{k'} and
+// its contraction with V^{k'k} over (Q, b), the sums over k' reduced in order. The FP64 pipe takes
+// 16 nao^3 flops per (k, k', Q): 36.2 ms on the 3x3x3 solid at nao = 26 (41 GFLOP); this way 12.1, half
+// of it packing. Below 2^23 multiply-adds in all, the former's single launch is the faster one. X and,
+// with a packed V, the unpacked blocks lie in P~ and P0 (not in use outside an evaluation), which hold
+// them for at least one k where ntau naux >= 2 nao^2; the same rule for a full V keeps the two
+// layouts' results alike.
+bool exchange_on_tensor(const gw_ctx* c) {
+  return c->oz_x.mem && c->nao >= 8 && (long long)c->ntau * c->naux >= 2 * c->nao2 &&
+         2.0 * c->nk * c->nk * (double)c->pair * c->nao >= 8388608.0;
+}
+
+int exchange_tensor(gw_ctx* c, bool packed, double2* S) {
+  const int nk = c->nk, nao = c->nao, naux = c->naux;
+  const long long nao2 = c->nao2, pair = c->pair;
+  // k per group: what the P arrays hold, and enough (k, k') tiles for two waves
+  const int room = (int)std::min<long long>((long long)c->ntau * c->naux / (2 * nao2), nk);
+  const int group = std::max(1, std::min(std::min(room, naux), (304 + nk - 1) / nk));
+  for (int k0 = 0; k0 < nk; k0 += group) {
+    const int m = std::min(group, nk - k0);
+    const double2* v1 = c->V + (long long)k0 * nk * pair;       // V^{kk'}: [k][k']
+    const double2* v2 = c->V + (long long)k0 * pair;            // V^{k'k}
+    long long v1k = (long long)nk * pair, v1p = pair, v2k = pair, v2p = (long long)nk * pair;
+    if (packed) {                                               // per k: V^{kk'} of every k', then V^{k'k}
+      for (int k = 0; k < m; ++k) {
+        VPairs L;
+        L.fixed = k0 + k;
+        GW_TRY(unpack_v_fp64(c->Vp, nk, nao, pair, L, 2 * nk, c->P0t + (long long)k * 2 * nk * pair, c->stream));
+      }
+      v1 = c->P0t;
+      v2 = c->P0t + (long long)nk * pair;
+      v1k = v2k = 2ll * nk * pair;
+      v1p = v2p = pair;
+    }
+    double2* X = c->Pt;                                         // [k][k'][b][Q][i]
+    ZGemm a;
+    a.M = naux * nao; a.N = nao; a.K = nao; a.nbatch = m * nk; a.bin = nk;
+    a.A = v1; a.va.rs_in = nao; a.va.ks_in = 1; a.ba.bs_in = v1p; a.ba.bs_out = v1k;
+    a.B = c->gamma; a.vb.rs_in = 1; a.vb.ks_in = nao; a.bb.bs_in = nao2;
+    a.C = X; a.vc.rs_in = 1; a.vc.ks_in = (long long)naux * nao; a.bc.bs_in = pair; a.bc.bs_out = (long long)nk * pair;
+    a.slot = SLOT_STATIC_FP64; a.ws = &c->oz_x;
+    GW_TRY(zgemm_fp64(a, c->stream));
+    ZGemm b;                                                    // k = (Q, b)
+    b.M = nao; b.N = nao; b.K = naux * nao; b.nbatch = m * nk; b.bin = nk;
+    b.A = X; b.va.rs_in = 1; b.va.kin = nao; b.va.ks_in = (long long)naux * nao; b.va.ks_out = nao;
+    b.ba.bs_in = pair; b.ba.bs_out = (long long)nk * pair;
+    b.B = v2; b.vb.rs_in = 1; b.vb.kin = nao; b.vb.ks_in = nao; b.vb.ks_out = nao2; b.bb.bs_in = v2p; b.bb.bs_out = v2k;
+    b.C = c->xinf; b.vc.rs_in = nao; b.vc.ks_in = 1; b.bc.bs_in = nao2; b.bc.bs_out = nk * nao2;
+    b.slot = SLOT_STATIC_FP64; b.ws = &c->oz_x;
+    GW_TRY(zgemm_fp64(b, c->stream));
+    GW_TRY(reduce_partials_fp64(c->xinf, S + k0 * nao2, m, (int)nao2, nk, -1.0 / nk, c->stream));
+  }
+  return GW_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 int gw_sigma_inf(gw_ctx* ctx, const gw_c128* G_dev, gw_c128* SigInf_dev) {
   ProfScope _ps(ctx ? &ctx->prof : nullptr);
   NvtxRange _nr("gw_sigma_inf");
@@ -950,6 +1016,7 @@ int gw_sigma_inf(gw_ctx* ctx, const gw_c128* G_dev, gw_c128* SigInf_dev) {
   const int packed = ctx->V ? 0 : 1;
   GW_TRY(hartree_fp64(Vs, ctx->gamma, ctx->rho, S, nk, naux, nao, ctx->cfg.spin_factor / nk, packed, ctx->stream));
   // exchange: -(1 / N_k) sum_{k'} sum_{Q b} X^{k'}_{Q i b} V^{k'k}_bj(Q), X^{k'}_{Q i b} = sum_a V^{kk'}_ia(Q) gamma^{k'}_ab
+  if (exchange_on_tensor(ctx)) return exchange_tensor(ctx, packed != 0, S);
   if (nao <= kExchangeMaxNao)
     return exchange_fp64(Vs, ctx->gamma, ctx->xinf, S, nk, naux, nao, -1.0 / nk, packed, ctx->stream);
   // per k: X^{k'} = V^{kk'} gamma^{k'} for every k' (one batched product), then S^k -= X^{k'} V^{k'k}

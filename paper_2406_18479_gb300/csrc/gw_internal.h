@@ -168,6 +168,7 @@ int exchange_fp64(const double2* V, const double2* gamma, double2* part, double2
 struct VPairs {
   const long long* tab = nullptr;
   int all = 0;
+  int fixed = -1;   // >= 0: the pairs (fixed, 0..nk-1), then (0..nk-1, fixed)
   int k1[4] = {0, 0, 0, 0}, k2[4] = {0, 0, 0, 0};
 };
 inline long long packed_pairs(int nk) { return (long long)nk * (nk + 1) / 2; }

@@ -726,6 +726,9 @@ __global__ void unpack_v_kernel(const double2* __restrict__ Vp, int nk, int nao,
     } else if (L.all) {
       k1 = b / nk;
       k2 = b % nk;
+    } else if (L.fixed >= 0) {
+      k1 = b < nk ? L.fixed : b - nk;
+      k2 = b < nk ? b : L.fixed;
     } else {
       k1 = L.k1[b];
       k2 = L.k2[b];
@@ -1209,7 +1212,7 @@ int exchange_fp64(const double2* V, const double2* gamma, double2* part, double2
 int unpack_v_fp64(const double2* Vp, int nk, int nao, long long pair, const VPairs& L, int nblocks, double2* dst,
                   void* stream) {
   if (nblocks <= 0) return GW_OK;
-  if (!L.tab && !L.all && nblocks > 4) return fail(GW_EINVAL, "unpack_v: at most four listed pairs");
+  if (!L.tab && !L.all && L.fixed < 0 && nblocks > 4) return fail(GW_EINVAL, "unpack_v: at most four listed pairs");
   const int gx = (int)std::min<long long>((pair + 255) / 256, 1024);
   prof_begin(SLOT_ELEMENTWISE, (cudaStream_t)stream);
   unpack_v_kernel<<<dim3(gx, std::min(nblocks, 65535)), 256, 0, (cudaStream_t)stream>>>(Vp, nk, nao, pair, L, nblocks,

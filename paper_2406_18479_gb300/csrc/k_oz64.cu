@@ -232,13 +232,15 @@ __device__ void pack_tile(const Side& s, const Job& j, long long t) {
                             : __longlong_as_double((long long)(E - 34 + 1023) << 52);
   unsigned char* base = s.dst + ((long long)p.pb * s.tiles + p.tile) * j.nks * (long long)(kDigits * kReal * 32);
   const int rr = PSIDE ? 2 * p.row : p.row;
+  // the padding rows of the last tile stay unwritten: a row of digits meets only its own row of the output
+  if (!p.row_ok) return;
   for (int g = 2 * p.k0 + p.grp; g < 2 * p.k1; g += kGroups) {
     unsigned long long u[8];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int k = 4 * g + c;
       double2 x = make_double2(0.0, 0.0);
-      if (p.row_ok && !zero && k < j.K) x = p.src[side_k(s, k)];
+      if (!zero && k < j.K) x = p.src[side_k(s, k)];
       u[2 * c] = digits_of(x.x, E);
       u[2 * c + 1] = digits_of(x.y, E);
     }

@@ -99,3 +99,32 @@ def test_fp64_contractions_match_oracle(nk3, nao, naux, ntau, chunk):
     assert np.abs(S.cpu().numpy() - ref["Sig"]).max() <= 1e-13 * np.abs(ref["Sig"]).max()
     gw.gw_check_guards(ctx)
     ctx.destroy()
+
+
+@pytest.mark.parametrize("nk3,nao,naux,ntau", [((2, 1, 1), 26, 104, 24), ((3, 1, 1), 27, 70, 30), ((1, 1, 1), 54, 60, 100)])
+def test_static_exchange_matches_oracle(nk3, nao, naux, ntau):
+    """Sigma^inf with its exchange on the tensor cores (both sides of the former kernel's nao limit), full and
+    packed V, against the oracle; the two layouts agree bit for bit."""
+    gw = _gw()
+    from oracle import gw as O
+    from paper_2406_18479_gb300 import inputs as I
+    w = I.Workload("t", nk3, nao, naux, ntau, ntau, 10.0, 0.0, naux / 4.0, nao, solid=nk3 != (1, 1, 1))
+    h, v, g = I.make_inputs(w)
+    # the density is the library's: its extrapolation to beta has its own rounding (1e-12 at 100 nodes)
+    out, ref = [], None
+    for precision, packed in (("fp64", False), ("bf16x4", False), ("bf16x4", True)):
+        ctx = gw.gw_create(nk3, nao, naux, ntau, w.beta, precision=precision, v_packed=packed)
+        V = torch.from_numpy(I.pack_v(v) if packed else v).cuda()
+        gw.gw_set_coulomb(ctx, V)
+        S = torch.empty(ctx.shapes()["H"], dtype=torch.complex128, device="cuda")
+        gamma = torch.empty_like(S)
+        gw.gw_density(ctx, torch.from_numpy(g).cuda(), gamma)
+        gw.gw_sigma_inf(ctx, torch.from_numpy(g).cuda(), S)
+        gw.gw_synchronize(ctx)
+        gw.gw_check_guards(ctx)
+        if ref is None:
+            ref = O.sigma_inf(v, gamma.cpu().numpy(), nk3, spin_factor=2.0)
+        out.append(S.cpu().numpy())
+        ctx.destroy()
+    assert np.abs(out[0] - ref).max() <= 1e-13 * np.abs(ref).max()
+    assert np.array_equal(out[1], out[2]) and np.array_equal(out[0], out[1])
