@@ -386,97 +386,108 @@ __global__ void __launch_bounds__(256) gj_inverse_blocked_kernel(double2* base, 
   }
 }
 
-// The same elimination for larger n, its rank-B updates on the tensor cores (zgemm_oz64): per panel
-// of B columns, this kernel (one block per matrix) eliminates the panel in shared memory, writes it
-// back, moves the rows its pivots interchanged, leaves the old pivot rows in ak ([B][n], zero in the
-// panel's columns) and zeros in their place, so that the update is A += P ak over the whole matrix.
-// What stays on the FP64 pipe is n B complex multiply-adds per column instead of n^2. Bound: that
-// (B = 16, n = 200: 6.4k clocks a column; two matrices an SM take 15 us) and the block-wide steps of
-// a column (pivot search, elimination). Against the whole inversion on the FP64 pipe: 2727 matrices of
-// 200 x 200 209 -> 68 ms, 81 of 480 x 480 120 -> 18 ms (one block per matrix left half the SMs idle
-// there; the updates use all). swp[c]: the row swapped with row c at step c.
+// The inversion for larger n, with only the pivots' search on the FP64 pipe. Per panel of B columns this
+// kernel (one block per matrix) factors rows k0.. of the panel (LU with partial pivoting, in shared
+// memory), inverts the pivot block D, and lays the panel's step out as two products over the whole
+// matrix, which run on the tensor cores (zgemm_oz64):
+//   W = D^{-1} ak,  ak [B][n]: the pivot rows, with the identity in the panel's columns
+//   A += ap W,      ap [n][B]: the negated panel, with the identity in the pivot rows
+// after the rows the pivots interchanged have moved and the panel's columns and the pivot rows of A
+// are zero: the pivot rows become D^{-1} A_p, the panel -A D^{-1}, its pivot block D^{-1}, the rest
+// A - A_panel D^{-1} A_p. On the FP64 pipe that leaves B^2/2 complex multiply-adds per row below k0, a
+// quarter of an elimination of every row; what bounds the kernel now is the chain of a column (search,
+// one division, swap, update: 5 block-wide steps). 303 matrices of 200 x 200 take 167 us a panel (an
+// elimination of every row 242), 81 of 480 x 480 142 us (226). The whole inversion against one block per
+// matrix on the FP64 pipe: 2727 of 200 x 200 209 -> 62 ms, 81 of 480 x 480 120 -> 16.6 ms (half the SMs had
+// no matrix there; the products use all). swp[c]: the row swapped with row c at step c.
 template <int B>
 size_t gj_panel_smem(int n) {
   return (size_t)n * (B + 1) * sizeof(double2);
 }
 template <int B>
 __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, long long stride, const int* list, int k0,
-                                                       double2* ak_all, int* swp_all, int* status) {
+                                                       double2* ak_all, double2* ap_all, double2* dinv_all,
+                                                       int* swp_all, int* status) {
   extern __shared__ double2 sm[];
-  __shared__ double red_v[8];
+  __shared__ long long red_v[8];
   __shared__ int red_i[8];
   __shared__ int s_p, s_bad, s_cnt;
   __shared__ int s_swp[B], s_row[2 * B], s_src[2 * B];
-  __shared__ double2 rowc[B];
+  __shared__ double2 s_inv, D[B][B + 1], drow[B], dcol[B];
   double2* M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
   double2* ak = ak_all + (long long)blockIdx.x * B * n;
+  double2* ap = ap_all + (long long)blockIdx.x * B * n;
+  double2* dinv = dinv_all + (long long)blockIdx.x * B * B;
   int* swp = swp_all + (long long)blockIdx.x * n;
-  double2* P = sm;                         // [n][B]  panel
-  double2* fcol = P + (size_t)n * B;       // [n]     pivot column of one step
+  const int nr = n - k0;                   // rows k0.. of the panel
+  double2* P = sm;                         // [nr][B]
+  double2* fcol = P + (size_t)nr * B;      // [nr]     multipliers of one step
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int kb = min(B, n - k0);
+  const int kb = min(B, nr);
+  auto inverse = [](double2 v) {
+    const double den = v.x * v.x + v.y * v.y;
+    return make_double2(v.x / den, -v.y / den);
+  };
   if (tid == 0) s_bad = 0;
-  for (int e = tid; e < n * B; e += blockDim.x) {
+  for (int e = tid; e < nr * B; e += blockDim.x) {
     const int i = e / B, j = e % B;
-    P[e] = j < kb ? M[(long long)i * n + k0 + j] : make_double2(0.0, 0.0);
+    P[e] = j < kb ? M[(long long)(k0 + i) * n + k0 + j] : make_double2(0.0, 0.0);
   }
   __syncthreads();
   for (int j = 0; j < kb; ++j) {
-    const int c = k0 + j;
-    double best = -1.0;
-    int bi = c;
-    for (int i = c + tid; i < n; i += blockDim.x) {
+    long long best = -1;                   // |v|^2 by its bits (ordered like the value)
+    int bi = j;
+    for (int i = j + tid; i < nr; i += blockDim.x) {
       const double2 v = P[i * B + j];
-      const double a = v.x * v.x + v.y * v.y;
+      const double q = v.x * v.x + v.y * v.y;
+      const long long a = isnan(q) ? -1 : __double_as_longlong(q);
       if (a > best) { best = a; bi = i; }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_down_sync(0xffffffffu, best, o);
+      const long long ob = __shfl_down_sync(0xffffffffu, best, o);
       const int oi = __shfl_down_sync(0xffffffffu, bi, o);
       if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
     }
     if (lane == 0) { red_v[warp] = best; red_i[warp] = bi; }
     __syncthreads();
     if (tid == 0) {
-      double bb = red_v[0];
+      long long bb = red_v[0];
       int ii = red_i[0];
       for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
         if (red_v[w] > bb || (red_v[w] == bb && red_i[w] < ii)) { bb = red_v[w]; ii = red_i[w]; }
       s_p = ii;
-      s_swp[j] = ii;
-      if (!(bb > 0.0)) s_bad = 1;
+      s_swp[j] = k0 + ii;
+      s_inv = inverse(P[ii * B + j]);      // one thread: 256 divisions would cost the FP64 pipe 3k clocks
+      if (!(bb > 0)) s_bad = 1;
     }
     __syncthreads();
     if (s_bad) break;
     const int p = s_p;
-    // rows p and c change places as they are read: row c's elimination writes what row p held
-    const double2 pv = P[p * B + j];
-    const double den = pv.x * pv.x + pv.y * pv.y;
-    const double2 inv = make_double2(pv.x / den, -pv.y / den);
-    for (int i = tid; i < n; i += blockDim.x) fcol[i] = P[(i == p ? c : i) * B + j];
-    double2 keep = make_double2(0.0, 0.0);
+    const double2 inv = s_inv;
+    // row j takes what row p holds and the other way round (columns j.. are all that is read again)
+    for (int i = j + 1 + tid; i < nr; i += blockDim.x) fcol[i] = cmul(P[(i == p ? j : i) * B + j], inv);
+    double2 rp = make_double2(0.0, 0.0), rj = rp;
     if (tid < B) {
-      keep = P[c * B + tid];
-      rowc[tid] = (tid == j) ? inv : cmul(P[p * B + tid], inv);
+      rp = P[p * B + tid];
+      rj = P[j * B + tid];
     }
     __syncthreads();
-    if (tid < B && p != c) P[p * B + tid] = keep;
+    if (tid < B && p != j) {
+      P[j * B + tid] = rp;
+      P[p * B + tid] = rj;
+    }
     __syncthreads();
-    for (int e = tid; e < n * B; e += blockDim.x) {
-      const int i = e / B, jj = e % B;
-      if (jj >= kb) continue;
-      if (i == c) {
-        P[e] = rowc[jj];
-      } else {
-        const double2 f = fcol[i], r = rowc[jj];
-        double2 v = jj == j ? make_double2(0.0, 0.0) : P[e];
-        v.x = fma(-f.x, r.x, v.x);
-        v.x = fma(f.y, r.y, v.x);
-        v.y = fma(-f.x, r.y, v.y);
-        v.y = fma(-f.y, r.x, v.y);
-        P[e] = v;
-      }
+    const int w = kb - j - 1;              // columns j + 1.. of the rows below j
+    for (int e = tid; e < w * (nr - j - 1); e += blockDim.x) {
+      const int i = j + 1 + e / w, jj = j + 1 + e % w;
+      const double2 f = fcol[i], r = P[j * B + jj];
+      double2 v = P[i * B + jj];
+      v.x = fma(-f.x, r.x, v.x);
+      v.x = fma(f.y, r.y, v.x);
+      v.y = fma(-f.x, r.y, v.y);
+      v.y = fma(-f.y, r.x, v.y);
+      P[i * B + jj] = v;
     }
     __syncthreads();
   }
@@ -484,10 +495,6 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
     if (tid == 0) atomicExch(status, 1);
     for (int t = tid; t < kb; t += blockDim.x) swp[k0 + t] = k0 + t;
     return;
-  }
-  for (int e = tid; e < n * B; e += blockDim.x) {
-    const int i = e / B, j = e % B;
-    if (j < kb) M[(long long)i * n + k0 + j] = P[e];
   }
   if (tid < kb) swp[k0 + tid] = s_swp[tid];
   if (tid == 0) {   // the swaps as one move: row s_row[t] takes what row s_src[t] held
@@ -510,9 +517,60 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
   }
   __syncthreads();
   const int cnt = s_cnt;
+  // ---- D^{-1}: Gauss-Jordan on the pivot block, whose rows are in pivot order
+  if (tid < B * B) {
+    const int a = tid / B, c = tid % B;
+    D[a][c] = a < kb && c < kb ? M[(long long)s_src[a] * n + k0 + c] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  for (int j = 0; j < kb; ++j) {
+    if (tid == 0) s_inv = inverse(D[j][j]);
+    __syncthreads();
+    if (tid < B) {
+      drow[tid] = tid == j ? s_inv : cmul(D[j][tid], s_inv);
+      dcol[tid] = D[tid][j];
+    }
+    __syncthreads();
+    if (tid < B * B) {
+      const int a = tid / B, c = tid % B;
+      const double2 f = dcol[a], r = drow[c];
+      double2 v = c == j ? make_double2(0.0, 0.0) : D[a][c];
+      v.x = fma(-f.x, r.x, v.x);
+      v.x = fma(f.y, r.y, v.x);
+      v.y = fma(-f.x, r.y, v.y);
+      v.y = fma(-f.y, r.x, v.y);
+      D[a][c] = a == j ? r : v;
+    }
+    __syncthreads();
+  }
+  if (tid < B * B) dinv[tid] = D[tid / B][tid % B];
+  // ---- the panel, negated, its rows in their new order, the identity in the pivot rows
+  for (int e = tid; e < n * B; e += blockDim.x) {
+    const int i = e / B, j = e % B;
+    double2 v = make_double2(0.0, 0.0);
+    if (i >= k0 && i < k0 + kb) v.x = i - k0 == j ? 1.0 : 0.0;
+    else if (j < kb) {
+      v = M[(long long)i * n + k0 + j];
+      v = make_double2(-v.x, -v.y);
+    }
+    ap[e] = v;
+  }
+  __syncthreads();
+  for (int e = tid; e < (cnt - kb) * B; e += blockDim.x) {
+    const int t = kb + e / B, j = e % B;
+    if (j >= kb) continue;
+    const double2 v = M[(long long)s_src[t] * n + k0 + j];
+    ap[(long long)s_row[t] * B + j] = make_double2(-v.x, -v.y);
+  }
+  __syncthreads();
+  for (int e = tid; e < n * B; e += blockDim.x) {
+    const int i = e / B, j = e % B;
+    if (j < kb) M[(long long)i * n + k0 + j] = make_double2(0.0, 0.0);
+  }
+  // ---- the other columns: pivot rows out, interchanged rows moved
   for (int col = tid; col < n; col += blockDim.x) {
     if (col >= k0 && col < k0 + kb) {
-      for (int t = 0; t < B; ++t) ak[(long long)t * n + col] = make_double2(0.0, 0.0);
+      for (int t = 0; t < B; ++t) ak[(long long)t * n + col] = make_double2(col - k0 == t ? 1.0 : 0.0, 0.0);
       continue;
     }
     double2 v[2 * B];
@@ -976,7 +1034,9 @@ bool gj_panel_attr() {
   return ok;
 }
 
-size_t gj_group_bytes(int n, int B) { return oz64_bytes(n, n, B) + (size_t)n * (B * sizeof(double2) + sizeof(int)); }
+// per matrix: the panel's ak, ap and W, D^{-1} and the swaps, and the digits of the larger product
+size_t gj_side_bytes(int n, int B) { return (size_t)(3 * B * n + B * B) * sizeof(double2) + (size_t)n * sizeof(int); }
+size_t gj_group_bytes(int n, int B) { return oz64_bytes(n, n, B) + gj_side_bytes(n, B) + 256; }
 
 // Panels and tensor-core updates of groups of matrices whose digits, pivot rows and swaps fit ws
 template <int B>
@@ -989,42 +1049,71 @@ int inverse_panels(double2* base, int n, long long stride, int nbatch, int* stat
     const int m0 = (int)((long long)nbatch * g / ngroups), m1 = (int)((long long)nbatch * (g + 1) / ngroups), m = m1 - m0;
     double2* b0 = list ? base : base + (long long)m0 * stride;
     const int* l0 = list ? list + m0 : nullptr;
+    const long long pn = (long long)B * n;
     double2* ak = reinterpret_cast<double2*>(ws.mem);
-    int* swp = reinterpret_cast<int*>(ak + (size_t)m * B * n);
-    const size_t head = ((size_t)m * n * (B * sizeof(double2) + sizeof(int)) + 255) / 256 * 256;
+    double2* ap = ak + m * pn;
+    double2* W = ap + m * pn;
+    double2* dinv = W + m * pn;
+    int* swp = reinterpret_cast<int*>(dinv + (long long)m * B * B);
+    const size_t head = (m * gj_side_bytes(n, B) + 255) / 256 * 256;
     Oz64Ws rest = ws;
     rest.mem = (unsigned char*)ws.mem + head;
     rest.bytes = ws.bytes - head;
+    auto product = [&](const ZGemm& z) {
+      bool done = false;
+      const int rc = zgemm_oz64(z, st, &done);
+      return rc != GW_OK || done ? rc : fail(GW_ENOMEM, "batched_inverse: digit workspace of %zu bytes too small for n=%d",
+                                             ws.bytes, n);
+    };
     for (int k0 = 0; k0 < n; k0 += B) {
       const int kb = std::min(B, n - k0);
       prof_begin(SLOT_INVERSE_FP64, st);
-      gj_panel_kernel<B><<<m, 256, gj_panel_smem<B>(n), st>>>(b0, n, stride, l0, k0, ak, swp, status);
-      prof_end(SLOT_INVERSE_FP64, st, 8.0 * m * (double)n * kb * kb, 32.0 * m * (double)n * (2 * kb));
-      ZGemm z;                               // A += P ak
+      gj_panel_kernel<B><<<m, 256, gj_panel_smem<B>(n - k0), st>>>(b0, n, stride, l0, k0, ak, ap, dinv, swp, status);
+      prof_end(SLOT_INVERSE_FP64, st, 4.0 * m * (double)(n - k0) * kb * kb, 32.0 * m * (double)n * (4 * kb));
+      ZGemm w;                               // W = D^{-1} ak
+      w.M = kb;
+      w.N = n;
+      w.K = kb;
+      w.nbatch = m;
+      w.A = dinv;
+      w.va.rs_in = B;
+      w.va.ks_in = 1;
+      w.ba.bs_in = B * B;
+      w.B = ak;
+      w.vb.rs_in = 1;
+      w.vb.ks_in = n;
+      w.bb.bs_in = pn;
+      w.C = W;
+      w.vc.rs_in = n;
+      w.vc.ks_in = 1;
+      w.bc.bs_in = pn;
+      w.slot = SLOT_INVERSE_FP64;
+      w.ws = &rest;
+      int rc = product(w);
+      if (rc != GW_OK) return rc;
+      ZGemm z;                               // A += ap W
       z.M = n;
       z.N = n;
       z.K = kb;
       z.nbatch = m;
-      z.A = b0 + k0;
-      z.va.rs_in = n;
+      z.A = ap;
+      z.va.rs_in = B;
       z.va.ks_in = 1;
-      z.ba.list = l0;
-      z.ba.bs_in = stride;
-      z.B = ak;
+      z.ba.bs_in = pn;
+      z.B = W;
       z.vb.rs_in = 1;
       z.vb.ks_in = n;
-      z.bb.bs_in = (long long)B * n;
+      z.bb.bs_in = pn;
       z.C = b0;
       z.vc.rs_in = n;
       z.vc.ks_in = 1;
-      z.bc = z.ba;
+      z.bc.list = l0;
+      z.bc.bs_in = stride;
       z.accumulate = 1;
       z.slot = SLOT_INVERSE_FP64;
       z.ws = &rest;
-      bool done = false;
-      const int rc = zgemm_oz64(z, st, &done);
+      rc = product(z);
       if (rc != GW_OK) return rc;
-      if (!done) return fail(GW_ENOMEM, "batched_inverse: digit workspace of %zu bytes too small for n=%d", ws.bytes, n);
     }
     const int rows = std::max(1, std::min((n + kPermRows - 1) / kPermRows, (1216 + m - 1) / m));
     prof_begin(SLOT_INVERSE_FP64, st);
