@@ -119,13 +119,13 @@ size_t oz64_counter_bytes();
 // base + b * stride). list (optional, device): the matrix indices to process, nbatch of them.
 // From kGjPanelMinN on, with a digit workspace of at least one matrix's digits, pivot rows and swaps,
 // the rank-B updates of the panels run on the tensor cores to FP64 accuracy; below it the whole
-// inversion is one block per matrix on the FP64 pipe; above kGjPanelMaxN8 (or without a workspace)
+// inversion runs in shared memory on the FP64 pipe; above kGjPanelMaxN8 (or without a workspace)
 // it goes column by column. The route follows n and the workspace's size, never the batch.
 int batched_inverse_fp64(double2* base, int n, long long stride, int nbatch, int* status_dev,
                          void* stream, const int* list = nullptr, const Oz64Ws* ws = nullptr);
 // panels of 16 columns up to kGjPanelMaxN16, of 8 up to kGjPanelMaxN8 (a panel and its pivot column in
 // shared memory: n (B + 1) 16 bytes)
-constexpr int kGjPanelMinN = 64, kGjPanelMaxN16 = 800, kGjPanelMaxN8 = 1536;
+constexpr int kGjPanelMinN = 80, kGjPanelMaxN16 = 800, kGjPanelMaxN8 = 1536;
 
 // Aux Dyson pieces: M <- I - M; and after inversion M <- M - I.
 int add_identity_fp64(double2* base, int n, long long stride, int nbatch, double scale_m,

@@ -214,177 +214,119 @@ __global__ void __launch_bounds__(256) gj_inverse_kernel(double2* base, int n, l
   }
 }
 
-// Blocked form of the same inversion (same pivots, same result up to rounding order), one block per
-// matrix, for small n (below kGjPanelMinN). Columns are taken in panels of B: the panel (n x B) is
-// eliminated in shared memory with partial pivoting (explicit row swaps), written back, the
-// panel's row swaps are applied to the other columns, and those columns receive the panel's
-// effect as one rank-B update,
-//   A[i][c] <- (i in the panel's pivot rows ? 0 : A[i][c]) + sum_t P[i][t] A_old[k0 + t][c],
-// so the matrix is read and written once per panel instead of once per column. The column
-// swaps that undo the row interchanges are applied at the end through one permutation.
-template <int B>
-size_t gj_blocked_smem(int n) {
-  return (size_t)n * (2 * B * sizeof(double2) + sizeof(double2) + 2 * sizeof(int));
-}
-
-// One matrix per block: matrix blockIdx.x of base (through list when given).
-template <int B>
-__global__ void __launch_bounds__(256) gj_inverse_blocked_kernel(double2* base, int n, long long stride,
-                                                                 const int* list, int* status) {
+// The same inversion for small n (below kGjPanelMinN), the matrix in shared memory, W warps per matrix:
+// one where many matrices share an SM (no block-wide step: the FP64 pipe finds work in the other
+// warps), eight where a matrix has an SM nearly to itself or fills most of its shared memory. The
+// arithmetic of an element does not depend on W. Bound: the FP64 pipe (n^3 complex multiply-adds a
+// matrix), or the chain of a column for a few matrices; lanes run along the elements of the whole
+// matrix, so that no width is padded. 2700 matrices of 26 x 26: 0.60 ms (2.3 with one 256-thread block
+// per matrix and 16-column panels); 17 of 32 x 32: 104 us (213); 2720 of
+// 63 x 63: 5.2 ms (11.3). From 80 on the panels on the tensor cores are as fast (204 of 80 x 80: 2.0 ms, here
+// 0.6 ms at 63) and this kernel has one block an SM. magic: 2^32 / n rounded up, for e / n
+// by multiply-high.
+constexpr int kGjSmallThreads = 256;
+template <int W>
+__global__ void __launch_bounds__(kGjSmallThreads) gj_inverse_small_kernel(double2* base, int n, long long stride,
+                                                                           int nbatch, const int* list, int* status,
+                                                                           unsigned int magic) {
   extern __shared__ double2 sm[];
-  __shared__ double red_v[8];
-  __shared__ int red_i[8];
-  __shared__ int s_p, s_bad;
-  __shared__ double2 rowc[B];
-  double2* M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
-  double2* P = sm;                         // [n][B]  panel
-  double2* AK = P + (size_t)n * B;         // [B][n]  pivot rows at the panel start; staging at the end
-  double2* fcol = AK + (size_t)n * B;      // [n]     pivot column of one step
-  int* swp = reinterpret_cast<int*>(fcol + n);   // [n] row swapped with row c at step c
-  int* pi = swp + n;                       // [n]     final column permutation
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_bad = 0;
-  __syncthreads();
-
-  for (int k0 = 0; k0 < n; k0 += B) {
-    const int kb = min(B, n - k0);
-    for (int e = tid; e < n * B; e += blockDim.x) {
-      const int i = e / B, j = e % B;
-      P[e] = j < kb ? M[(long long)i * n + k0 + j] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    // ---- elimination of the panel, column by column
-    for (int j = 0; j < kb; ++j) {
-      const int c = k0 + j;
+  constexpr int kPer = 32 * W, kOwn = 64 / kPer > 1 ? 64 / kPer : 1;   // threads a matrix; rows (columns) a thread
+  const int tid = threadIdx.x % kPer, slot = threadIdx.x / kPer, lane = threadIdx.x & 31, nn = n * n;
+  const int m = blockIdx.x * (kGjSmallThreads / kPer) + slot;
+  if (m >= nbatch) return;                         // W = 8: one matrix a block, so whole blocks return
+  auto sync = [] {
+    if (W == 1) __syncwarp();
+    else __syncthreads();
+  };
+  double2* A = sm + (size_t)slot * (nn + 2 * n + 2);   // [n][n]
+  double2* f = A + nn;                             // [n]  pivot column of one step
+  int* piv = reinterpret_cast<int*>(f + n);        // [n]  row swapped with row j at step j
+  int* pi = piv + n;                               // [n]  final column permutation
+  double2* s_inv = f + 2 * n;
+  int* s_p = reinterpret_cast<int*>(s_inv + 1);    // -1: no pivot
+  double2* M = base + (long long)(list ? list[m] : m) * stride;
+  for (int e = tid; e < nn; e += kPer) A[e] = M[e];
+  sync();
+  for (int j = 0; j < n; ++j) {
+    if (tid < 32) {                                // one warp searches and divides
       double best = -1.0;
-      int bi = c;
-      for (int i = c + tid; i < n; i += blockDim.x) {
-        const double2 v = P[i * B + j];
+      int p = j;
+      for (int i = j + lane; i < n; i += 32) {
+        const double2 v = A[i * n + j];
         const double a = v.x * v.x + v.y * v.y;
-        if (a > best) { best = a; bi = i; }
+        if (a > best) { best = a; p = i; }
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_down_sync(0xffffffffu, best, o);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, p, o);
+        if (ob > best || (ob == best && oi < p)) { best = ob; p = oi; }
       }
-      if (lane == 0) { red_v[warp] = best; red_i[warp] = bi; }
-      __syncthreads();
-      if (tid == 0) {
-        double bb = red_v[0];
-        int ii = red_i[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-          if (red_v[w] > bb || (red_v[w] == bb && red_i[w] < ii)) { bb = red_v[w]; ii = red_i[w]; }
-        s_p = ii;
-        swp[c] = ii;
-        if (!(bb > 0.0)) s_bad = 1;
-      }
-      __syncthreads();
-      if (s_bad) break;
-      const int p = s_p;
-      if (p != c && tid < B) {
-        const double2 t = P[c * B + tid];
-        P[c * B + tid] = P[p * B + tid];
-        P[p * B + tid] = t;
-      }
-      __syncthreads();
-      const double2 pv = P[c * B + j];
+      const double2 pv = A[p * n + j];
       const double den = pv.x * pv.x + pv.y * pv.y;
       const double2 inv = make_double2(pv.x / den, -pv.y / den);
-      for (int i = tid; i < n; i += blockDim.x) fcol[i] = P[i * B + j];
-      if (tid < B) rowc[tid] = (tid == j) ? inv : cmul(P[c * B + tid], inv);
-      __syncthreads();
-      for (int e = tid; e < n * B; e += blockDim.x) {
-        const int i = e / B, jj = e % B;
-        if (jj >= kb) continue;
-        if (i == c) {
-          P[e] = rowc[jj];
-        } else {
-          const double2 f = fcol[i];
-          if (jj == j) {
-            const double2 t = cmul(f, inv);
-            P[e] = make_double2(-t.x, -t.y);
-          } else {
-            const double2 t = cmul(f, rowc[jj]);
-            P[e] = make_double2(P[e].x - t.x, P[e].y - t.y);
-          }
-        }
-      }
-      __syncthreads();
-    }
-    if (s_bad) break;
-    // ---- panel back; its row swaps on the other columns (each thread keeps its columns)
-    for (int e = tid; e < n * B; e += blockDim.x) {
-      const int i = e / B, j = e % B;
-      if (j < kb) M[(long long)i * n + k0 + j] = P[e];
-    }
-    for (int j = 0; j < kb; ++j) {
-      const int c = k0 + j, p = swp[c];
-      if (p == c) continue;
-      for (int col = tid; col < n; col += blockDim.x) {
-        if (col >= k0 && col < k0 + kb) continue;
-        const double2 t = M[(long long)c * n + col];
-        M[(long long)c * n + col] = M[(long long)p * n + col];
-        M[(long long)p * n + col] = t;
+      if (lane == 0) {
+        *s_inv = inv;
+        *s_p = best > 0.0 ? p : -1;
+        piv[j] = p;
       }
     }
-    __syncthreads();
-    for (int e = tid; e < B * n; e += blockDim.x) {
-      const int t = e / n, col = e % n;
-      AK[e] = t < kb ? M[(long long)(k0 + t) * n + col] : make_double2(0.0, 0.0);
+    sync();
+    const int p = *s_p;
+    const double2 inv = *s_inv;
+    if (p < 0) {                                   // the same on every thread of the matrix
+      if (tid == 0) atomicExch(status, 1);
+      return;
     }
-    __syncthreads();
-    // ---- rank-kb update of the other columns: one warp per row, lanes along the columns
-    for (int i = warp; i < n; i += (int)(blockDim.x >> 5)) {
-      const bool pivot_row = i >= k0 && i < k0 + kb;
-      double2 pr[B];
+    double2 a[kOwn], b[kOwn], g[kOwn];             // rows p and j change places, row j scaled; the column of j
 #pragma unroll
-      for (int t = 0; t < B; ++t) pr[t] = P[i * B + t];
-      for (int col = lane; col < n; col += 32) {
-        if (col >= k0 && col < k0 + kb) continue;
-        double2 v = pivot_row ? make_double2(0.0, 0.0) : M[(long long)i * n + col];
-#pragma unroll
-        for (int t = 0; t < B; ++t) {
-          const double2 a = AK[t * n + col];
-          v.x = fma(pr[t].x, a.x, v.x);
-          v.x = fma(-pr[t].y, a.y, v.x);
-          v.y = fma(pr[t].x, a.y, v.y);
-          v.y = fma(pr[t].y, a.x, v.y);
-        }
-        M[(long long)i * n + col] = v;
-      }
+    for (int u = 0; u < kOwn; ++u) {
+      const int c = tid + u * kPer;
+      if (c >= n) continue;
+      a[u] = A[p * n + c];
+      b[u] = A[j * n + c];
+      g[u] = A[(c == p ? j : c) * n + j];
     }
-    __syncthreads();
+    sync();
+#pragma unroll
+    for (int u = 0; u < kOwn; ++u) {
+      const int c = tid + u * kPer;
+      if (c >= n) continue;
+      if (p != j) A[p * n + c] = b[u];
+      A[j * n + c] = c == j ? inv : cmul(a[u], inv);
+      f[c] = g[u];
+    }
+    sync();
+#pragma unroll 4
+    for (int e = tid; e < nn; e += kPer) {
+      const int i = (int)__umulhi((unsigned)e, magic), c = e - i * n;
+      if (i == j) continue;
+      const double2 x = f[i], r = A[j * n + c];
+      double2 v = c == j ? make_double2(0.0, 0.0) : A[e];
+      v.x = fma(-x.x, r.x, v.x);
+      v.x = fma(x.y, r.y, v.x);
+      v.y = fma(-x.x, r.y, v.y);
+      v.y = fma(-x.y, r.x, v.y);
+      A[e] = v;
+    }
+    sync();
   }
-  if (s_bad) {
-    if (tid == 0) atomicExch(status, 1);
-    return;
-  }
-  // ---- undo the row interchanges as column swaps in reverse order, composed into one permutation
+  // the row interchanges undone as column swaps in reverse order, composed into one permutation
   if (tid == 0) {
     for (int i = 0; i < n; ++i) pi[i] = i;
     for (int c = n - 1; c >= 0; --c) {
-      const int r = swp[c];
-      if (r != c) {
-        const int t = pi[c];
-        pi[c] = pi[r];
-        pi[r] = t;
-      }
+      const int r = piv[c], t = pi[c];
+      pi[c] = pi[r];
+      pi[r] = t;
     }
   }
-  __syncthreads();
-  for (int r0 = 0; r0 < n; r0 += B) {
-    const int rb = min(B, n - r0);
-    for (int e = tid; e < rb * n; e += blockDim.x) AK[e] = M[(long long)r0 * n + e];
-    __syncthreads();
-    for (int e = tid; e < rb * n; e += blockDim.x) {
-      const int t = e / n, y = e % n;
-      M[(long long)(r0 + t) * n + y] = AK[t * n + pi[y]];
-    }
-    __syncthreads();
+  sync();
+  for (int e = tid; e < nn; e += kPer) {
+    const int i = (int)__umulhi((unsigned)e, magic), c = e - i * n;
+    M[e] = A[i * n + pi[c]];
   }
 }
+inline size_t gj_small_smem(int n) { return (size_t)(n * n + 2 * n + 2) * sizeof(double2); }   // of one matrix
 
 // The inversion for larger n, with only the pivots' search on the FP64 pipe. Per panel of B columns this
 // kernel (one block per matrix) factors rows k0.. of the panel (LU with partial pivoting, in shared
@@ -1138,11 +1080,22 @@ int batched_inverse_fp64(double2* base, int n, long long stride, int nbatch, int
   }
   const double flops = 8.0 * (double)n * n * n * nbatch, bytes = 32.0 * (double)n * n * nbatch;
   if (n < kGjPanelMinN) {
+    static const bool attr = cudaFuncSetAttribute(gj_inverse_small_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)(8 * gj_small_smem(32))) == cudaSuccess &&
+                             cudaFuncSetAttribute(gj_inverse_small_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)gj_small_smem(kGjPanelMinN)) == cudaSuccess;
+    if (!attr) return fail(GW_ECUDA, "gj_inverse_small: shared memory attribute refused");
+    const unsigned int magic = (unsigned int)((0x100000000ull + n - 1) / n);
     prof_begin(SLOT_INVERSE_FP64, st);
-    gj_inverse_blocked_kernel<16><<<nbatch, 256, gj_blocked_smem<16>(n), st>>>(base, n, stride, list, status_dev);
+    if (n <= 32 && nbatch >= 8 * 152)       // a warp per matrix where that gives every SM a block of them
+      gj_inverse_small_kernel<1><<<(nbatch + 7) / 8, kGjSmallThreads, 8 * gj_small_smem(n), st>>>(base, n, stride, nbatch,
+                                                                                                 list, status_dev, magic);
+    else
+      gj_inverse_small_kernel<8><<<nbatch, kGjSmallThreads, gj_small_smem(n), st>>>(base, n, stride, nbatch, list,
+                                                                                   status_dev, magic);
     prof_end(SLOT_INVERSE_FP64, st, flops, bytes);
     const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "gj_inverse_blocked launch: %s", cudaGetErrorString(e));
+    return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "gj_inverse_small launch: %s", cudaGetErrorString(e));
   }
   const size_t smem = 2 * (size_t)n * sizeof(double2) + (size_t)n * sizeof(int);
   if (smem > 200 * 1024) return fail(GW_EINVAL, "batched_inverse_fp64: n=%d too large", n);

@@ -1,5 +1,5 @@
-"""The inversion of the aux Dyson equation (gw_aux_dyson) at the sizes where its route changes: one block per
-matrix below 64, panels of 16 columns with tensor-core updates up to 800, of 8 above; remainders of panels
+"""The inversion of the aux Dyson equation (gw_aux_dyson) at the sizes where its route changes: in shared
+memory below 80, panels of 16 columns with tensor-core updates up to 800, of 8 above; remainders of panels
 and row tiles; matrices that need row interchanges; a singular one."""
 import numpy as np
 import pytest
@@ -24,7 +24,7 @@ def _solve(gw, m):
         ctx.destroy()
 
 
-@pytest.mark.parametrize("n", [1, 15, 63, 64, 65, 80, 127, 200, 257, 480, 801])
+@pytest.mark.parametrize("n", [1, 15, 32, 33, 79, 80, 81, 127, 200, 257, 480, 801])
 def test_aux_dyson_inverts(n):
     """Random matrices (every column needs its pivot searched), one of them with a zero diagonal, and one
     with rows over six decades; backward error of the inverse as a partially pivoted elimination gives it."""
