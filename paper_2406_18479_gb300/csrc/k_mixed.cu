@@ -342,16 +342,15 @@ struct OzShape {
   static constexpr int kBBlock = kBN * kRowBytes;      // bytes of one B group block
   static constexpr uint32_t kStageBytes = 2 * kAGroup + 3 * kBBlock;
   static constexpr uint32_t kTxBytes = 2 * kAGroup + 2 * kBBlock;   // what TMA brings per stage
-  static constexpr int kThreads = 352;                 // producer, MMA, 8 epilogue warps, negation warp
   static constexpr int kOrderCols = 2 * kBN;           // [im | re] of one order
   static constexpr int kTmemCols = 512;
   // accumulator sets in TMEM: two where they fit (tiles up to 40 columns), so that the MMAs of
   // the next chunk run while the epilogue drains the last one
   static constexpr int kBufCols = 3 * kOrderCols;
   static constexpr int kBufs = 2 * kBufCols <= kTmemCols ? 2 : 1;
-  // slice output: maxima exchanged between column halves (two tiles in flight x 4 lane quarters x
-  // 2 halves x 32 lanes)
-  static constexpr int kXmaxBytes = 2 * 4 * 2 * 32 * 4;
+  // slice output: maxima exchanged between a lane quarter's warps (two tiles in flight x 4 quarters x
+  // 2 or 4 warps x 32 lanes)
+  static constexpr int kXmaxBytes = 2 * 4 * 4 * 32 * 4;
   static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + 256 + kXmaxBytes;
   static_assert(3 * kOrderCols <= kTmemCols, "three orders must fit in TMEM");
   static_assert(kStageBytes % 1024 == 0, "stages must keep the 1024-byte swizzle alignment");
@@ -380,8 +379,16 @@ __device__ __forceinline__ void tmem_ldg(uint32_t taddr, float* v) {
   else tmem_ld4(taddr, v);
 }
 
-template <int BN_, bool SO>
-__global__ void __launch_bounds__(352, 1)
+// EW epilogue warps: 8, each a lane quarter by half the tile's columns, or 16 (one-chunk slice output
+// only), each a lane quarter by every fourth group of 4 columns. The slice output is a long FP32 chain per
+// value (normalisation, four rounded cuts, packing), which two warps a scheduler did not cover; the X and Y
+// products of P0 at the 4x4x4 solid's sizes (56-column tiles, no second accumulator set to hide it):
+// 20.8 -> 18.6 ms on four k-points; the 40-column Z product, whose epilogue runs under the next tile's MMAs,
+// stays at 14.5 ms. What bounds them now: 30k instructions a tile at half the issue rate, and the MMAs
+// (a quarter of the time) that wait for the 56-column tile's only accumulator set.
+constexpr int oz_threads(int ew) { return 96 + 32 * ew; }   // producer, MMA, epilogue, negation warp
+template <int BN_, bool SO, int EW>
+__global__ void __launch_bounds__(oz_threads(EW), 1)
     oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const OzParams p) {
   using S = OzShape<BN_>;
   constexpr int G = S::kG;
@@ -409,10 +416,10 @@ __global__ void __launch_bounds__(352, 1)
     }
     for (int b = 0; b < S::kBufs; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 8);           // one arrival per epilogue warp
+      mbar_init(&acc_empty[b], EW);          // one arrival per epilogue warp
     }
     mbar_init(drain_bar, 1);
-    mbar_init(xbar, 8);
+    mbar_init(xbar, EW);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -517,7 +524,7 @@ __global__ void __launch_bounds__(352, 1)
       while (!mbar_try(drain_bar, 0) && globaltimer() - t0 < kWaitLimitNs) {
       }
     }
-  } else if (warp == 10) {
+  } else if (warp == 2 + EW) {
     // ---------------- -Bi block of each stage: sign flip of the Bi block (same swizzle phase)
     uint32_t step = 0;
     bool ok = true;
@@ -627,9 +634,9 @@ __global__ void __launch_bounds__(352, 1)
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
         if (p.so_xhalf) {
-          // the chunk's other columns belong to the warp with the same lanes and the other half
+          // the chunk's other columns belong to the warps with the same lanes
           const uint32_t par = so_tile & 1;
-          xmax[((par * 4 + quarter) * 2 + half) * 32 + lane] = mx;
+          xmax[((par * 4 + quarter) * (EW / 4) + half) * 32 + lane] = mx;
           __syncwarp();
           int w = 1;
           if (lane == 0) {
@@ -638,8 +645,12 @@ __global__ void __launch_bounds__(352, 1)
           }
           w = __shfl_sync(0xffffffffu, w, 0);
           __syncwarp();
-          if (w) mx = max(mx, xmax[((par * 4 + quarter) * 2 + (half ^ 1)) * 32 + lane]);
-          else ok = false;
+          if (w) {
+#pragma unroll
+            for (int o = 0; o < EW / 4; ++o) mx = max(mx, xmax[((par * 4 + quarter) * (EW / 4) + o) * 32 + lane]);
+          } else {
+            ok = false;
+          }
           ++so_tile;
         }
         const int eb = (int)((mx >> 23) & 0xFF);
@@ -698,19 +709,21 @@ __global__ void __launch_bounds__(352, 1)
           // ---- slice output of a one-chunk contraction straight from TMEM: pass 1 finds the row
           //      maximum, pass 2 slices 4 columns at a time; TMEM is released after pass 2
           uint32_t mx = 0;
+          // this warp's column groups: its half of the tile, or (16 warps) every fourth group of 4
+          constexpr int GS = EW == 8 ? G : 4;
+          constexpr int kFirst = EW == 8 ? kCols : 4, kNext = EW == 8 ? GS : EW, kEnd = EW == 8 ? kCols : BN;
 #pragma unroll 1
-          for (int g = 0; g < kCols / G; ++g) {
-            const int cb = half * kCols + g * G;
-            float v[2][2][G];                         // orders 0 and 1: the maximum takes the hi word
+          for (int cb = half * kFirst; cb < (EW == 8 ? half * kFirst + kEnd : kEnd); cb += kNext) {
+            float v[2][2][GS];                        // orders 0 and 1: the maximum takes the hi word
             const uint32_t taddr = tbase + (uint32_t)cb;
 #pragma unroll
             for (int o = 0; o < 2; ++o) {
-              tmem_ldg<G>(taddr + o * S::kOrderCols, v[o][0]);
-              tmem_ldg<G>(taddr + o * S::kOrderCols + BN, v[o][1]);
+              tmem_ldg<GS>(taddr + o * S::kOrderCols, v[o][0]);
+              tmem_ldg<GS>(taddr + o * S::kOrderCols + BN, v[o][1]);
             }
             tmem_wait_ld();
 #pragma unroll
-            for (int u = 0; u < G; ++u) {
+            for (int u = 0; u < GS; ++u) {
               if (!col_ok(cb + u)) continue;
               float rh, rl, ih, il;
               two_sum(v[0][1][u], v[1][1][u], rh, rl);
@@ -721,8 +734,7 @@ __global__ void __launch_bounds__(352, 1)
           float magic[4];
           const bool zero = so_alignment(mx, magic);
 #pragma unroll 1
-          for (int g4 = 0; g4 < kCols / 4; ++g4) {
-            const int c0 = half * kCols + 4 * g4;
+          for (int c0 = half * kFirst; c0 < (EW == 8 ? half * kFirst + kEnd : kEnd); c0 += EW == 8 ? 4 : EW) {
             float v[3][2][4];
             const uint32_t taddr = tbase + (uint32_t)c0;
 #pragma unroll
@@ -748,6 +760,7 @@ __global__ void __launch_bounds__(352, 1)
           if (lane == 0) mbar_arrive(&acc_empty[buf]);
           continue;
         }
+        if constexpr (EW == 8) {                      // 16 warps: one-chunk slice output only
         if (single) {
           // ---- one-chunk contraction: TMEM -> value (an exact FP32 pair per part) -> output
 #pragma unroll 1
@@ -866,8 +879,9 @@ __global__ void __launch_bounds__(352, 1)
             }
           }
         }
+        }
       }
-      if (SO && nchunks > 1 && ok) {
+      if (EW == 8 && SO && nchunks > 1 && ok) {
         // ---- slice output of a chunked contraction: the final values wait in cw; the next
         //      group's loads are issued before the current group is sliced
         float magic[4];
@@ -1000,6 +1014,8 @@ int launch_slice(const SliceJob& j, cudaStream_t st) {
 template <int BN_>
 int launch_oz_bn(const Planes& A, const Planes& B, OzParams p, int slot, cudaStream_t st) {
   using S = OzShape<BN_>;
+  // slice output through the narrow tiles is the V.G products' (one chunk, maxima over the whole tile)
+  constexpr int kSoWarps = BN_ <= 56 ? 16 : 8;
   if (A.Kpad != B.Kpad || A.Kc != B.Kc) return fail(GW_EINVAL, "oz_gemm: operand chunking differs");
   if (A.groups != 2 || B.groups != 2) return fail(GW_EINVAL, "oz_gemm: operands need two slice groups");
   p.nsteps = A.Kpad / kStepK;
@@ -1009,6 +1025,8 @@ int launch_oz_bn(const Planes& A, const Planes& B, OzParams p, int slot, cudaStr
   if (p.so) {
     // a chunk is 4 rows (a lane group) by so_cb columns within one tile, or one column half
     const bool halves_ok = p.so_xhalf ? p.so_cb >= nstride : (S::kBN / 2) % p.so_cb == 0;
+    if (kSoWarps == 16 && (!p.so_xhalf || p.nsteps > p.steps_per_chunk))
+      return fail(GW_EINVAL, "oz_gemm: slice output of narrow tiles takes one chunk and whole-tile maxima");
     if (p.dblock || !p.so_dst || p.so_mdiv % 4 || p.so_cb % 4 || p.so_cb <= 0 || p.M % 4 || p.N % 4 ||
         nstride % 4 || !halves_ok || p.so_ksteps <= 0 || p.so_rows <= 0)
       return fail(GW_EINVAL, "oz_gemm: slice output layout not supported");
@@ -1028,17 +1046,17 @@ int launch_oz_bn(const Planes& A, const Planes& B, OzParams p, int slot, cudaStr
   GW_TRY_INTERNAL(make_map(B, S::kBN, &mb));
   // one-time setup; function-local statics initialise once even when contexts run on several threads
   static const bool attr = [] {
-    cudaFuncSetAttribute(oz_gemm_kernel<BN_, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
-    cudaFuncSetAttribute(oz_gemm_kernel<BN_, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+    cudaFuncSetAttribute(oz_gemm_kernel<BN_, false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+    cudaFuncSetAttribute(oz_gemm_kernel<BN_, true, kSoWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
     return true;
   }();
   (void)attr;
   const int grid = (int)std::min<long long>(total, num_sms());
   prof_begin(slot, st);
   if (p.so)
-    oz_gemm_kernel<BN_, true><<<grid, S::kThreads, S::kSmem, st>>>(ma, mb, p);
+    oz_gemm_kernel<BN_, true, kSoWarps><<<grid, oz_threads(kSoWarps), S::kSmem, st>>>(ma, mb, p);
   else
-    oz_gemm_kernel<BN_, false><<<grid, S::kThreads, S::kSmem, st>>>(ma, mb, p);
+    oz_gemm_kernel<BN_, false, 8><<<grid, oz_threads(8), S::kSmem, st>>>(ma, mb, p);
   // executed bf16 tensor flops: 10 slice products x 2 real MMAs of 128 x (2 BN) x 16 per k-step
   prof_end(slot, st, 2.0 * 20.0 * (double)total * kBM * (2 * S::kBN) * (double)p.nsteps * kStepK,
            (double)total * p.nsteps * S::kTxBytes);
