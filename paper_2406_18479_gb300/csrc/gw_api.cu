@@ -289,8 +289,9 @@ int polarization_fp64(gw_ctx* c, const double2* G, double2* P0t, int q0, int q1)
   const long long nao2 = c->nao2, pair = c->pair;
   for (int q = q0; q < q1; ++q) {
     const int tend = canonical_end(c, q, ntau, q0, q1);
-    for (int t0 = 0; t0 < tend; t0 += c->nt) {
-      const int nt = std::min(c->nt, tend - t0);
+    const int nb = (tend + c->nt - 1) / c->nt;      // equal batches: no short last one
+    for (int i = 0; i < nb; ++i) {
+      const int t0 = (int)((long long)tend * i / nb), nt = (int)((long long)tend * (i + 1) / nb) - t0;
       double2* Abuf = c->work;
       double2* Bbuf = c->work + (long long)c->nt * nk * pair;
       // A^Q_{db}(k,t) = sum_a V^{k,k+q}_da(Q) G^{k+q}_ab(t), stored [Q][d][b]
@@ -321,8 +322,9 @@ int self_energy_fp64(gw_ctx* c, const double2* G, const double2* Pt, double2* Si
   if (cudaMemsetAsync(Sig, 0, (size_t)nk * ntau * nao2 * sizeof(double2), c->stream) != cudaSuccess)
     return cuda_check("memset Sigma");
   for (int q = q0; q < q1; ++q) {
-    for (int t0 = 0; t0 < ntau; t0 += c->nt) {
-      const int nt = std::min(c->nt, ntau - t0);
+    const int nb = (ntau + c->nt - 1) / c->nt;
+    for (int i = 0; i < nb; ++i) {
+      const int t0 = (int)((long long)ntau * i / nb), nt = (int)((long long)ntau * (i + 1) / nb) - t0;
       double2* Rbuf = c->work;
       double2* Zbuf = c->work + (long long)c->nt * nk * pair;
       {  // R^Q_{bj}(k,t) = sum_Q' P~^q_QQ'(t) V^{k-q,k}_bj(Q')
@@ -590,8 +592,10 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
       // again. More digits than fit are made in pieces, with the same result.
       const double dig_t = (double)oz64_bytes(c->naux, c->naux, nk * (int)c->nao2);
       const double budget = std::max(c->nt * per_t, 67108864.0);
-      if (cfg->tau_chunk <= 0) c->nt = std::max(1, std::min(c->nt, (int)(budget / (per_t + dig_t))));
-      c->oz_bytes = (size_t)std::min(c->nt * dig_t, cfg->tau_chunk > 0 ? budget : std::max(budget - c->nt * per_t, 0.0));
+      // (a sixteenth is left for the partial sums of products that split K)
+      if (cfg->tau_chunk <= 0) c->nt = std::max(1, std::min(c->nt, (int)(budget * 15 / 16 / (per_t + dig_t))));
+      const double most = std::max(dig_t, (double)nk * oz64_bytes(c->nao, c->nao, c->naux * c->nao));   // P0's or Sigma's
+      c->oz_bytes = (size_t)std::min(c->nt * most + budget / 16, cfg->tau_chunk > 0 ? budget : std::max(budget - c->nt * per_t, 0.0));
       if ((rc = dev_alloc(c, &c->work, (size_t)c->nt * 2 * nk * c->pair)) != GW_OK) break;
       if (cfg->v_packed && (rc = dev_alloc(c, &c->Vfull, (size_t)nk * nk * c->pair)) != GW_OK) break;
     }
@@ -944,23 +948,32 @@ int gw_density(gw_ctx* ctx, const gw_c128* G_dev, gw_c128* gamma_dev) {
 namespace {
 
 // The exchange term as two digit products over all (k, k') of a group of k: X = V^{kk'} gamma^{k'} and
-// its contraction with V^{k'k} over (Q, b), the sums over k' reduced in order. The FP64 pipe takes
-// 16 nao^3 flops per (k, k', Q): 36.2 ms on the 3x3x3 solid at nao = 26 (41 GFLOP); this way 12.1, half
-// of it packing. Below 2^23 multiply-adds in all, the former's single launch is the faster one. X and,
-// with a packed V, the unpacked blocks lie in P~ and P0 (not in use outside an evaluation), which hold
-// them for at least one k where ntau naux >= 2 nao^2; the same rule for a full V keeps the two
-// layouts' results alike.
-bool exchange_on_tensor(const gw_ctx* c) {
-  return c->oz_x.mem && c->nao >= 8 && (long long)c->ntau * c->naux >= 2 * c->nao2 &&
-         2.0 * c->nk * c->nk * (double)c->pair * c->nao >= 8388608.0;
+// its contraction with V^{k'k} over (Q, b), the partial sums over k' (and pieces of Q) reduced in order.
+// The FP64 pipe takes 16 nao^3 flops per (k, k', Q): 36.2 ms on the 3x3x3 solid at nao = 26 (41 GFLOP);
+// this way 12.1, half of it packing. Below 2^26 multiply-adds in all (half a millisecond on the FP64
+// pipe) the six launches and their long packed rows cost more than they save. X and, with a packed
+// V, the unpacked blocks lie in P~ and P0 (not in use outside an evaluation), which hold them for at
+// least one k where ntau naux >= 2 nao^2; the same rule for a full V keeps the two layouts' results
+// alike. The pieces of Q: the least number, a divisor of naux, for which the digits of eight (k, k') (or
+// all) fit the workspace; 0: none, the former path.
+int exchange_pieces(const gw_ctx* c) {
+  if (!c->oz_x.mem || c->nao < 8 || (long long)c->ntau * c->naux < 2 * c->nao2 ||
+      2.0 * c->nk * c->nk * (double)c->pair * c->nao < 67108864.0)
+    return 0;
+  const size_t pairs = (size_t)std::min(8, c->nk * c->nk);
+  for (int d = 1; d <= std::min(16, c->naux); ++d)
+    if (c->naux % d == 0 && pairs * oz64_bytes(c->nao, c->nao, c->naux / d * c->nao) <= c->oz_x.bytes) return d;
+  return 0;
 }
 
-int exchange_tensor(gw_ctx* c, bool packed, double2* S) {
+int exchange_tensor(gw_ctx* c, bool packed, int pieces, double2* S) {
   const int nk = c->nk, nao = c->nao, naux = c->naux;
   const long long nao2 = c->nao2, pair = c->pair;
   // k per group: what the P arrays hold, and enough (k, k') tiles for two waves
   const int room = (int)std::min<long long>((long long)c->ntau * c->naux / (2 * nao2), nk);
-  const int group = std::max(1, std::min(std::min(room, naux), (304 + nk - 1) / nk));
+  const int parts = nao <= kExchangeMaxNao ? nk * exchange_chunks(nk, naux) : naux;   // xinf holds so many per k'
+  const int group = std::max(1, std::min(std::min(room, parts / pieces), (304 + nk - 1) / nk));
+  const int nq = naux / pieces;
   for (int k0 = 0; k0 < nk; k0 += group) {
     const int m = std::min(group, nk - k0);
     const double2* v1 = c->V + (long long)k0 * nk * pair;       // V^{kk'}: [k][k']
@@ -985,15 +998,19 @@ int exchange_tensor(gw_ctx* c, bool packed, double2* S) {
     a.C = X; a.vc.rs_in = 1; a.vc.ks_in = (long long)naux * nao; a.bc.bs_in = pair; a.bc.bs_out = (long long)nk * pair;
     a.slot = SLOT_STATIC_FP64; a.ws = &c->oz_x;
     GW_TRY(zgemm_fp64(a, c->stream));
-    ZGemm b;                                                    // k = (Q, b)
-    b.M = nao; b.N = nao; b.K = naux * nao; b.nbatch = m * nk; b.bin = nk;
-    b.A = X; b.va.rs_in = 1; b.va.kin = nao; b.va.ks_in = (long long)naux * nao; b.va.ks_out = nao;
-    b.ba.bs_in = pair; b.ba.bs_out = (long long)nk * pair;
-    b.B = v2; b.vb.rs_in = 1; b.vb.kin = nao; b.vb.ks_in = nao; b.vb.ks_out = nao2; b.bb.bs_in = v2p; b.bb.bs_out = v2k;
-    b.C = c->xinf; b.vc.rs_in = nao; b.vc.ks_in = 1; b.bc.bs_in = nao2; b.bc.bs_out = nk * nao2;
-    b.slot = SLOT_STATIC_FP64; b.ws = &c->oz_x;
-    GW_TRY(zgemm_fp64(b, c->stream));
-    GW_TRY(reduce_partials_fp64(c->xinf, S + k0 * nao2, m, (int)nao2, nk, -1.0 / nk, c->stream));
+    for (int q = 0; q < pieces; ++q) {                          // part [k][q][k']
+      ZGemm b;                                                  // k = (Q, b)
+      b.M = nao; b.N = nao; b.K = nq * nao; b.nbatch = m * nk; b.bin = nk;
+      b.A = X + (long long)q * nq * nao; b.va.rs_in = 1; b.va.kin = nao; b.va.ks_in = (long long)naux * nao; b.va.ks_out = nao;
+      b.ba.bs_in = pair; b.ba.bs_out = (long long)nk * pair;
+      b.B = v2 + (long long)q * nq * nao2; b.vb.rs_in = 1; b.vb.kin = nao; b.vb.ks_in = nao; b.vb.ks_out = nao2;
+      b.bb.bs_in = v2p; b.bb.bs_out = v2k;
+      b.C = c->xinf + (long long)q * nk * nao2; b.vc.rs_in = nao; b.vc.ks_in = 1;
+      b.bc.bs_in = nao2; b.bc.bs_out = (long long)pieces * nk * nao2;
+      b.slot = SLOT_STATIC_FP64; b.ws = &c->oz_x;
+      GW_TRY(zgemm_fp64(b, c->stream));
+    }
+    GW_TRY(reduce_partials_fp64(c->xinf, S + k0 * nao2, m, (int)nao2, nk * pieces, -1.0 / nk, c->stream));
   }
   return GW_OK;
 }
@@ -1016,7 +1033,7 @@ int gw_sigma_inf(gw_ctx* ctx, const gw_c128* G_dev, gw_c128* SigInf_dev) {
   const int packed = ctx->V ? 0 : 1;
   GW_TRY(hartree_fp64(Vs, ctx->gamma, ctx->rho, S, nk, naux, nao, ctx->cfg.spin_factor / nk, packed, ctx->stream));
   // exchange: -(1 / N_k) sum_{k'} sum_{Q b} X^{k'}_{Q i b} V^{k'k}_bj(Q), X^{k'}_{Q i b} = sum_a V^{kk'}_ia(Q) gamma^{k'}_ab
-  if (exchange_on_tensor(ctx)) return exchange_tensor(ctx, packed != 0, S);
+  if (const int pieces = exchange_pieces(ctx)) return exchange_tensor(ctx, packed != 0, pieces, S);
   if (nao <= kExchangeMaxNao)
     return exchange_fp64(Vs, ctx->gamma, ctx->xinf, S, nk, naux, nao, -1.0 / nk, packed, ctx->stream);
   // per k: X^{k'} = V^{kk'} gamma^{k'} for every k' (one batched product), then S^k -= X^{k'} V^{k'k}

@@ -55,7 +55,8 @@ constexpr int kScaleMax = 480;      // |E| beyond this takes the plain FP64 loop
 constexpr int kEpiWarps = 16;
 constexpr int kSegSteps = 8;        // least k-steps of a packing segment
 constexpr int kMaxSegs = 32;
-constexpr int kSplitUnits = 152;    // tiles x splits of a split-K launch, at most (one wave)
+constexpr int kSplitTiles = 608;    // tiles of a split-K launch, at most (four waves)
+constexpr int kMaxSplit = 16;
 
 // x / d for x < 2^31: multiply-high (see FastDiv in k_mixed.cu)
 struct Div {
@@ -695,7 +696,7 @@ inline long long up(long long x, long long m) { return (x + m - 1) / m * m; }
 
 }  // namespace
 
-size_t oz64_counter_bytes() { return (size_t)kSplitUnits * kEpiWarps * sizeof(unsigned int); }
+size_t oz64_counter_bytes() { return (size_t)kSplitTiles * kEpiWarps * sizeof(unsigned int); }
 
 size_t oz64_bytes(long long p_rows, long long q_rows, int K) {
   const long long nks = (K + 7) / 8;
@@ -783,24 +784,34 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
           j.q.dst = m + pn * j.nks * 512;
           j.p.scale = reinterpret_cast<double*>(j.q.dst + qn * j.nks * 256);
           j.q.scale = j.p.scale + pn;
-          // few tiles, long K: share a tile's chunks among CTAs so that every SM has work (the partial
-          // sums take what the digits leave of the workspace)
-          const long long tiles = (long long)j.p.tiles * j.q.tiles * j.no * j.ni;
-          const int nchunks = (j.nks + kChunkSteps - 1) / kChunkSteps;
-          j.ksplit = 1;
-          // long rows are packed in segments where the row tiles alone leave SMs idle (4 blocks an SM)
+          // long rows are packed in segments where the row tiles alone leave SMs idle (8 blocks an SM)
           const long long blocks = (long long)j.p.no * j.p.ni * j.p.tiles + (long long)j.q.no * j.q.ni * j.q.tiles;
           const int segs = (int)std::min<long long>(std::min(j.nks / kSegSteps, kMaxSegs), (8LL * sm_count() + blocks - 1) / blocks);
           j.seg_steps = (j.nks + std::max(segs, 1) - 1) / std::max(segs, 1);
           j.segs = (j.nks + j.seg_steps - 1) / j.seg_steps;
           j.p.pmax = reinterpret_cast<unsigned long long*>(j.q.scale + qn);
           j.q.pmax = j.p.pmax + (j.segs > 1 ? pn * j.segs : 0);
+          // Tiles that leave the last wave short of work (or never fill one) share their chunks of K among
+          // CTAs: the split with the least waves times chunks, a chunk's time for each partial sum that is
+          // written and read again. The partial sums take what the digits leave of the workspace. 80 tiles
+          // of 85 chunks on 152 SMs (P0 of a 2x2x2 solid): 12.5 -> 7.7 ms (with
+          // equal tau batches).
+          const long long tiles = (long long)j.p.tiles * j.q.tiles * j.no * j.ni;
+          const int nchunks = (j.nks + kChunkSteps - 1) / kChunkSteps;
+          j.ksplit = 1;
           j.part_hi = reinterpret_cast<long long*>(j.q.pmax + (j.segs > 1 ? qn * j.segs : 0));
           const long long room = (m + g.ws->bytes - reinterpret_cast<unsigned char*>(j.part_hi)) / (128 * nt * 12);
-          if (g.ws->counters && nchunks > 1 && 2 * tiles <= std::min<long long>(kSplitUnits, room)) {
-            const int ks = (int)std::min<long long>(std::min<long long>(kSplitUnits, room) / tiles, nchunks);
-            j.split_chunks = (nchunks + ks - 1) / ks;
-            j.ksplit = (nchunks + j.split_chunks - 1) / j.split_chunks;
+          if (g.ws->counters && nchunks > 1 && tiles <= kSplitTiles) {
+            long long best = (tiles + sm_count() - 1) / sm_count() * nchunks;
+            for (int ks = 2; ks <= std::min(nchunks, kMaxSplit) && tiles * ks <= room; ++ks) {
+              const int per = (nchunks + ks - 1) / ks, used = (nchunks + per - 1) / per;
+              const long long cost = (tiles * used + sm_count() - 1) / sm_count() * (per + 1);
+              if (cost < best) {
+                best = cost;
+                j.split_chunks = per;
+                j.ksplit = used;
+              }
+            }
             j.counter = reinterpret_cast<unsigned int*>(g.ws->counters);
             j.part_lo = reinterpret_cast<uint32_t*>(j.part_hi + tiles * j.ksplit * 128 * nt);
           }

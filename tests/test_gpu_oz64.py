@@ -101,9 +101,11 @@ def test_fp64_contractions_match_oracle(nk3, nao, naux, ntau, chunk):
     ctx.destroy()
 
 
-@pytest.mark.parametrize("nk3,nao,naux,ntau", [((2, 1, 1), 26, 104, 24), ((3, 1, 1), 27, 70, 30), ((1, 1, 1), 54, 60, 100)])
+@pytest.mark.parametrize("nk3,nao,naux,ntau", [((2, 1, 1), 26, 104, 24), ((3, 1, 1), 27, 70, 30), ((1, 1, 1), 54, 60, 100),
+                                               ((3, 1, 1), 40, 80, 40), ((1, 1, 1), 70, 100, 99)])
 def test_static_exchange_matches_oracle(nk3, nao, naux, ntau):
-    """Sigma^inf with its exchange on the tensor cores (both sides of the former kernel's nao limit), full and
+    """Sigma^inf with its exchange on the tensor cores (from 2^26 multiply-adds on: the last two sizes, both
+    sides of the fused kernel's nao limit, the last one in pieces of Q) or not, full and
     packed V, against the oracle; the two layouts agree bit for bit."""
     gw = _gw()
     from oracle import gw as O
