@@ -70,7 +70,8 @@ typedef enum {
 } gw_status;
 
 typedef enum {
-  GW_FP64 = 0,          /* every contraction in FP64 */
+  GW_FP64 = 0,          /* every contraction to FP64 accuracy (on the tensor cores through exact integer
+                           digits where that pays, with a smaller error than a running FP64 sum) */
   GW_MIXED_BF16X4 = 1,  /* V.G.V contractions on tcgen05 tensor cores: each operand row is cut,
                            per chunk of at most 256 k, into four bf16 slices on one power-of-two
                            alignment; slice products of order 0 and 1 sum exactly in their own
@@ -359,7 +360,7 @@ int gw_synchronize(gw_ctx* ctx);
  *       V^{k k1}_ip(Q) V^{k3 k2}_mk(Q) G^{k1}_pq(tau) G^{k2}_kl(tau) G^{k3}_nm(beta - tau),
  * k3 = k1 + k2 - k, s = spin_factor. The direct (first) term is the GW self-energy contraction
  * with P0 in place of P~ (gw_polarization then gw_self_energy, in the context's precision); the
- * exchange term runs in FP64, contracted over Q and Q' first (2 nao^4 naux + nao^5 complex MACs
+ * exchange term's V.G products run in FP64, contracted over Q and Q' first (2 nao^4 naux + nao^5 complex MACs
  * per (k, k1, k2, tau)), through a device workspace of at most about 2 GiB (fewer tau nodes per
  * batch with cfg.tau_chunk), allocated on first use. Writes Sig_dev [nk][ntau][nao][nao];
  * uses the context's P0 buffer. gw_gf2_exchange writes the exchange term alone,
