@@ -650,7 +650,11 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
       c->oz_x = c->oz_w;       // P(i Omega) for the exchange: its long rows fill the GPU in large pieces only
       const size_t nw_bytes = (size_t)nk * c->nwb * c->naux2 * sizeof(double2);
       if (nw_bytes > c->oz_x.bytes) c->oz_x.bytes = std::min(nw_bytes, kOz64InvBytes);
+      // the FP64 contractions: P(i Omega) too where it is the larger (large solids, whose intermediates of one
+      // tau node leave no room: q = 0 of the 4x4x4 solid in FP64 28.9 -> 3.0 s, 57.7 on the FP64 pipe), else memory of
+      // their own
       c->oz = c->oz_w;
+      if (cfg->precision == GW_FP64 && nw_bytes > c->oz.bytes) c->oz.bytes = std::min<size_t>(nw_bytes, 4ull << 30);
       if (c->oz_bytes > c->oz.bytes) {
         if ((rc = dev_alloc(c, &c->oz_mem, c->oz_bytes)) != GW_OK) break;
         c->oz.mem = c->oz_mem;
