@@ -17,12 +17,12 @@
 // value is rounded to FP64. The result does not depend on tiling or batching, and its error is
 // below that of a running FP64 sum.
 //
-// Bound: the tensor cores and the L2 reads of the digit tiles (48 KB per k-step of a 128 x 64 tile),
-// about 23 TFLOP/s of complex products at long K (R of a molecule, nao = 45) and 13 where the output is
-// as large as the work (transforms), against 0.7..1.1 on the FP64 pipe. P0 of a 2x2x2 solid (nao = 26,
-// naux = 104, 80 nodes): 313 -> 31.3 ms; Sigma of a molecule (nao = 45): 76.9 -> 5.8 ms; the two
-// transforms of a 3x3x3 solid (naux = 200, 100 nodes): 198 -> 21 ms. Error against 64-bit references
-// on these: 2e-16 and 4e-16 (FP64 pipe: 3e-15 and 6e-15).
+// Bound: the L2 reads of the digit tiles at long K (48 KB per k-step of a 128 x 64 tile, 5.5 TB/s), the
+// epilogue's three FP64 operations an output at short K. 27 TFLOP/s of complex products at long K (R of a
+// molecule, nao = 45) and 16 where the output is as large as the work (transforms), against 0.7..1.1 on
+// the FP64 pipe. P0 of a 2x2x2 solid (nao = 26, naux = 104, 80 nodes): 313 -> 21.3 ms; Sigma of a molecule
+// (nao = 45): 76.9 -> 5.1 ms; the two transforms of a 3x3x3 solid (naux = 200, 100 nodes): 198 -> 19 ms with
+// their packing. Error against 64-bit references on these: 2e-16 and 4e-16 (FP64 pipe: 3e-15 and 6e-15).
 //
 // Rows with a non-finite element, or whose scale lies outside 2^+-480 (where the scaled product
 // could over- or underflow), carry a NaN scale; outputs that meet one are computed by a plain
