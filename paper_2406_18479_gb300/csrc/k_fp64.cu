@@ -328,38 +328,40 @@ __global__ void __launch_bounds__(kGjSmallThreads) gj_inverse_small_kernel(doubl
 }
 inline size_t gj_small_smem(int n) { return (size_t)(n * n + 2 * n + 2) * sizeof(double2); }   // of one matrix
 
-// The inversion for larger n, with only the pivots' search on the FP64 pipe. Per panel of B columns this
-// kernel (one block per matrix) factors rows k0.. of the panel (LU with partial pivoting, in shared
-// memory), inverts the pivot block D, and lays the panel's step out as two products over the whole
-// matrix, which run on the tensor cores (zgemm_oz64):
-//   W = D^{-1} ak,  ak [B][n]: the pivot rows, with the identity in the panel's columns
-//   A += ap W,      ap [n][B]: the negated panel, with the identity in the pivot rows
-// after the rows the pivots interchanged have moved and the panel's columns and the pivot rows of A
-// are zero: the pivot rows become D^{-1} A_p, the panel -A D^{-1}, its pivot block D^{-1}, the rest
-// A - A_panel D^{-1} A_p. On the FP64 pipe that leaves B^2/2 complex multiply-adds per row below k0, a
-// quarter of an elimination of every row; what bounds the kernel now is the chain of a column (search,
-// one division, swap, update: 5 block-wide steps). 303 matrices of 200 x 200 take 167 us a panel (an
-// elimination of every row 242), 81 of 480 x 480 142 us (226). The whole inversion against one block per
-// matrix on the FP64 pipe: 2727 of 200 x 200 209 -> 62 ms, 81 of 480 x 480 120 -> 16.6 ms (half the SMs had
-// no matrix there; the products use all). swp[c]: the row swapped with row c at step c.
+// The inversion for larger n, with its n^3 work on the tensor cores. Per panel of B columns this kernel (one
+// block per matrix) factors rows k0.. of the panel (LU with partial pivoting, in shared memory) and lays the
+// panel's step out as one product over the whole matrix (zgemm_oz64),
+//   A += ap W,   W [B][n] = L11^{-1} ak,  ak: the pivot rows, with the identity in the panel's columns
+//                ap [n][B]: -L21 below the pivot rows, -A_panel U11^{-1} above them, U11^{-1} in them
+// after the rows the pivots interchanged have moved and the panel's columns and the pivot rows of A are zero:
+// the pivot rows become D^{-1} A_p (D = L11 U11 the pivot block), the panel -A_panel D^{-1}, its pivot block
+// D^{-1}, the rest A - A_panel D^{-1} A_p. Both triangles are applied by substitution (a thread per row of ap or
+// column of W), never D^{-1} itself: rounding of W then meets multipliers of at most 1 instead of
+// |A_panel| |D^{-1}|, as in an elimination column by column (with D^{-1} the error grows with cond(D): 1e-3
+// instead of 1e-9 for column pairs that differ by 1e-6).
+// The digits of a row share one scale, so the B terms of the product are balanced by exact powers of two: row t
+// of W is brought to about 1 and column t of ap takes its size (without: 2e-7 where five rows of a panel are 1e10
+// times the others).
+// What bounds the kernel is the chain of a column (search, one division, swap, update: 5 block-wide steps), then
+// the FP64 pipe: B^2/2 complex multiply-adds per row and per column. swp[c]: the row swapped with row c at step c.
 template <int B>
 size_t gj_panel_smem(int n) {
   return (size_t)n * (B + 1) * sizeof(double2);
 }
+constexpr int kGjBalanceMax = 400;       // powers of two of the balance: no over- or underflow of ordinary values
 template <int B>
 __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, long long stride, const int* list, int k0,
-                                                       double2* ak_all, double2* ap_all, double2* dinv_all,
-                                                       int* swp_all, int* status) {
+                                                       double2* ap_all, double2* w_all, int* swp_all, int* status) {
   extern __shared__ double2 sm[];
   __shared__ long long red_v[8];
   __shared__ int red_i[8];
   __shared__ int s_p, s_bad, s_cnt;
   __shared__ int s_swp[B], s_row[2 * B], s_src[2 * B];
-  __shared__ double2 s_inv, D[B][B + 1], drow[B], dcol[B];
+  __shared__ unsigned int s_max[B];        // largest |re|, |im| of a row of W (leading 32 bits)
+  __shared__ double2 s_inv, s_dinv[B];
   double2* M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
-  double2* ak = ak_all + (long long)blockIdx.x * B * n;
   double2* ap = ap_all + (long long)blockIdx.x * B * n;
-  double2* dinv = dinv_all + (long long)blockIdx.x * B * B;
+  double2* W = w_all + (long long)blockIdx.x * B * n;
   int* swp = swp_all + (long long)blockIdx.x * n;
   const int nr = n - k0;                   // rows k0.. of the panel
   double2* P = sm;                         // [nr][B]
@@ -370,7 +372,14 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
     const double den = v.x * v.x + v.y * v.y;
     return make_double2(v.x / den, -v.y / den);
   };
+  auto msub = [](double2& v, double2 f, double2 r) {   // v -= f r
+    v.x = fma(-f.x, r.x, v.x);
+    v.x = fma(f.y, r.y, v.x);
+    v.y = fma(-f.x, r.y, v.y);
+    v.y = fma(-f.y, r.x, v.y);
+  };
   if (tid == 0) s_bad = 0;
+  if (tid < B) s_max[tid] = 0;
   for (int e = tid; e < nr * B; e += blockDim.x) {
     const int i = e / B, j = e % B;
     P[e] = j < kb ? M[(long long)(k0 + i) * n + k0 + j] : make_double2(0.0, 0.0);
@@ -400,14 +409,14 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
         if (red_v[w] > bb || (red_v[w] == bb && red_i[w] < ii)) { bb = red_v[w]; ii = red_i[w]; }
       s_p = ii;
       s_swp[j] = k0 + ii;
-      s_inv = inverse(P[ii * B + j]);      // one thread: 256 divisions would cost the FP64 pipe 3k clocks
+      s_inv = s_dinv[j] = inverse(P[ii * B + j]);   // one thread: 256 divisions would cost the FP64 pipe 3k clocks
       if (!(bb > 0)) s_bad = 1;
     }
     __syncthreads();
     if (s_bad) break;
     const int p = s_p;
     const double2 inv = s_inv;
-    // row j takes what row p holds and the other way round (columns j.. are all that is read again)
+    // row j takes what row p holds and the other way round
     for (int i = j + 1 + tid; i < nr; i += blockDim.x) fcol[i] = cmul(P[(i == p ? j : i) * B + j], inv);
     double2 rp = make_double2(0.0, 0.0), rj = rp;
     if (tid < B) {
@@ -420,22 +429,23 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
       P[p * B + tid] = rj;
     }
     __syncthreads();
-    const int w = kb - j - 1;              // columns j + 1.. of the rows below j
+    const int w = kb - j;                  // columns j.. of the rows below j; column j keeps the multipliers
     for (int e = tid; e < w * (nr - j - 1); e += blockDim.x) {
-      const int i = j + 1 + e / w, jj = j + 1 + e % w;
-      const double2 f = fcol[i], r = P[j * B + jj];
-      double2 v = P[i * B + jj];
-      v.x = fma(-f.x, r.x, v.x);
-      v.x = fma(f.y, r.y, v.x);
-      v.y = fma(-f.x, r.y, v.y);
-      v.y = fma(-f.y, r.x, v.y);
+      const int i = j + 1 + e / w, jj = j + e % w;
+      double2 v = fcol[i];
+      if (jj > j) {
+        const double2 f = v;
+        v = P[i * B + jj];
+        msub(v, f, P[j * B + jj]);
+      }
       P[i * B + jj] = v;
     }
     __syncthreads();
   }
-  if (s_bad) {
+  if (s_bad) {                             // no step: the product adds nothing to this matrix
     if (tid == 0) atomicExch(status, 1);
     for (int t = tid; t < kb; t += blockDim.x) swp[k0 + t] = k0 + t;
+    for (int e = tid; e < n * B; e += blockDim.x) ap[e] = W[e] = make_double2(0.0, 0.0);
     return;
   }
   if (tid < kb) swp[k0 + tid] = s_swp[tid];
@@ -459,72 +469,85 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
   }
   __syncthreads();
   const int cnt = s_cnt;
-  // ---- D^{-1}: Gauss-Jordan on the pivot block, whose rows are in pivot order
-  if (tid < B * B) {
-    const int a = tid / B, c = tid % B;
-    D[a][c] = a < kb && c < kb ? M[(long long)s_src[a] * n + k0 + c] : make_double2(0.0, 0.0);
+  // ---- the other columns: pivot rows out, interchanged rows moved; W = L11^{-1} ak
+  unsigned int mx[B];
+#pragma unroll
+  for (int t = 0; t < B; ++t) mx[t] = 0;
+  for (int col = tid; col < n; col += blockDim.x) {
+    const bool panel = col >= k0 && col < k0 + kb;
+    double2 v[2 * B];
+    if (panel) {
+#pragma unroll
+      for (int t = 0; t < B; ++t) v[t] = make_double2(col - k0 == t ? 1.0 : 0.0, 0.0);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 2 * B; ++t)
+        if (t < cnt) v[t] = M[(long long)s_src[t] * n + col];
+#pragma unroll
+      for (int t = 0; t < 2 * B; ++t)
+        if (t < cnt) M[(long long)s_row[t] * n + col] = t < kb ? make_double2(0.0, 0.0) : v[t];
+    }
+#pragma unroll
+    for (int t = 0; t < B; ++t)
+      if (t < kb) {
+        double2 x = v[t];
+#pragma unroll
+        for (int s = 0; s < t; ++s) msub(x, P[t * B + s], v[s]);
+        v[t] = x;
+        W[(long long)t * n + col] = x;
+        if (!panel) mx[t] = max(mx[t], (unsigned int)max(__double2hiint(x.x) & 0x7FFFFFFF, __double2hiint(x.y) & 0x7FFFFFFF));
+      }
+  }
+#pragma unroll
+  for (int t = 0; t < B; ++t) {
+    const unsigned int m = __reduce_max_sync(0xffffffffu, mx[t]);
+    if (lane == 0) atomicMax(&s_max[t], m);
   }
   __syncthreads();
-  for (int j = 0; j < kb; ++j) {
-    if (tid == 0) s_inv = inverse(D[j][j]);
-    __syncthreads();
-    if (tid < B) {
-      drow[tid] = tid == j ? s_inv : cmul(D[j][tid], s_inv);
-      dcol[tid] = D[tid][j];
-    }
-    __syncthreads();
-    if (tid < B * B) {
-      const int a = tid / B, c = tid % B;
-      const double2 f = dcol[a], r = drow[c];
-      double2 v = c == j ? make_double2(0.0, 0.0) : D[a][c];
-      v.x = fma(-f.x, r.x, v.x);
-      v.x = fma(f.y, r.y, v.x);
-      v.y = fma(-f.x, r.y, v.y);
-      v.y = fma(-f.y, r.x, v.y);
-      D[a][c] = a == j ? r : v;
-    }
-    __syncthreads();
+  auto size_of = [&](int t) {              // about log2 of the largest element of row t of W
+    const int ex = (int)(s_max[t] >> 20);
+    return ex == 0 || ex == 0x7FF ? 0 : max(-kGjBalanceMax, min(kGjBalanceMax, ex - 1022));
+  };
+  auto pow2 = [](int e) { return __longlong_as_double((long long)(e + 1023) << 52); };
+  for (int e = tid; e < n * kb; e += blockDim.x) {
+    const double2 v = W[e];
+    const double f = pow2(-size_of(e / n));
+    W[e] = make_double2(v.x * f, v.y * f);
   }
-  if (tid < B * B) dinv[tid] = D[tid / B][tid % B];
-  // ---- the panel, negated, its rows in their new order, the identity in the pivot rows
-  for (int e = tid; e < n * B; e += blockDim.x) {
-    const int i = e / B, j = e % B;
-    double2 v = make_double2(0.0, 0.0);
-    if (i >= k0 && i < k0 + kb) v.x = i - k0 == j ? 1.0 : 0.0;
-    else if (j < kb) {
-      v = M[(long long)i * n + k0 + j];
-      v = make_double2(-v.x, -v.y);
+  // ---- ap: the multipliers below, x U11 = -A_panel (above) or the identity (pivot rows) by substitution
+  for (int i = tid; i < n; i += blockDim.x) {
+    double2 v[B];
+    if (i >= k0 + kb) {
+#pragma unroll
+      for (int t = 0; t < B; ++t) v[t] = make_double2(-P[(i - k0) * B + t].x, -P[(i - k0) * B + t].y);
+    } else {
+#pragma unroll
+      for (int t = 0; t < B; ++t) {
+        v[t] = make_double2(i - k0 == t ? 1.0 : 0.0, 0.0);
+        if (i < k0 && t < kb) {
+          const double2 a = M[(long long)i * n + k0 + t];
+          v[t] = make_double2(-a.x, -a.y);
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < B; ++t)
+        if (t < kb) {
+          double2 x = v[t];
+#pragma unroll
+          for (int s = 0; s < t; ++s) msub(x, v[s], P[s * B + t]);
+          v[t] = cmul(x, s_dinv[t]);
+        }
     }
-    ap[e] = v;
-  }
-  __syncthreads();
-  for (int e = tid; e < (cnt - kb) * B; e += blockDim.x) {
-    const int t = kb + e / B, j = e % B;
-    if (j >= kb) continue;
-    const double2 v = M[(long long)s_src[t] * n + k0 + j];
-    ap[(long long)s_row[t] * B + j] = make_double2(-v.x, -v.y);
+#pragma unroll
+    for (int t = 0; t < B; ++t) {
+      const double f = t < kb ? pow2(size_of(t)) : 0.0;
+      ap[(long long)i * B + t] = t < kb ? make_double2(v[t].x * f, v[t].y * f) : make_double2(0.0, 0.0);
+    }
   }
   __syncthreads();
   for (int e = tid; e < n * B; e += blockDim.x) {
     const int i = e / B, j = e % B;
     if (j < kb) M[(long long)i * n + k0 + j] = make_double2(0.0, 0.0);
-  }
-  // ---- the other columns: pivot rows out, interchanged rows moved
-  for (int col = tid; col < n; col += blockDim.x) {
-    if (col >= k0 && col < k0 + kb) {
-      for (int t = 0; t < B; ++t) ak[(long long)t * n + col] = make_double2(col - k0 == t ? 1.0 : 0.0, 0.0);
-      continue;
-    }
-    double2 v[2 * B];
-#pragma unroll
-    for (int t = 0; t < 2 * B; ++t)
-      if (t < cnt) v[t] = M[(long long)s_src[t] * n + col];
-#pragma unroll
-    for (int t = 0; t < 2 * B; ++t)
-      if (t < cnt) {
-        if (t < kb) ak[(long long)t * n + col] = v[t];
-        M[(long long)s_row[t] * n + col] = t < kb ? make_double2(0.0, 0.0) : v[t];
-      }
   }
 }
 
@@ -976,8 +999,8 @@ bool gj_panel_attr() {
   return ok;
 }
 
-// per matrix: the panel's ak, ap and W, D^{-1} and the swaps, and the digits of the larger product
-size_t gj_side_bytes(int n, int B) { return (size_t)(3 * B * n + B * B) * sizeof(double2) + (size_t)n * sizeof(int); }
+// per matrix: the panel's ap and W, the swaps, and the digits of the product
+size_t gj_side_bytes(int n, int B) { return (size_t)(2 * B * n) * sizeof(double2) + (size_t)n * sizeof(int); }
 size_t gj_group_bytes(int n, int B) { return oz64_bytes(n, n, B) + gj_side_bytes(n, B) + 256; }
 
 // Panels and tensor-core updates of groups of matrices whose digits, pivot rows and swaps fit ws
@@ -992,47 +1015,18 @@ int inverse_panels(double2* base, int n, long long stride, int nbatch, int* stat
     double2* b0 = list ? base : base + (long long)m0 * stride;
     const int* l0 = list ? list + m0 : nullptr;
     const long long pn = (long long)B * n;
-    double2* ak = reinterpret_cast<double2*>(ws.mem);
-    double2* ap = ak + m * pn;
+    double2* ap = reinterpret_cast<double2*>(ws.mem);
     double2* W = ap + m * pn;
-    double2* dinv = W + m * pn;
-    int* swp = reinterpret_cast<int*>(dinv + (long long)m * B * B);
+    int* swp = reinterpret_cast<int*>(W + m * pn);
     const size_t head = (m * gj_side_bytes(n, B) + 255) / 256 * 256;
     Oz64Ws rest = ws;
     rest.mem = (unsigned char*)ws.mem + head;
     rest.bytes = ws.bytes - head;
-    auto product = [&](const ZGemm& z) {
-      bool done = false;
-      const int rc = zgemm_oz64(z, st, &done);
-      return rc != GW_OK || done ? rc : fail(GW_ENOMEM, "batched_inverse: digit workspace of %zu bytes too small for n=%d",
-                                             ws.bytes, n);
-    };
     for (int k0 = 0; k0 < n; k0 += B) {
       const int kb = std::min(B, n - k0);
       prof_begin(SLOT_INVERSE_FP64, st);
-      gj_panel_kernel<B><<<m, 256, gj_panel_smem<B>(n - k0), st>>>(b0, n, stride, l0, k0, ak, ap, dinv, swp, status);
-      prof_end(SLOT_INVERSE_FP64, st, 4.0 * m * (double)(n - k0) * kb * kb, 32.0 * m * (double)n * (4 * kb));
-      ZGemm w;                               // W = D^{-1} ak
-      w.M = kb;
-      w.N = n;
-      w.K = kb;
-      w.nbatch = m;
-      w.A = dinv;
-      w.va.rs_in = B;
-      w.va.ks_in = 1;
-      w.ba.bs_in = B * B;
-      w.B = ak;
-      w.vb.rs_in = 1;
-      w.vb.ks_in = n;
-      w.bb.bs_in = pn;
-      w.C = W;
-      w.vc.rs_in = n;
-      w.vc.ks_in = 1;
-      w.bc.bs_in = pn;
-      w.slot = SLOT_INVERSE_FP64;
-      w.ws = &rest;
-      int rc = product(w);
-      if (rc != GW_OK) return rc;
+      gj_panel_kernel<B><<<m, 256, gj_panel_smem<B>(n - k0), st>>>(b0, n, stride, l0, k0, ap, W, swp, status);
+      prof_end(SLOT_INVERSE_FP64, st, 4.0 * m * (double)(3 * n - k0) * kb * kb, 32.0 * m * (double)n * (3 * kb));
       ZGemm z;                               // A += ap W
       z.M = n;
       z.N = n;
@@ -1054,8 +1048,10 @@ int inverse_panels(double2* base, int n, long long stride, int nbatch, int* stat
       z.accumulate = 1;
       z.slot = SLOT_INVERSE_FP64;
       z.ws = &rest;
-      rc = product(z);
+      bool done = false;
+      const int rc = zgemm_oz64(z, st, &done);
       if (rc != GW_OK) return rc;
+      if (!done) return fail(GW_ENOMEM, "batched_inverse: digit workspace of %zu bytes too small for n=%d", ws.bytes, n);
     }
     const int rows = std::max(1, std::min((n + kPermRows - 1) / kPermRows, (1216 + m - 1) / m));
     prof_begin(SLOT_INVERSE_FP64, st);
