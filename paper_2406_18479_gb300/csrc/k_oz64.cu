@@ -25,8 +25,10 @@
 // their packing. Error against 64-bit references on these: 2e-16 and 4e-16 (FP64 pipe: 3e-15 and 6e-15).
 //
 // Rows with a non-finite element, or whose scale lies outside 2^+-480 (where the scaled product
-// could over- or underflow), carry a NaN scale; outputs that meet one are computed by a plain
-// FP64 loop in the epilogue, so infinities, NaN and extreme ranges behave as in zgemm_fp64.
+// could over- or underflow), carry a NaN scale. The epilogue leaves outputs that meet one alone, and the CTA
+// computes them on the FP64 pipe after its last tile (plain_tiles), so infinities, NaN and extreme ranges
+// behave as in zgemm_fp64. (A loop over K in the epilogue itself would keep the CTA's other warps in waits that
+// give up after 4 s: reached from K of about 10^6.)
 //
 // Kernels
 //   oz64_pack_kernel  FP64 views -> digit tiles, in the order the tensor core reads shared memory
@@ -51,7 +53,7 @@ constexpr int kDigits = 8;
 constexpr int kK = 16;              // real k per MMA
 constexpr int kChunkSteps = 8;      // k-steps per exact chunk (128 real k)
 constexpr int kPTile = 64;          // complex rows of P per tile (128 TMEM lanes)
-constexpr int kScaleMax = 480;      // |E| beyond this takes the plain FP64 loop
+constexpr int kScaleMax = 480;      // |E| beyond this has no digit form
 constexpr int kEpiWarps = 16;
 constexpr int kSegSteps = 8;        // least k-steps of a packing segment
 constexpr int kMaxSegs = 32;
@@ -86,7 +88,7 @@ struct Side {
   int dep_o = 0, dep_i = 0;             // whether the operand varies with the outer / inner batch index
   int no = 1, ni = 1;                   // packed batches
   unsigned char* dst = nullptr;
-  double* scale = nullptr;              // per packed row: 2^(E - 34), NaN: plain FP64 loop
+  double* scale = nullptr;              // per packed row: 2^(E - 34), NaN: no digit form
   unsigned long long* pmax = nullptr;   // segs > 1: largest |value| bits of each row and K segment
 };
 
@@ -278,16 +280,103 @@ __global__ void __launch_bounds__(256) oz64_pack_kernel(const __grid_constant__ 
   else pack_tile<NT, false>(j.q, j, blockIdx.x - np);
 }
 
-// the plain FP64 loop of one real output (part 0: re, 1: im), for rows without a digit form
-__device__ __noinline__ double plain_dot(const Job& j, int bo, int bi, int pr, int qr, int part) {
-  const double2* a = side_base(j.p, bo, bi) + side_row(j.p, pr);
-  const double2* b = side_base(j.q, bo, bi) + side_row(j.q, qr);
-  double s = 0.0;
-  for (int k = 0; k < j.K; ++k) {
-    const double2 x = a[side_k(j.p, k)], y = b[side_k(j.q, k)];
-    s = part ? fma(x.y, y.x, fma(x.x, y.y, s)) : fma(-x.y, y.y, fma(x.x, y.x, s));
+// The outputs of this CTA's tiles that the digits do not give: a group of 256 threads per 32 x 32 complex outputs, the
+// terms in order of k on the FP64 pipe as in zgemm_fp64_kernel. A thread has 2 x 2 outputs and a warp skips those that
+// none of its lanes needs, so a few of them cost the staging of their operands and little arithmetic. Of CTAs that share
+// a tile's K the first takes it. sm: the group's 2 kPlainK rows of 33 elements and the masks.
+constexpr int kPlainK = 16, kPlainGroups = kEpiWarps / 8;
+constexpr size_t kPlainSmem = 2 * kPlainK * 33 * sizeof(double2) + 256;   // of a group
+template <int NT>
+__device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, int group, int tid, unsigned char* sm) {
+  double2(*Ps)[33] = reinterpret_cast<double2(*)[33]>(sm);
+  double2(*Qs)[33] = Ps + kPlainK;
+  uint32_t* s_row = reinterpret_cast<uint32_t*>(Qs + kPlainK);          // rows of P, rows of Q without a digit form
+  auto sync = [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + group) : "memory"); };
+  constexpr int kSub = 2 * (NT / 32);                 // 32 x 32 pieces of a GEMM tile
+  const int per_batch = j.p.tiles * j.q.tiles, total = per_batch * j.no * j.ni * ksplit;
+  const int tx = tid & 15, ty = tid >> 4;
+  for (int unit = blockIdx.x; unit < total; unit += gridDim.x) {
+    const int tile = unit / ksplit;
+    if (unit != tile * ksplit) continue;
+    const int b = tile / per_batch, w = tile - b * per_batch, o = b / j.ni, i = b - o * j.ni;
+    const int pt = w / j.q.tiles, qt = w - pt * j.q.tiles;
+#pragma unroll 1
+    for (int sub = group; sub < kSub; sub += kPlainGroups) {
+      const int p0 = (sub & 1) * 32, q0 = (sub >> 1) * 32;        // of the tile
+      const int np = min(32, j.p.rows - pt * kPTile - p0), nq = min(32, j.q.rows - qt * NT - q0);
+      if (np <= 0 || nq <= 0) continue;
+      sync();
+      if (tid < 64) {
+        const Side& s = tid < 32 ? j.p : j.q;
+        const long long at = (((long long)(s.dep_o ? o : 0) * s.ni + (s.dep_i ? i : 0)) * s.tiles + (tid < 32 ? pt : qt)) *
+                             (tid < 32 ? kPTile : NT) + (tid < 32 ? p0 : q0) + (tid & 31);
+        const uint32_t m = __ballot_sync(0xffffffffu, isnan(s.scale[at]));
+        if ((tid & 31) == 0) s_row[tid >> 5] = m;
+      }
+      sync();
+      const uint32_t rows = s_row[0] & (np < 32 ? (1u << np) - 1 : ~0u), cols = s_row[1] & (nq < 32 ? (1u << nq) - 1 : ~0u);
+      if ((rows | cols) == 0) continue;
+      bool need[2][2];
+      double2 acc[2][2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          const int r = 2 * tx + u, c = 2 * ty + v;
+          need[u][v] = r < np && c < nq && (((rows >> r) | (cols >> c)) & 1);
+          acc[u][v] = make_double2(0.0, 0.0);
+        }
+      const int bo = j.o0 + o, bi = j.i0 + i;
+      const double2* A = side_base(j.p, bo, bi);
+      const double2* B = side_base(j.q, bo, bi);
+      const int pr = j.p.row0 + pt * kPTile + p0, qr = j.q.row0 + qt * NT + q0;
+      const bool pk = j.p.ks_in == 1, qk = j.q.ks_in == 1;         // neighbouring threads on neighbouring elements
+#pragma unroll 1
+      for (int k0 = 0; k0 < j.K; k0 += kPlainK) {
+        sync();
+#pragma unroll
+        for (int e = tid; e < 32 * kPlainK; e += 256) {
+          const int rp = pk ? e / kPlainK : e % 32, kp = pk ? e % kPlainK : e / 32;
+          const int rq = qk ? e / kPlainK : e % 32, kq = qk ? e % kPlainK : e / 32;
+          Ps[kp][rp] = rp < np && k0 + kp < j.K ? A[side_row(j.p, pr + rp) + side_k(j.p, k0 + kp)] : make_double2(0.0, 0.0);
+          Qs[kq][rq] = rq < nq && k0 + kq < j.K ? B[side_row(j.q, qr + rq) + side_k(j.q, k0 + kq)] : make_double2(0.0, 0.0);
+        }
+        sync();
+        const int kn = min(kPlainK, j.K - k0);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int v = 0; v < 2; ++v) {
+            if (!need[u][v]) continue;
+            double2 s = acc[u][v];
+#pragma unroll 4
+            for (int k = 0; k < kn; ++k) {
+              const double2 x = Ps[k][2 * tx + u], y = Qs[k][2 * ty + v];
+              s.x = fma(-x.y, y.y, fma(x.x, y.x, s.x));
+              s.y = fma(x.y, y.x, fma(x.x, y.y, s.y));
+            }
+            acc[u][v] = s;
+          }
+      }
+      double2* C = j.C + batch_in(j.bc, bi) + (long long)bo * j.bc.bs_out;
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          if (!need[u][v]) continue;
+          const int a = pr + 2 * tx + u, aq = div_by(a, j.cp_div), c = qr + 2 * ty + v, cq = div_by(c, j.cq_div);
+          double2* at = C + (long long)aq * j.cp_out + (long long)(a - aq * j.cp_div.d) * j.cp_in + (long long)cq * j.cq_out +
+                        (long long)(c - cq * j.cq_div.d) * j.cq_in;
+          double2 x = make_double2(j.alpha * acc[u][v].x, j.alpha * acc[u][v].y);
+          if (j.accumulate) {
+            const double2 old = *at;
+            x.x += old.x;
+            x.y += old.y;
+          }
+          *at = x;
+        }
+    }
   }
-  return s;
 }
 
 template <int NT>
@@ -301,6 +390,7 @@ struct Oz64Shape {
   static constexpr int kThreads = 64 + 32 * kEpiWarps;          // producer, MMA, epilogue warps
   static constexpr size_t kSmem = 128 + (size_t)kStages * kStageBytes + 256;
   static_assert(kSmem <= 232448, "stages exceed shared memory");
+  static_assert(kPlainGroups * kPlainSmem <= (size_t)kStages * kStageBytes, "plain_tiles works in the stages");
 };
 
 // K-major operand without swizzle: 8 x 16-byte core matrices, 128 bytes between the two k halves
@@ -383,6 +473,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
   uint64_t* drain_bar = acc_full + 4;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* plain_flag = abort_flag + 1;    // some output of this CTA's tiles is left to plain_tiles
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -396,6 +487,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
+    *plain_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -515,7 +607,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
       const int bo = j.o0 + o, bi = j.i0 + i;
       const int pr = pt * kPTile + (lrow >> 1);
       const bool p_ok = pr < j.p.rows;
-      // biased exponents of the scales (0x7FF: a row for the plain loop)
+      // biased exponents of the scales (0x7FF: a row without a digit form)
       const int ep = __double2hiint(j.p.scale[((long long)packed(j.p, o, i) * j.p.tiles + pt) * kPTile + (lrow >> 1)]) >> 20;
       const double* sq = j.q.scale + ((long long)packed(j.q, o, i) * j.q.tiles + qt) * NT;
       const int ap = j.p.row0 + (p_ok ? pr : 0), apq = div_by(ap, j.cp_div);
@@ -527,7 +619,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
         return C + 2 * ((long long)aqq * j.cq_out + (long long)(aq - aqq * j.cq_div.d) * j.cq_in);
       };
       auto col_ok = [&](int col) { return p_ok && qt * NT + col < j.q.rows; };
-      bool special = false;           // some output needs the plain loop (done after the others)
+      if (ep == 0x7FF || (lane < kCols && qt * NT + half * kCols + lane < j.q.rows && isnan(sq[half * kCols + lane]))) *plain_flag = 1;
       const bool quick = j.nks <= kFinishSteps;
       auto put = [&](int col, long long hi, long long lo, double old) {
         const int eq = col_ok(col) ? __double2hiint(sq[col]) >> 20 : 1023;
@@ -536,7 +628,6 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
         const double x = !MULTI || quick ? finish(hi, lo, e, j.alpha, old)
                                          : fma(to_fp64(hi, (uint32_t)lo, e), j.alpha, old);
         if (col_ok(col) && !plain) *at(col) = x;
-        special |= plain && col_ok(col);
       };
       // outputs that are added to are read ahead of the wait for the accumulators (a load behind every
       // store would put 16 memory latencies in a row: 24k clocks a tile instead of 5k)
@@ -624,21 +715,16 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
           for (int u = 0; u < 4; ++u) put(half * kCols + u0 + u, hi[u0 + u], lo[u0 + u], o4[u]);
         }
       }
-      if (special) {
-#pragma unroll 1
-        for (int col = half * kCols; col < half * kCols + kCols; ++col) {
-          if (!col_ok(col) || (ep != 0x7FF && __double2hiint(sq[col]) >> 20 != 0x7FF)) continue;
-          const double x = j.alpha * plain_dot(j, bo, bi, ap, j.q.row0 + qt * NT + col, part);
-          double* c = at(col);
-          *c = j.accumulate ? *c + x : x;
-        }
-      }
     }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+  if (*plain_flag && !*abort_flag && warp >= 2) {
+    const int t = threadIdx.x - 64;
+    plain_tiles<NT>(j, ksplit, t >> 8, t & 255, smem + (t >> 8) * kPlainSmem);
+  }
 }
 
 int sm_count() {
