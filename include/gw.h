@@ -70,8 +70,9 @@ typedef enum {
 } gw_status;
 
 typedef enum {
-  GW_FP64 = 0,          /* every contraction to FP64 accuracy (on the tensor cores through exact integer
-                           digits where that pays, with a smaller error than a running FP64 sum) */
+  GW_FP64 = 0,          /* every contraction within the error bound of an FP64 sum of its terms (on the
+                           tensor cores through exact integer digits where that pays; outputs whose
+                           operands are graded against one another stay on the FP64 pipe) */
   GW_MIXED_BF16X4 = 1,  /* V.G.V contractions on tcgen05 tensor cores: each operand row is cut,
                            per chunk of at most 256 k, into four bf16 slices on one power-of-two
                            alignment; slice products of order 0 and 1 sum exactly in their own

@@ -124,6 +124,7 @@ struct gw_ctx {
   int nk = 0, nao = 0, naux = 0, ntau = 0, nwb = 0, nwf = 0, nt = 1;
   long long nao2 = 0, naux2 = 0, pair = 0;
   double2 *Fb = nullptr, *Bb = nullptr, *Ff = nullptr, *Bf = nullptr;
+  int *Fbe = nullptr, *Bbe = nullptr, *Ffe = nullptr, *Bfe = nullptr;   // powers of two of their columns (ZGemm::kexp)
   double* wf = nullptr;                   // fermionic frequencies (device)
   long long* tabs = nullptr;              // 6 tables [nq][nk]
   long long *tab_kkpq = nullptr, *tab_kpqk = nullptr, *tab_gkpq = nullptr;
@@ -219,7 +220,7 @@ int cuda_check(const char* what) {
 void free_ctx(gw_ctx* c) {
   if (!c) return;
   mixed_destroy(c->mixed);
-  void* ptrs[] = {c->Fb, c->Bb, c->Ff, c->Bf, c->wf, c->tabs, c->mq_dev, c->wlist, c->wlist_q, c->work, c->P0t, c->Pw,
+  void* ptrs[] = {c->Fb, c->Bb, c->Ff, c->Bf, c->Fbe, c->Bbe, c->Ffe, c->Bfe, c->wf, c->tabs, c->mq_dev, c->wlist, c->wlist_q, c->work, c->P0t, c->Pw,
                   c->Pt, c->dyson_ws, c->status, c->maxdiff, c->nonfinite, c->wbeta, c->gamma, c->rho,
                   c->xinf, c->scal, c->gw_w, c->heff, c->gf2_ws, c->Vfull, c->cw_tmp, c->oz_mem, c->oz_small, c->oz_count};
   for (void* p : ptrs)
@@ -227,7 +228,34 @@ void free_ctx(gw_ctx* c) {
   delete c;
 }
 
-int upload_grid(gw_ctx* c, int stat, double2** F, double2** B, int* nw_out) {
+// Powers of two for the k of a transform's matrix m [rows][cols] (ZGemm::kexp), which keep its outputs with the digits:
+// first rows and columns are brought to a common largest element (a caller's grid may weigh its nodes by any
+// amount), then the columns, halfway, to 1. Fully to 1 the inputs of noise lose (up to 90% of their back transforms
+// left to the FP64 pipe), not at all the bosonic functions of low energy (up to 10%); halfway at most 2% of either,
+// mostly none (32 to 200 nodes, beta 20 to 400).
+std::vector<int> column_exponents(const gw_c128* m, int rows, int cols) {
+  std::vector<double> l((size_t)rows * cols), r(rows, 0.0), c(cols, 0.0), h(cols, -1e9);
+  double top = 0.0;
+  for (size_t i = 0; i < l.size(); ++i) top = std::max(top, l[i] = std::max(std::fabs(m[i].re), std::fabs(m[i].im)));
+  if (!(top > 0.0 && std::isfinite(top))) return std::vector<int>(cols, 0);
+  for (double& x : l) x = std::max(x > 0.0 ? std::log2(x / top) : -100.0, -100.0);
+  for (int it = 0; it < 3; ++it) {
+    for (int n = 0; n < rows; ++n) {
+      r[n] = -1e9;
+      for (int k = 0; k < cols; ++k) r[n] = std::max(r[n], l[(size_t)n * cols + k] - c[k]);
+    }
+    c.assign(cols, -1e9);
+    for (int n = 0; n < rows; ++n)
+      for (int k = 0; k < cols; ++k) c[k] = std::max(c[k], l[(size_t)n * cols + k] - r[n]);
+  }
+  for (int n = 0; n < rows; ++n)
+    for (int k = 0; k < cols; ++k) h[k] = std::max(h[k], l[(size_t)n * cols + k] - std::rint(c[k]));
+  std::vector<int> e(cols);
+  for (int k = 0; k < cols; ++k) e[k] = (int)std::rint(std::rint(c[k]) + 0.5 * h[k]);
+  return e;
+}
+
+int upload_grid(gw_ctx* c, int stat, double2** F, double2** B, int** Fe, int** Be, int* nw_out) {
   const int nw = sample_count(c->ntau, stat);
   std::vector<gw_c128> hF((size_t)nw * c->ntau), hB((size_t)c->ntau * nw);
   std::vector<int64_t> idx(nw);
@@ -236,6 +264,11 @@ int upload_grid(gw_ctx* c, int stat, double2** F, double2** B, int* nw_out) {
   GW_TRY(dev_alloc(c, B, hB.size()));
   upload(c, *F, hF.data(), hF.size() * sizeof(double2));
   upload(c, *B, hB.data(), hB.size() * sizeof(double2));
+  const std::vector<int> eF = column_exponents(hF.data(), nw, c->ntau), eB = column_exponents(hB.data(), c->ntau, nw);
+  GW_TRY(dev_alloc(c, Fe, eF.size()));
+  GW_TRY(dev_alloc(c, Be, eB.size()));
+  upload(c, *Fe, eF.data(), eF.size() * sizeof(int));
+  upload(c, *Be, eB.data(), eB.size() * sizeof(int));
   if (stat == 1) {
     std::vector<double> w(nw);
     for (int n = 0; n < nw; ++n) w[n] = (2.0 * (double)idx[n] + 1.0) * M_PI / c->cfg.beta;
@@ -375,6 +408,7 @@ int transform(gw_ctx* c, int stat, bool forward, const double2* in, double2* out
     g.C = out + (long long)b0 * nout * nelem; g.vc.rs_in = nelem; g.vc.ks_in = 1; g.bc.bs_in = nout * nelem;
     g.slot = SLOT_TRANSFORM_FP64;
     g.ws = stat == 0 ? (forward ? &c->oz_fwd : &c->oz_back) : &c->oz_w;
+    g.kexp = forward ? (stat == 0 ? c->Fbe : c->Ffe) : (stat == 0 ? c->Bbe : c->Bfe);
     GW_TRY(zgemm_fp64(g, c->stream));
   }
   return GW_OK;
@@ -394,6 +428,7 @@ int transform_q(gw_ctx* c, int stat, bool forward, const double2* in, double2* o
   g.C = out + ((long long)q * nout + row0) * nelem; g.vc.rs_in = nelem; g.vc.ks_in = 1;
   g.slot = SLOT_TRANSFORM_FP64;
   g.ws = stat == 0 ? (forward ? &c->oz_fwd : &c->oz_back) : &c->oz_w;
+  g.kexp = forward ? (stat == 0 ? c->Fbe : c->Ffe) : (stat == 0 ? c->Bbe : c->Bfe);
   return zgemm_fp64(g, c->stream);
 }
 
@@ -542,8 +577,8 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
   c->pair = (long long)c->naux * c->nao2;
   int rc = GW_OK;
   do {
-    if ((rc = upload_grid(c, 0, &c->Fb, &c->Bb, &c->nwb)) != GW_OK) break;
-    if ((rc = upload_grid(c, 1, &c->Ff, &c->Bf, &c->nwf)) != GW_OK) break;
+    if ((rc = upload_grid(c, 0, &c->Fb, &c->Bb, &c->Fbe, &c->Bbe, &c->nwb)) != GW_OK) break;
+    if ((rc = upload_grid(c, 1, &c->Ff, &c->Bf, &c->Ffe, &c->Bfe, &c->nwf)) != GW_OK) break;
     // k-mesh gather tables (element offsets), [q][k]
     std::vector<long long> t(6 * (size_t)nk * nk);
     const long long gk = (long long)c->ntau * c->nao2;
@@ -767,6 +802,11 @@ int gw_set_grids(gw_ctx* ctx, const double* tau_host, const gw_c128* Fb_host, co
       cudaMemcpy(ctx->Bf, Bf_host, sf, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(ctx->wf, omega_f_host, (size_t)nf * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
     return cuda_check("gw_set_grids copy");
+  const std::pair<int*, std::vector<int>> exps[] = {{ctx->Fbe, column_exponents(Fb_host, nb, T)}, {ctx->Bbe, column_exponents(Bb_host, T, nb)},
+                                                    {ctx->Ffe, column_exponents(Ff_host, nf, T)}, {ctx->Bfe, column_exponents(Bf_host, T, nf)}};
+  for (const auto& e : exps)
+    if (cudaMemcpy(e.first, e.second.data(), e.second.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+      return cuda_check("gw_set_grids copy");
   std::vector<double> w;
   weights_at_beta(tau_host, T, beta, w);
   if (cudaMemcpy(ctx->wbeta, w.data(), (size_t)T * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)

@@ -102,10 +102,12 @@ struct ZGemm {
   int slot = SLOT_VG_FP64;       // profiling slot of this launch
   const Oz64Ws* ws = nullptr;    // digit workspace: with one, products that pay run on the tensor cores
   double unit = 0.0;             // complex multiply-adds of one (k, tau) matrix where a product joins several
+  int skip0 = 0, skip1 = 0;      // outputs with m and n both in [skip0, skip1) are not written (K <= 64 and the digits only)
+  const int* kexp = nullptr;     // digits of A(m, k) 2^-kexp[k] and B(n, k) 2^kexp[k] (device, K; the product is the same)
 };
 
-// C = alpha A B^T (+ C) to FP64 accuracy: on the tensor cores through exact digits (k_oz64.cu) where
-// g.ws is given and oz64_takes(g), else on the FP64 pipe.
+// C = alpha A B^T (+ C) within the error bound of an FP64 sum, K 2^-52 sum |a| |b| per output: on the tensor cores
+// through exact digits (k_oz64.cu) where g.ws is given and oz64_takes(g), else on the FP64 pipe.
 int zgemm_fp64(const ZGemm& g, void* stream);
 bool oz64_takes(const ZGemm& g);
 // *done = false: the workspace cannot hold one pair of row tiles (nothing was launched)

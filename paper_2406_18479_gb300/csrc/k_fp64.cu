@@ -333,17 +333,20 @@ inline size_t gj_small_smem(int n) { return (size_t)(n * n + 2 * n + 2) * sizeof
 // panel's step out as one product over the whole matrix (zgemm_oz64),
 //   A += ap W,   W [B][n] = L11^{-1} ak,  ak: the pivot rows, with the identity in the panel's columns
 //                ap [n][B]: -L21 below the pivot rows, -A_panel U11^{-1} above them, U11^{-1} in them
-// after the rows the pivots interchanged have moved and the panel's columns and the pivot rows of A are zero:
-// the pivot rows become D^{-1} A_p (D = L11 U11 the pivot block), the panel -A_panel D^{-1}, its pivot block
-// D^{-1}, the rest A - A_panel D^{-1} A_p. Both triangles are applied by substitution (a thread per row of ap or
-// column of W), never D^{-1} itself: rounding of W then meets multipliers of at most 1 instead of
-// |A_panel| |D^{-1}|, as in an elimination column by column (with D^{-1} the error grows with cond(D): 1e-3
-// instead of 1e-9 for column pairs that differ by 1e-6).
-// The digits of a row share one scale, so the B terms of the product are balanced by exact powers of two: row t
-// of W is brought to about 1 and column t of ap takes its size (without: 2e-7 where five rows of a panel are 1e10
-// times the others).
+// after the rows the pivots interchanged have moved: the pivot rows become D^{-1} A_p (D = L11 U11 the pivot block),
+// the panel -A_panel D^{-1}, the pivot block D^{-1}, the rest A - A_panel D^{-1} A_p. Both triangles are applied
+// by substitution (a thread per row of ap or column of W), never D^{-1}: rounding of W then meets multipliers of at
+// most 1 instead of |A_panel| |D^{-1}|, as in an elimination column by column (with D^{-1} the error grows with
+// cond(D): 1e-3 instead of 1e-9 for column pairs that differ by 1e-6).
+// The digits of a row share one scale. So the B terms of the product are balanced by exact powers of two: row t of W
+// is brought to about 1 and column t of ap takes its size (without: 2e-7 where five rows of a panel are 1e10 times the
+// others). And the triangles keep their diagonals out of it: the panel's column s is L11^{-1} e_s = e_s + small ones,
+// the pivot row r likewise, whose products would meet the small elements of the other operand (a tenth of them left to
+// the FP64 pipe). The diagonal's term, the last kGjTail columns and pivot rows (of few terms), and the pivot block
+// are put into A here; the product adds the rest and spares the block.
 // What bounds the kernel is the chain of a column (search, one division, swap, update: 5 block-wide steps), then
 // the FP64 pipe: B^2/2 complex multiply-adds per row and per column. swp[c]: the row swapped with row c at step c.
+constexpr int kGjTail = 4;
 template <int B>
 size_t gj_panel_smem(int n) {
   return (size_t)n * (B + 1) * sizeof(double2);
@@ -358,7 +361,7 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
   __shared__ int s_p, s_bad, s_cnt;
   __shared__ int s_swp[B], s_row[2 * B], s_src[2 * B];
   __shared__ unsigned int s_max[B];        // largest |re|, |im| of a row of W (leading 32 bits)
-  __shared__ double2 s_inv, s_dinv[B];
+  __shared__ double2 s_inv, s_dinv[B], Ui[B][B + 1];   // U11^{-1}
   double2* M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
   double2* ap = ap_all + (long long)blockIdx.x * B * n;
   double2* W = w_all + (long long)blockIdx.x * B * n;
@@ -484,8 +487,13 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
       for (int t = 0; t < 2 * B; ++t)
         if (t < cnt) v[t] = M[(long long)s_src[t] * n + col];
 #pragma unroll
-      for (int t = 0; t < 2 * B; ++t)
-        if (t < cnt) M[(long long)s_row[t] * n + col] = t < kb ? make_double2(0.0, 0.0) : v[t];
+      for (int t = B; t < 2 * B; ++t)
+        if (t < cnt) M[(long long)s_row[t] * n + col] = v[t];
+      if (kb < B) {
+#pragma unroll
+        for (int t = 0; t < B; ++t)
+          if (t >= kb && t < cnt) M[(long long)s_row[t] * n + col] = v[t];
+      }
     }
 #pragma unroll
     for (int t = 0; t < B; ++t)
@@ -509,13 +517,11 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
     return ex == 0 || ex == 0x7FF ? 0 : max(-kGjBalanceMax, min(kGjBalanceMax, ex - 1022));
   };
   auto pow2 = [](int e) { return __longlong_as_double((long long)(e + 1023) << 52); };
-  for (int e = tid; e < n * kb; e += blockDim.x) {
-    const double2 v = W[e];
-    const double f = pow2(-size_of(e / n));
-    W[e] = make_double2(v.x * f, v.y * f);
-  }
-  // ---- ap: the multipliers below, x U11 = -A_panel (above) or the identity (pivot rows) by substitution
+  const int tail = max(0, kb - kGjTail);
+  // ---- ap: the multipliers below, x U11 = -A_panel (above) or the identity (pivot rows) by substitution; the panel's
+  // part of A: the diagonal's term, all terms of the tail
   for (int i = tid; i < n; i += blockDim.x) {
+    const bool pivot = i >= k0 && i < k0 + kb;
     double2 v[B];
     if (i >= k0 + kb) {
 #pragma unroll
@@ -540,14 +546,54 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
     }
 #pragma unroll
     for (int t = 0; t < B; ++t) {
-      const double f = t < kb ? pow2(size_of(t)) : 0.0;
-      ap[(long long)i * B + t] = t < kb ? make_double2(v[t].x * f, v[t].y * f) : make_double2(0.0, 0.0);
+      const double f = t < kb && !(pivot && (i - k0 >= tail || i - k0 == t)) ? pow2(size_of(t)) : 0.0;
+      ap[(long long)i * B + t] = f != 0.0 ? make_double2(v[t].x * f, v[t].y * f) : make_double2(0.0, 0.0);
+      if (pivot) Ui[i - k0][t] = v[t];
+      if (pivot || t >= kb) continue;
+      double2 x = v[t];
+      if (t >= tail) {
+#pragma unroll
+        for (int s = t + 1; s < min(B, t + kGjTail); ++s)
+          if (s < kb) {
+            const double2 w = W[(long long)s * n + k0 + t];
+            msub(x, make_double2(-v[s].x, -v[s].y), w);
+          }
+      }
+      M[(long long)i * n + k0 + t] = x;
     }
   }
   __syncthreads();
-  for (int e = tid; e < n * B; e += blockDim.x) {
-    const int i = e / B, j = e % B;
-    if (j < kb) M[(long long)i * n + k0 + j] = make_double2(0.0, 0.0);
+  if (tid < kb * kb) {                     // the pivot block D^{-1}
+    const int a = tid / kb, c = tid % kb;
+    double2 v = make_double2(0.0, 0.0);
+    for (int t = max(a, c); t < kb; ++t) {
+      const double2 u = Ui[a][t], w = W[(long long)t * n + k0 + c];
+      msub(v, make_double2(-u.x, -u.y), w);
+    }
+    M[(long long)(k0 + a) * n + k0 + c] = v;
+  }
+  __syncthreads();
+  // ---- W scaled, the panel's diagonal and tail out; the pivot rows of A: the diagonal's term, all terms of the tail
+  for (int col = tid; col < n; col += blockDim.x) {
+    const bool panel = col >= k0 && col < k0 + kb;
+    double2 v[B];
+#pragma unroll
+    for (int t = 0; t < B; ++t)
+      if (t < kb) v[t] = W[(long long)t * n + col];
+#pragma unroll
+    for (int t = 0; t < B; ++t) {
+      if (t >= kb) continue;
+      const double f = panel && (col - k0 == t || col - k0 >= tail) ? 0.0 : pow2(-size_of(t));
+      W[(long long)t * n + col] = f != 0.0 ? make_double2(v[t].x * f, v[t].y * f) : make_double2(0.0, 0.0);
+      if (panel) continue;
+      double2 x = cmul(Ui[t][t], v[t]);
+      if (t >= tail) {
+#pragma unroll
+        for (int s = t + 1; s < min(B, t + kGjTail); ++s)
+          if (s < kb) msub(x, make_double2(-Ui[t][s].x, -Ui[t][s].y), v[s]);
+      }
+      M[(long long)(k0 + t) * n + col] = x;
+    }
   }
 }
 
@@ -1046,6 +1092,8 @@ int inverse_panels(double2* base, int n, long long stride, int nbatch, int* stat
       z.bc.list = l0;
       z.bc.bs_in = stride;
       z.accumulate = 1;
+      z.skip0 = k0;
+      z.skip1 = k0 + kb;
       z.slot = SLOT_INVERSE_FP64;
       z.ws = &rest;
       bool done = false;

@@ -13,9 +13,16 @@
 // element). Digits are exact in bf16. Products of order o = i + j are summed in their own FP32
 // accumulator over at most 128 real k: |sum| <= 8 * 128 * 2^14 = 2^24, exact whatever order the
 // tensor core adds in. The 8 accumulators (o = 0..7; higher orders are below 2^-59) are joined
-// into a 96-bit integer, summed over the chunks of 128 k without rounding, and only the final
-// value is rounded to FP64. The result does not depend on tiling or batching, and its error is
-// below that of a running FP64 sum.
+// into a 96-bit integer, summed over the chunks of 128 k without rounding, and brought to FP64 at the
+// end. The result does not depend on tiling or batching.
+//
+// The error of K complex terms is at most K 2^-58 2^Ep 2^Eq: it goes with the largest elements of the two
+// rows, an FP64 sum's (at most K 2^-52 sum |p| |q|) with the terms. Where the large elements of one row meet
+// the small ones of the other the digits hold too little. So every output has a lower bound
+// S <= sum |p| |q| 2^-(Ep + Eq) made for it (oz64_bound_kernel: one bf16 product of the magnitudes), and those
+// with S < 2^-6 (but not 0: then every term is exactly 0) are left to the FP64 pipe:
+// no output has a larger error bound than an FP64 sum of its terms. Transforms avoid the case through a power of
+// two per k that moves the grading of the matrix's columns into the input (ZGemm::kexp).
 //
 // Bound: the L2 reads of the digit tiles at long K (48 KB per k-step of a 128 x 64 tile, 5.5 TB/s), the
 // epilogue's three FP64 operations an output at short K. 27 TFLOP/s of complex products at long K (R of a
@@ -25,15 +32,16 @@
 // their packing. Error against 64-bit references on these: 2e-16 and 4e-16 (FP64 pipe: 3e-15 and 6e-15).
 //
 // Rows with a non-finite element, or whose scale lies outside 2^+-480 (where the scaled product
-// could over- or underflow), carry a NaN scale. The epilogue leaves outputs that meet one alone, and the CTA
-// computes them on the FP64 pipe after its last tile (plain_tiles), so infinities, NaN and extreme ranges
-// behave as in zgemm_fp64. (A loop over K in the epilogue itself would keep the CTA's other warps in waits that
-// give up after 4 s: reached from K of about 10^6.)
+// could over- or underflow), carry a NaN scale, and outputs that meet one are left as well, so infinities, NaN and
+// extreme ranges behave as in zgemm_fp64. The epilogue leaves an output alone, and the CTA computes it after its last
+// tile (plain_tiles): a loop over K in the epilogue itself would keep the CTA's other warps in waits that give up
+// after 4 s, reached from K of about 10^6.
 //
 // Kernels
 //   oz64_pack_kernel  FP64 views -> digit tiles, in the order the tensor core reads shared memory
 //                     (8-row x 16-byte core matrices, no swizzle): a k-step of a tile is one
 //                     contiguous block, moved by one bulk copy, no tensor map
+//   oz64_bound_kernel the bound S of every output, one bit for each that is left
 //   oz64_gemm_kernel  persistent GEMM, 128 real rows of P x NT rows of Q per tile. The 8 digit
 //                     tiles of Q lie behind one another in N, and the accumulator of order o in
 //                     TMEM columns [o NT, (o + 1) NT): one MMA of digit i of P against the digits
@@ -59,6 +67,11 @@ constexpr int kSegSteps = 8;        // least k-steps of a packing segment
 constexpr int kMaxSegs = 32;
 constexpr int kSplitTiles = 608;    // tiles of a split-K launch, at most (four waves)
 constexpr int kMaxSplit = 16;
+constexpr int kMagTile = 128;       // rows of a tile of magnitudes
+constexpr int kMagK = 16;           // complex k of one of its steps
+constexpr int kMagStep = kMagTile * kMagK * 2;   // bytes of a step
+constexpr float kLeastSum = 0.015625f;           // S below which the digits hold too little
+constexpr int kMapBits = 1024;      // of a CTA's map of units with outputs that are left (a warp's lanes x 32)
 
 // x / d for x < 2^31: multiply-high (see FastDiv in k_mixed.cu)
 struct Div {
@@ -90,11 +103,16 @@ struct Side {
   unsigned char* dst = nullptr;
   double* scale = nullptr;              // per packed row: 2^(E - 34), NaN: no digit form
   unsigned long long* pmax = nullptr;   // segs > 1: largest |value| bits of each row and K segment
+  unsigned char* mag = nullptr;         // magnitudes max(|re|, |im|) 2^-E, bf16 rounded down, steps of 128 rows x 16 k
+  int mtiles = 0;                       // tiles of 128 rows of a packed batch
+  const int* kexp = nullptr;            // element (r, k) counts as x 2^(ksign kexp[k])
+  int ksign = 0;
 };
 
 struct Job {
   Side p, q;
   int K = 0, nks = 0;                   // complex k; k-steps of 16 real k
+  int nms = 0;                          // steps of 16 complex k of the magnitudes
   int segs = 1, seg_steps = 0;          // packing: K segments per row tile, k-steps of one
   int o0 = 0, i0 = 0, no = 1, ni = 1;   // batch range of this launch: bo in [o0, o0 + no), bi likewise
   double2* C = nullptr;
@@ -104,6 +122,7 @@ struct Job {
   Div cp_div, cq_div;
   double alpha = 1.0;
   int accumulate = 0;
+  int skip0 = 0, skip1 = 0;             // outputs with both indices in [skip0, skip1) are not written
   // split K: ksplit CTAs share a tile, each summing split_chunks chunks; their 96-bit integers meet in
   // part ([tile][split][column][128 lanes], hi and lo apart), and the last to arrive (a counter per
   // tile and epilogue warp) adds them, exactly, and writes the output
@@ -111,6 +130,7 @@ struct Job {
   long long* part_hi = nullptr;
   uint32_t* part_lo = nullptr;
   unsigned int* counter = nullptr;
+  uint32_t* left = nullptr;             // [tile][64 rows of P][NT / 32]: bit c: column c is left to plain_tiles
   int* status = nullptr;
 };
 
@@ -129,6 +149,16 @@ __device__ __forceinline__ const double2* side_base(const Side& s, int bo, int b
   return s.src + batch_in(s.b, bi) + (long long)bo * s.b.bs_out;
 }
 
+template <bool KX>
+__device__ __forceinline__ double2 side_elem(const Side& s, const double2* row, int k) {
+  double2 x = row[side_k(s, k)];
+  if (KX) {
+    const double f = __longlong_as_double((long long)(1023 + s.ksign * s.kexp[k]) << 52);
+    x = make_double2(x.x * f, x.y * f);
+  }
+  return x;
+}
+
 // round(x 2^(62 - E)) + 0x80..80 for |x| < 2^E: byte 7 - i of the result is digit i plus 128
 __device__ __forceinline__ unsigned long long digits_of(double x, int E) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
@@ -140,6 +170,14 @@ __device__ __forceinline__ unsigned long long digits_of(double x, int E) {
   else n = sh > 54 ? 0ull : (m + (1ull << (sh - 1))) >> sh;
   const unsigned long long neg = (unsigned long long)((long long)bits >> 63);
   return ((n ^ neg) - neg) + 0x8080808080808080ull;
+}
+
+// max(|re|, |im|) 2^-E < 1 as bf16, rounded down, from the leading words of digits_of; what is below 2^-22 but not
+// zero counts as 2^-60, so that a sum of products is zero only where every product is
+__device__ __forceinline__ uint32_t magnitude(double2 x, unsigned long long re, unsigned long long im) {
+  const int a = abs((int)((uint32_t)(re >> 32) - 0x80808080u)), b = abs((int)((uint32_t)(im >> 32) - 0x80808080u));
+  const float m = __int2float_rz(max(a, b)) * 9.313225746154785e-10f;     // 2^-30
+  return max(a, b) >= 256 ? __float_as_uint(m) >> 16 : x.x != 0.0 || x.y != 0.0 ? 67u << 7 : 0u;
 }
 
 // digit j (0: leading) of four words as two bf16 pairs
@@ -182,7 +220,7 @@ struct PackPos {
   }
 };
 
-template <int kRows>
+template <int kRows, bool KX>
 __device__ __forceinline__ unsigned long long row_max(const Side& s, const Job& j, const PackPos<kRows>& p) {
   constexpr int kGroups = 256 / kRows;
   unsigned long long mx = 0;
@@ -192,7 +230,7 @@ __device__ __forceinline__ unsigned long long row_max(const Side& s, const Job& 
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         if (k + u >= kend) break;
-        const double2 x = p.src[side_k(s, k + u)];
+        const double2 x = side_elem<KX>(s, p.src, k + u);
         mx = max(mx, max((unsigned long long)__double_as_longlong(x.x) & 0x7FFFFFFFFFFFFFFFull,
                          (unsigned long long)__double_as_longlong(x.y) & 0x7FFFFFFFFFFFFFFFull));
       }
@@ -206,14 +244,14 @@ __device__ __forceinline__ unsigned long long row_max(const Side& s, const Job& 
   return mx;
 }
 
-template <int kRows>
+template <int kRows, bool KX>
 __device__ void scale_tile(const Side& s, const Job& j, long long t) {
   const PackPos<kRows> p(s, j, t);
-  const unsigned long long mx = row_max<kRows>(s, j, p);
+  const unsigned long long mx = row_max<kRows, KX>(s, j, p);
   if (p.grp == 0) s.pmax[p.prow * j.segs + p.seg] = mx;
 }
 
-template <int RT, bool PSIDE>
+template <int RT, bool PSIDE, bool KX>
 __device__ void pack_tile(const Side& s, const Job& j, long long t) {
   constexpr int kRows = PSIDE ? kPTile : RT;      // complex rows of the tile
   constexpr int kReal = PSIDE ? 2 * kPTile : RT;  // real rows of the tile
@@ -221,7 +259,7 @@ __device__ void pack_tile(const Side& s, const Job& j, long long t) {
   const PackPos<kRows> p(s, j, t);
   unsigned long long mx = 0;
   if (j.segs == 1) {
-    mx = row_max<kRows>(s, j, p);
+    mx = row_max<kRows, KX>(s, j, p);
   } else {
     for (int g = 0; g < j.segs; ++g) mx = max(mx, s.pmax[p.prow * j.segs + g]);
   }
@@ -237,16 +275,24 @@ __device__ void pack_tile(const Side& s, const Job& j, long long t) {
   const int rr = PSIDE ? 2 * p.row : p.row;
   // the padding rows of the last tile stay unwritten: a row of digits meets only its own row of the output
   if (!p.row_ok) return;
+  const int mrow = p.tile * kRows + p.row;
+  unsigned char* mag = s.mag + ((long long)p.pb * s.mtiles + mrow / kMagTile) * j.nms * (long long)kMagStep +
+                       (mrow % kMagTile >> 3) * 256 + (mrow & 7) * 16;
+  auto mag_at = [&](int g) { return reinterpret_cast<uint2*>(mag + (long long)(g >> 2) * kMagStep + (g >> 1 & 1) * 128 + (g & 1) * 8); };
+  if (p.k1 == j.nks && (j.nks & 1) && p.grp < 2) *mag_at(2 * j.nks + p.grp) = make_uint2(0u, 0u);   // half a step beyond K
   for (int g = 2 * p.k0 + p.grp; g < 2 * p.k1; g += kGroups) {
     unsigned long long u[8];
+    uint32_t m[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int k = 4 * g + c;
       double2 x = make_double2(0.0, 0.0);
-      if (!zero && k < j.K) x = p.src[side_k(s, k)];
+      if (!zero && k < j.K) x = side_elem<KX>(s, p.src, k);
       u[2 * c] = digits_of(x.x, E);
       u[2 * c + 1] = digits_of(x.y, E);
+      m[c] = magnitude(x, u[2 * c], u[2 * c + 1]);
     }
+    *mag_at(g) = make_uint2(m[0] | m[1] << 16, m[2] | m[3] << 16);
     unsigned char* d = base + (long long)(g >> 1) * (kDigits * kReal * 32) + (rr >> 3) * 256 + (g & 1) * 128 +
                        (rr & 7) * 16;
 #pragma unroll
@@ -266,36 +312,48 @@ __device__ void pack_tile(const Side& s, const Job& j, long long t) {
   }
 }
 
-template <int NT>
+template <int NT, bool KX>
 __global__ void __launch_bounds__(256) oz64_scale_kernel(const __grid_constant__ Job j) {
   const long long np = (long long)j.p.tiles * j.p.no * j.p.ni * j.segs;
-  if (blockIdx.x < np) scale_tile<kPTile>(j.p, j, blockIdx.x);
-  else scale_tile<NT>(j.q, j, blockIdx.x - np);
+  if (blockIdx.x < np) scale_tile<kPTile, KX>(j.p, j, blockIdx.x);
+  else scale_tile<NT, KX>(j.q, j, blockIdx.x - np);
 }
 
-template <int NT>
+template <int NT, bool KX>
 __global__ void __launch_bounds__(256) oz64_pack_kernel(const __grid_constant__ Job j) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const long long np = (long long)j.p.tiles * j.p.no * j.p.ni * j.segs;
-  if (blockIdx.x < np) pack_tile<2 * kPTile, true>(j.p, j, blockIdx.x);
-  else pack_tile<NT, false>(j.q, j, blockIdx.x - np);
+  if (blockIdx.x < np) pack_tile<2 * kPTile, true, KX>(j.p, j, blockIdx.x);
+  else pack_tile<NT, false, KX>(j.q, j, blockIdx.x - np);
 }
 
-// The outputs of this CTA's tiles that the digits do not give: a group of 256 threads per 32 x 32 complex outputs, the
+// bits of the columns c, c + 1, .. (n <= 32) within [skip0, skip1)
+__device__ __forceinline__ uint32_t skip_bits(const Job& j, int c, int n) {
+  const int lo = min(max(j.skip0 - c, 0), n), hi = min(max(j.skip1 - c, 0), n);
+  return (uint32_t)((1ull << hi) - (1ull << lo));
+}
+
+// The outputs of this CTA's tiles that are left to the FP64 pipe: a group of 256 threads per 32 x 32 complex outputs, the
 // terms in order of k on the FP64 pipe as in zgemm_fp64_kernel. A thread has 2 x 2 outputs and a warp skips those that
 // none of its lanes needs, so a few of them cost the staging of their operands and little arithmetic. Of CTAs that share
 // a tile's K the first takes it. sm: the group's 2 kPlainK rows of 33 elements and the masks.
 constexpr int kPlainK = 16, kPlainGroups = kEpiWarps / 8;
 constexpr size_t kPlainSmem = 2 * kPlainK * 33 * sizeof(double2) + 256;   // of a group
 template <int NT>
-__device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, int group, int tid, unsigned char* sm) {
+__device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, const uint32_t* map, int map_sh, int group, int tid,
+                                            unsigned char* sm) {
   double2(*Ps)[33] = reinterpret_cast<double2(*)[33]>(sm);
   double2(*Qs)[33] = Ps + kPlainK;
-  uint32_t* s_row = reinterpret_cast<uint32_t*>(Qs + kPlainK);          // rows of P, rows of Q without a digit form
+  uint32_t* s_left = reinterpret_cast<uint32_t*>(Qs + kPlainK);         // left columns of each row; whether any
   auto sync = [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + group) : "memory"); };
   constexpr int kSub = 2 * (NT / 32);                 // 32 x 32 pieces of a GEMM tile
   const int per_batch = j.p.tiles * j.q.tiles, total = per_batch * j.no * j.ni * ksplit;
   const int tx = tid & 15, ty = tid >> 4;
-  for (int unit = blockIdx.x; unit < total; unit += gridDim.x) {
+  int own = 0;
+#pragma unroll 1
+  for (int unit = blockIdx.x; unit < total; unit += gridDim.x, ++own) {
+    if (!(map[own >> map_sh >> 5] >> (own >> map_sh & 31) & 1)) continue;
     const int tile = unit / ksplit;
     if (unit != tile * ksplit) continue;
     const int b = tile / per_batch, w = tile - b * per_batch, o = b / j.ni, i = b - o * j.ni;
@@ -306,16 +364,13 @@ __device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, int group,
       const int np = min(32, j.p.rows - pt * kPTile - p0), nq = min(32, j.q.rows - qt * NT - q0);
       if (np <= 0 || nq <= 0) continue;
       sync();
-      if (tid < 64) {
-        const Side& s = tid < 32 ? j.p : j.q;
-        const long long at = (((long long)(s.dep_o ? o : 0) * s.ni + (s.dep_i ? i : 0)) * s.tiles + (tid < 32 ? pt : qt)) *
-                             (tid < 32 ? kPTile : NT) + (tid < 32 ? p0 : q0) + (tid & 31);
-        const uint32_t m = __ballot_sync(0xffffffffu, isnan(s.scale[at]));
-        if ((tid & 31) == 0) s_row[tid >> 5] = m;
+      if (tid < 32) {
+        s_left[tid] = tid < np ? j.left[((long long)tile * kPTile + p0 + tid) * (NT / 32) + q0 / 32] : 0u;
+        const bool any = __any_sync(0xffffffffu, s_left[tid] != 0);
+        if (tid == 0) s_left[32] = any;
       }
       sync();
-      const uint32_t rows = s_row[0] & (np < 32 ? (1u << np) - 1 : ~0u), cols = s_row[1] & (nq < 32 ? (1u << nq) - 1 : ~0u);
-      if ((rows | cols) == 0) continue;
+      if (!s_left[32]) continue;
       bool need[2][2];
       double2 acc[2][2];
 #pragma unroll
@@ -323,7 +378,7 @@ __device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, int group,
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
           const int r = 2 * tx + u, c = 2 * ty + v;
-          need[u][v] = r < np && c < nq && (((rows >> r) | (cols >> c)) & 1);
+          need[u][v] = s_left[r] >> c & 1;
           acc[u][v] = make_double2(0.0, 0.0);
         }
       const int bo = j.o0 + o, bi = j.i0 + i;
@@ -388,7 +443,7 @@ struct Oz64Shape {
   static constexpr int kBufCols = kDigits * NT;
   static constexpr int kBufs = 512 / kBufCols;                  // accumulator sets in TMEM
   static constexpr int kThreads = 64 + 32 * kEpiWarps;          // producer, MMA, epilogue warps
-  static constexpr size_t kSmem = 128 + (size_t)kStages * kStageBytes + 256;
+  static constexpr size_t kSmem = 128 + (size_t)kStages * kStageBytes + 512;
   static_assert(kSmem <= 232448, "stages exceed shared memory");
   static_assert(kPlainGroups * kPlainSmem <= (size_t)kStages * kStageBytes, "plain_tiles works in the stages");
 };
@@ -461,6 +516,193 @@ __device__ __forceinline__ double to_fp64(long long hi, uint32_t lo, int e) {
   return __longlong_as_double((long long)((((unsigned long long)(E - 1) << 52) + m) | ((unsigned long long)neg & (1ull << 63))));
 }
 
+// S of every output: magnitudes of 128 rows of P times 128 rows of Q, summed over K in one FP32 accumulator (truncated,
+// so from below), two tiles in flight. Long K in two passes: 512 of its k spread evenly, which is enough for every output
+// of most tiles, then all of it for the other tiles (P0 of a 2x2x2 solid, 13 tiles of K = 5408: 50 us for all of it).
+// Bound: launch and copy latency; 1/70 of the digit MMAs and 1/30 of their bytes, and one load and compare an output.
+constexpr int kMagStages = 3, kMagPer = 4;           // stages, steps of a stage
+constexpr int kMagFirst = 8;                         // stages of a first pass (512 k)
+constexpr int kMagThreads = 192;                     // producer, MMA, four epilogue warps
+constexpr size_t kMagSmem = 128 + (size_t)kMagStages * kMagPer * 2 * kMagStep + 384;
+template <int NT>
+__global__ void __launch_bounds__(kMagThreads) oz64_bound_kernel(const __grid_constant__ Job j) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+  constexpr int kHalf = kMagPer * kMagStep;          // P's part of a stage
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)kMagStages * 2 * kHalf);
+  uint64_t* empty = full + kMagStages;
+  uint64_t* acc_full = empty + kMagStages;           // [2]
+  uint64_t* acc_empty = acc_full + 2;
+  uint64_t* drain_bar = acc_full + 4;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 5);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  uint32_t* map = tmem_slot + 2;                     // tiles for a second pass, as in oz64_gemm_kernel
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kMagStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], 4);
+    }
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 2) map[lane] = 0;
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(256));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the packing
+  const int per_batch = j.p.mtiles * j.q.mtiles, total = per_batch * j.no * j.ni;
+  auto packed = [](const Side& s, int b, int ni) {
+    const int o = b / ni, i = b - o * ni;
+    return (s.dep_o ? o : 0) * s.ni + (s.dep_i ? i : 0);
+  };
+  const int nstages = (j.nms + kMagPer - 1) / kMagPer;
+  const int npass = nstages > kMagFirst ? 2 : 1;
+  int map_sh = 0;
+  while ((total / (int)gridDim.x) >> map_sh >= kMapBits) ++map_sh;
+  uint32_t step = 0, n = 0;           // stages and tiles so far (of a role)
+  bool ok = true;
+#pragma unroll 1
+  for (int pass = 0; pass < npass; ++pass) {
+    // the stages of this pass: all, or kMagFirst spread over K
+    const int ns = npass == 2 && pass == 0 ? kMagFirst : nstages;
+    auto stage_at = [&](int s) { return ns == nstages ? s : (int)((long long)s * (nstages - 1) / (kMagFirst - 1)); };
+    auto steps_of = [&](int s) { return min(kMagPer, j.nms - s * kMagPer); };
+    if (warp == 0) {
+      if (lane == 0) {
+        int own = 0;
+        for (int tile = blockIdx.x; tile < total && !*abort_flag; tile += gridDim.x, ++own) {
+          if (pass && !(map[own >> map_sh >> 5] >> (own >> map_sh & 31) & 1)) continue;
+          const int b = tile / per_batch, w = tile - b * per_batch, pt = w / j.q.mtiles, qt = w - pt * j.q.mtiles;
+          const unsigned char* a = j.p.mag + ((long long)packed(j.p, b, j.ni) * j.p.mtiles + pt) * j.nms * (long long)kMagStep;
+          const unsigned char* q = j.q.mag + ((long long)packed(j.q, b, j.ni) * j.q.mtiles + qt) * j.nms * (long long)kMagStep;
+          const uint32_t pb = min(kMagTile, (j.p.rows - pt * kMagTile + 7) / 8 * 8) * (2 * kMagK);   // bytes of a step that hold rows
+          const uint32_t qb = min(kMagTile, (j.q.rows - qt * kMagTile + 7) / 8 * 8) * (2 * kMagK);
+          for (int i = 0; i < ns; ++i, ++step) {
+            const int st = step % kMagStages, s = stage_at(i), nk = steps_of(s);
+            if (!mbar_wait(&empty[st], ((step / kMagStages) & 1) ^ 1, abort_flag, j.status, 25)) break;
+            uint8_t* sa = smem + (size_t)st * 2 * kHalf;
+            mbar_expect_tx(&full[st], nk * (pb + qb));
+            if (pb + qb == 2 * kMagStep) {
+              bulk_load(sa, a + (long long)s * kHalf, nk * kMagStep, &full[st]);
+              bulk_load(sa + kHalf, q + (long long)s * kHalf, nk * kMagStep, &full[st]);
+            } else {     // only the 8-row groups that hold rows (small matrices: a quarter of the reads)
+              for (int k = 0; k < nk; ++k) {
+                bulk_load(sa + k * kMagStep, a + (long long)s * kHalf + k * kMagStep, pb, &full[st]);
+                bulk_load(sa + kHalf + k * kMagStep, q + (long long)s * kHalf + k * kMagStep, qb, &full[st]);
+              }
+            }
+          }
+        }
+      }
+    } else if (warp == 1) {
+      if (lane == 0) {
+        const uint64_t desc0 = core_desc(smem_u32(smem));
+        int own = 0;
+        for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x, ++own) {
+          if (pass && !(map[own >> map_sh >> 5] >> (own >> map_sh & 31) & 1)) continue;
+          const uint32_t buf = n & 1;
+          if (!mbar_wait(&acc_empty[buf], ((n >> 1) & 1) ^ 1, abort_flag, j.status, 26)) { ok = false; break; }
+          ++n;
+          tc_fence_after();
+          for (int i = 0; i < ns; ++i, ++step) {
+            const int st = step % kMagStages, nk = steps_of(stage_at(i));
+            if (!mbar_wait(&full[st], (step / kMagStages) & 1, abort_flag, j.status, 27)) { ok = false; break; }
+            tc_fence_after();
+            const uint64_t sa = desc0 + (uint64_t)((st * 2 * kHalf) >> 4);
+            for (int k = 0; k < nk; ++k)
+              mma_bf16(tmem + buf * kMagTile, sa + (uint64_t)(k * kMagStep >> 4), sa + (uint64_t)((kHalf + k * kMagStep) >> 4),
+                       idesc_bf16(kMagTile, false), i == 0 && k == 0 ? 0u : 1u);
+            mma_commit(&empty[st]);
+          }
+          if (ok) mma_commit(&acc_full[buf]);
+        }
+      }
+    } else {
+      const int quarter = warp & 3;
+      int own = 0;
+      for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x, ++own) {
+        if (pass && !(map[own >> map_sh >> 5] >> (own >> map_sh & 31) & 1)) continue;
+        const int b = tile / per_batch, w = tile - b * per_batch, pt = w / j.q.mtiles, qt = w - pt * j.q.mtiles;
+        const int r = pt * kMagTile + quarter * 32 + lane;
+        const bool row_ok = r < j.p.rows;
+        const bool row_bad = row_ok && isnan(j.p.scale[(long long)packed(j.p, b, j.ni) * j.p.tiles * kPTile + r]);
+        const double* sq = j.q.scale + (long long)packed(j.q, b, j.ni) * j.q.tiles * NT;
+        uint32_t* left = j.left + ((long long)(b * j.p.tiles + r / kPTile) * j.q.tiles * kPTile + r % kPTile) * (NT / 32);
+        uint32_t bad[kMagTile / 32], in[kMagTile / 32];   // columns without a digit form, columns there are
+#pragma unroll
+        for (int g = 0; g < kMagTile / 32; ++g) {
+          const int c = qt * kMagTile + g * 32 + lane;
+          in[g] = __ballot_sync(0xffffffffu, c < j.q.rows);
+          bad[g] = __ballot_sync(0xffffffffu, c < j.q.rows && isnan(sq[c]));
+        }
+        const uint32_t buf = n & 1;
+        if (!mbar_wait(&acc_full[buf], (n >> 1) & 1, abort_flag, j.status, 28)) { ok = false; break; }
+        ++n;
+        tc_fence_after();
+        bool again = false;               // below the bound with part of K
+#pragma unroll
+        for (int g = 0; g < kMagTile / 32; ++g) {
+          float v[32];
+#pragma unroll
+          for (int u = 0; u < 32; u += 8) tmem_ld8(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kMagTile + g * 32 + u, v + u);
+          tmem_wait_ld();
+          if (g == kMagTile / 32 - 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+          }
+          const int c0 = qt * kMagTile + g * 32;
+          uint32_t m = 0, z = 0;
+#pragma unroll
+          for (int u = 0; u < 32; ++u) {
+            m |= (v[u] < kLeastSum ? 1u : 0u) << u;
+            z |= (v[u] == 0.0f ? 1u : 0u) << u;
+          }
+          again |= (row_ok && !row_bad ? m & ~bad[g] & in[g] : 0u) != 0;
+          m = (row_bad ? ~0u : (m & ~z) | bad[g]) & in[g];
+          if (j.p.row0 + r >= j.skip0 && j.p.row0 + r < j.skip1) m &= ~skip_bits(j, j.q.row0 + c0, 32);
+          if (row_ok && c0 < j.q.tiles * NT)
+            left[(long long)(c0 / NT) * kPTile * (NT / 32) + (c0 % NT) / 32] = m;
+        }
+        if (ns < nstages && __any_sync(0xffffffffu, again) && lane == 0) atomicOr(&map[own >> map_sh >> 5], 1u << (own >> map_sh & 31));
+      }
+    }
+    __syncthreads();
+  }
+  if (warp == 0 && lane == 0 && *abort_flag) {   // let every issued copy land before the CTA exits (bounded)
+    const uint64_t t0 = globaltimer();
+    for (int k = 0; k < kMagStages && step > (uint32_t)k; ++k) {
+      const uint32_t s2 = step - 1 - k;
+      while (!mbar_try(&full[s2 % kMagStages], (s2 / kMagStages) & 1) && globaltimer() - t0 < kWaitLimitNs) {
+      }
+    }
+  }
+  if (warp == 1 && lane == 0) {
+    mma_commit(drain_bar);   // the last MMAs end before TMEM is released
+    const uint64_t t0 = globaltimer();
+    while (!mbar_try(drain_bar, 0) && globaltimer() - t0 < kWaitLimitNs) {
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
+}
+
 template <int NT, bool MULTI>
 __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const __grid_constant__ Job j) {
   using S = Oz64Shape<NT>;
@@ -473,7 +715,8 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
   uint64_t* drain_bar = acc_full + 4;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* plain_flag = abort_flag + 1;    // some output of this CTA's tiles is left to plain_tiles
+  // which of this CTA's units have outputs that are left to plain_tiles: a bit for 2^map_sh units in order
+  uint32_t* map = tmem_slot + 2;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -487,10 +730,10 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
-    *plain_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (warp == 2) map[lane] = 0;
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(512));
@@ -500,9 +743,12 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the bounds (and the packing, which they wait for)
   const int per_batch = j.p.tiles * j.q.tiles;
   const int ksplit = MULTI ? j.ksplit : 1;
   const int total = per_batch * j.no * j.ni * ksplit;
+  int map_sh = 0;
+  while ((total / (int)gridDim.x) >> map_sh >= kMapBits) ++map_sh;
   // work unit -> batch, P tile, Q tile (Q fastest: neighbouring CTAs share the larger P tile in L2),
   // and its k-steps [s0, s1)
   auto split = [&](int unit, int& o, int& i, int& pt, int& qt, int& s0, int& s1) {
@@ -600,14 +846,20 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
     const int lrow = quarter * 32 + lane;
     const int part = lrow & 1;
     uint32_t chunk = 0;
-    for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
+    int own = 0;
+    // this warp's columns of the row that are left to plain_tiles, read a unit ahead
+    auto left_at = [&](int tile) {
+      return j.left[((long long)(MULTI ? tile / ksplit : tile) * kPTile + (lrow >> 1)) * (NT / 32) + half * kCols / 32];
+    };
+    uint32_t left_next = blockIdx.x < total ? left_at(blockIdx.x) : 0u;
+    for (int tile = blockIdx.x; tile < total; tile += gridDim.x, ++own) {
       int o, i, pt, qt, s0, s1;
       split(tile, o, i, pt, qt, s0, s1);
       const int nchunks = (s1 - s0 + kChunkSteps - 1) / kChunkSteps;
       const int bo = j.o0 + o, bi = j.i0 + i;
       const int pr = pt * kPTile + (lrow >> 1);
       const bool p_ok = pr < j.p.rows;
-      // biased exponents of the scales (0x7FF: a row without a digit form)
+      // biased exponents of the scales
       const int ep = __double2hiint(j.p.scale[((long long)packed(j.p, o, i) * j.p.tiles + pt) * kPTile + (lrow >> 1)]) >> 20;
       const double* sq = j.q.scale + ((long long)packed(j.q, o, i) * j.q.tiles + qt) * NT;
       const int ap = j.p.row0 + (p_ok ? pr : 0), apq = div_by(ap, j.cp_div);
@@ -619,15 +871,17 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
         return C + 2 * ((long long)aqq * j.cq_out + (long long)(aq - aqq * j.cq_div.d) * j.cq_in);
       };
       auto col_ok = [&](int col) { return p_ok && qt * NT + col < j.q.rows; };
-      if (ep == 0x7FF || (lane < kCols && qt * NT + half * kCols + lane < j.q.rows && isnan(sq[half * kCols + lane]))) *plain_flag = 1;
+      uint32_t left = left_next >> (half * kCols % 32) & ((1u << kCols) - 1);
+      if (tile + (int)gridDim.x < total) left_next = left_at(tile + gridDim.x);
+      const bool mark = p_ok && left;
+      if (!MULTI && j.p.row0 + pr >= j.skip0 && j.p.row0 + pr < j.skip1) left |= skip_bits(j, j.q.row0 + qt * NT + half * kCols, kCols);
       const bool quick = j.nks <= kFinishSteps;
       auto put = [&](int col, long long hi, long long lo, double old) {
         const int eq = col_ok(col) ? __double2hiint(sq[col]) >> 20 : 1023;
-        const bool plain = ep == 0x7FF || eq == 0x7FF;
-        const int e = plain ? 0 : ep + eq - 2046;
+        const int e = ep + eq - 2046;
         const double x = !MULTI || quick ? finish(hi, lo, e, j.alpha, old)
                                          : fma(to_fp64(hi, (uint32_t)lo, e), j.alpha, old);
-        if (col_ok(col) && !plain) *at(col) = x;
+        if (col_ok(col) && !(left >> (col - half * kCols) & 1)) *at(col) = x;
       };
       // outputs that are added to are read ahead of the wait for the accumulators (a load behind every
       // store would put 16 memory latencies in a row: 24k clocks a tile instead of 5k)
@@ -690,6 +944,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
             n = atomicAdd(&j.counter[t * kEpiWarps + warp - 2], 1u);
             if (n == (unsigned)ksplit - 1) j.counter[t * kEpiWarps + warp - 2] = 0;   // ready for the next launch
           }
+          if (me == 0 && __any_sync(0xffffffffu, mark) && lane == 0) atomicOr(&map[own >> map_sh >> 5], 1u << (own >> map_sh & 31));
           if (__shfl_sync(0xffffffffu, n, 0) != (unsigned)ksplit - 1) continue;
           __threadfence();
           for (int m = 0; m < ksplit; ++m) {
@@ -715,15 +970,16 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
           for (int u = 0; u < 4; ++u) put(half * kCols + u0 + u, hi[u0 + u], lo[u0 + u], o4[u]);
         }
       }
+      if (__any_sync(0xffffffffu, mark) && lane == 0) atomicOr(&map[own >> map_sh >> 5], 1u << (own >> map_sh & 31));
     }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
-  if (*plain_flag && !*abort_flag && warp >= 2) {
+  if (!*abort_flag && warp >= 2) {
     const int t = threadIdx.x - 64;
-    plain_tiles<NT>(j, ksplit, t >> 8, t & 255, smem + (t >> 8) * kPlainSmem);
+    plain_tiles<NT>(j, ksplit, map, map_sh, t >> 8, t & 255, smem + (t >> 8) * kPlainSmem);
   }
 }
 
@@ -737,25 +993,55 @@ int sm_count() {
   return n;
 }
 
+// Launch whose blocks may start while the kernel before it ends (its launch latency, TMEM allocation and barriers
+// under that kernel's tail); they wait for it (griddepcontrol.wait) before they touch memory. A small evaluation
+// (nao = 8, 8 products): 384 -> 353 us.
+template <class... A>
+void launch_after(void (*k)(A...), long long grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+template <int NT, bool KX>
+void launch_pack(const Job& j, long long np, long long nq, cudaStream_t st) {
+  if (j.segs > 1) {
+    prof_begin(SLOT_LIMBS, st);
+    oz64_scale_kernel<NT, KX><<<(unsigned)((np + nq) * j.segs), 256, 0, st>>>(j);
+    prof_end(SLOT_LIMBS, st, 0.0, ((double)np * kPTile + (double)nq * NT) * 16.0 * j.K);
+  }
+  prof_begin(SLOT_LIMBS, st);
+  oz64_pack_kernel<NT, KX><<<(unsigned)((np + nq) * j.segs), 256, 0, st>>>(j);
+  prof_end(SLOT_LIMBS, st, 0.0, ((double)np * kPTile * (32.0 + 64.0) + (double)nq * NT * (32.0 + 32.0)) * 8.0 * j.nks);
+}
+
 template <int NT, bool MULTI>
 int launch_gemm(const Job& j, int slot, cudaStream_t st) {
   using S = Oz64Shape<NT>;
   static const bool attr = cudaFuncSetAttribute(oz64_gemm_kernel<NT, MULTI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)S::kSmem) == cudaSuccess;
+                                                (int)S::kSmem) == cudaSuccess &&
+                           cudaFuncSetAttribute(oz64_bound_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)kMagSmem) == cudaSuccess;
   if (!attr) return fail(GW_ECUDA, "oz64_gemm: shared memory attribute refused");
   const long long total = (long long)j.p.tiles * j.q.tiles * j.no * j.ni * j.ksplit;
   const long long np = (long long)j.p.tiles * j.p.no * j.p.ni, nq = (long long)j.q.tiles * j.q.no * j.q.ni;
   if (total > 2147483647LL || (np + nq) * j.segs > 2147483647LL) return fail(GW_EINVAL, "oz64_gemm: too many tiles");
-  if (j.segs > 1) {
-    prof_begin(SLOT_LIMBS, st);
-    oz64_scale_kernel<NT><<<(unsigned)((np + nq) * j.segs), 256, 0, st>>>(j);
-    prof_end(SLOT_LIMBS, st, 0.0, ((double)np * kPTile + (double)nq * NT) * 16.0 * j.K);
-  }
+  if (j.p.kexp) launch_pack<NT, true>(j, np, nq, st);
+  else launch_pack<NT, false>(j, np, nq, st);
+  const long long mags = (long long)j.p.mtiles * j.q.mtiles * j.no * j.ni;
   prof_begin(SLOT_LIMBS, st);
-  oz64_pack_kernel<NT><<<(unsigned)((np + nq) * j.segs), 256, 0, st>>>(j);
-  prof_end(SLOT_LIMBS, st, 0.0, ((double)np * kPTile * (32.0 + 64.0) + (double)nq * NT * (32.0 + 32.0)) * 8.0 * j.nks);
+  launch_after(oz64_bound_kernel<NT>, std::min<long long>(mags, 2LL * sm_count()), kMagThreads, kMagSmem, st, j);
+  prof_end(SLOT_LIMBS, st, 0.0, (double)mags * j.nms * 2 * kMagStep);
   prof_begin(slot, st);
-  oz64_gemm_kernel<NT, MULTI><<<(int)std::min<long long>(total, sm_count()), S::kThreads, S::kSmem, st>>>(j);
+  launch_after(oz64_gemm_kernel<NT, MULTI>, std::min<long long>(total, sm_count()), S::kThreads, S::kSmem, st, j);
   // algorithmic flops: 8 per complex multiply-add
   prof_end(slot, st, 8.0 * j.p.rows * (double)j.q.rows * j.K * j.no * j.ni,
            (double)total / j.ksplit * j.nks * S::kStageBytes);
@@ -786,9 +1072,10 @@ size_t oz64_counter_bytes() { return (size_t)kSplitTiles * kEpiWarps * sizeof(un
 
 size_t oz64_bytes(long long p_rows, long long q_rows, int K) {
   const long long nks = (K + 7) / 8;
-  // digit tiles (64-row Q tiles bound the padding) and scales
-  const long long extra = 8 + (nks >= 2 * kSegSteps ? 8 * kMaxSegs : 0);
-  return (size_t)(up(p_rows, kPTile) * (nks * 512 + extra) + up(q_rows, 64) * (nks * 256 + extra) + 1024);
+  // digit tiles (64-row Q tiles bound the padding) and scales; magnitudes; a bit for every output
+  const long long extra = 8 + (nks >= 2 * kSegSteps ? 8 * kMaxSegs : 0), mag = (nks + 1) / 2 * 2 * kMagK;
+  return (size_t)(up(p_rows, kPTile) * (nks * 512 + extra) + up(q_rows, 64) * (nks * 256 + extra) +
+                  (up(p_rows, kMagTile) + up(q_rows, kMagTile)) * mag + up(p_rows, kPTile) * up(q_rows, 64) / 8 + 1024);
 }
 
 // Where digits pay: below 8 complex k most of a k-step is padding, and tiny products (under 2^13
@@ -809,13 +1096,22 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
   Job j;
   j.p = p_is_b ? make_side(g.B, g.vb, g.bb, no, ni) : make_side(g.A, g.va, g.ba, no, ni);
   j.q = p_is_b ? make_side(g.A, g.va, g.ba, no, ni) : make_side(g.B, g.vb, g.bb, no, ni);
+  if (g.kexp) {
+    j.p.kexp = j.q.kexp = g.kexp;
+    j.p.ksign = p_is_b ? 1 : -1;
+    j.q.ksign = -j.p.ksign;
+  }
   const int pr = p_is_b ? g.N : g.M, qr = p_is_b ? g.M : g.N;
   j.K = g.K;
   j.nks = (g.K + 7) / 8;
+  j.nms = (j.nks + 1) / 2;
   j.C = g.C;
   j.bc = g.bc;
   j.alpha = g.alpha;
   j.accumulate = g.accumulate;
+  j.skip0 = g.skip0;
+  j.skip1 = g.skip1;
+  if (g.skip1 > g.skip0 && j.nks > kChunkSteps) return fail(GW_EINVAL, "oz64_gemm: a block of outputs is spared in products of one chunk");
   j.status = g.ws->status;
   const Div rd = make_div(g.vc.rin), kd = make_div(g.vc.kin);
   j.cp_div = p_is_b ? kd : rd;
@@ -829,19 +1125,23 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
   const int nt = (j.nks > 2 * kChunkSteps && up(qr, 64) == up(qr, 32)) ? 64 : 32;
   // bytes per packed row: digits, scale, and the segment maxima of long rows
   const long long row_extra = 8 + (j.nks >= 2 * kSegSteps ? 8 * kMaxSegs : 0);
-  const long long pb = (long long)j.nks * 512 + row_extra, qb = (long long)j.nks * 256 + row_extra;
+  const long long pb = (long long)j.nks * 512 + row_extra, qb = (long long)j.nks * 256 + row_extra, mb = j.nms * 2LL * kMagK;
   const long long W = (long long)g.ws->bytes - 1024;
+  auto p_bytes = [&](long long r) { return up(r, kPTile) * pb + up(r, kMagTile) * mb; };
+  auto q_bytes = [&](long long r) { return up(r, nt) * qb + up(r, kMagTile) * mb; };
   auto need = [&](long long prow, long long qrow, long long o, long long i) {
-    return up(prow, kPTile) * pb * (j.p.dep_o ? o : 1) * (j.p.dep_i ? i : 1) +
-           up(qrow, nt) * qb * (j.q.dep_o ? o : 1) * (j.q.dep_i ? i : 1);
+    return p_bytes(prow) * (j.p.dep_o ? o : 1) * (j.p.dep_i ? i : 1) + q_bytes(qrow) * (j.q.dep_o ? o : 1) * (j.q.dep_i ? i : 1) +
+           o * i * (up(prow, kPTile) * up(qrow, nt) / 8);
   };
   long long go = no, gi = ni, prc = pr, qrc = qr;
   while (go > 1 && need(pr, qr, go, gi) > W) go = (go + 1) / 2;
   while (gi > 1 && need(pr, qr, go, gi) > W) gi = (gi + 1) / 2;
   if (need(pr, qr, go, gi) > W) {
     qrc = std::min<long long>(qr, (W / 2) / qb / nt * nt);
+    while (qrc > 0 && q_bytes(qrc) > W / 2) qrc = (qrc - 1) / nt * nt;
     if (qrc <= 0) return GW_OK;
-    prc = std::min<long long>(pr, (W - up(qrc, nt) * qb) / pb / kPTile * kPTile);
+    prc = std::min<long long>(pr, (W - q_bytes(qrc)) / pb / kPTile * kPTile);
+    while (prc > 0 && need(prc, qrc, 1, 1) > W) prc = (prc - 1) / kPTile * kPTile;
     if (prc <= 0) return GW_OK;
   }
   *done = true;
@@ -863,12 +1163,16 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
           j.q.row0 = (int)q0;
           j.q.rows = (int)std::min(qrc, qr - q0);
           j.q.tiles = (j.q.rows + nt - 1) / nt;
+          j.p.mtiles = (j.p.rows + kMagTile - 1) / kMagTile;
+          j.q.mtiles = (j.q.rows + kMagTile - 1) / kMagTile;
           const long long pn = (long long)j.p.no * j.p.ni * j.p.tiles * kPTile;
           const long long qn = (long long)j.q.no * j.q.ni * j.q.tiles * nt;
           unsigned char* m = (unsigned char*)g.ws->mem;
           j.p.dst = m;
           j.q.dst = m + pn * j.nks * 512;
-          j.p.scale = reinterpret_cast<double*>(j.q.dst + qn * j.nks * 256);
+          j.p.mag = j.q.dst + qn * j.nks * 256;
+          j.q.mag = j.p.mag + (long long)j.p.no * j.p.ni * j.p.mtiles * j.nms * kMagStep;
+          j.p.scale = reinterpret_cast<double*>(j.q.mag + (long long)j.q.no * j.q.ni * j.q.mtiles * j.nms * kMagStep);
           j.q.scale = j.p.scale + pn;
           // long rows are packed in segments where the row tiles alone leave SMs idle (8 blocks an SM)
           const long long blocks = (long long)j.p.no * j.p.ni * j.p.tiles + (long long)j.q.no * j.q.ni * j.q.tiles;
@@ -883,9 +1187,10 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
           // of 85 chunks on 152 SMs (P0 of a 2x2x2 solid): 12.5 -> 7.7 ms (with
           // equal tau batches).
           const long long tiles = (long long)j.p.tiles * j.q.tiles * j.no * j.ni;
+          j.left = reinterpret_cast<uint32_t*>(j.q.pmax + (j.segs > 1 ? qn * j.segs : 0));
           const int nchunks = (j.nks + kChunkSteps - 1) / kChunkSteps;
           j.ksplit = 1;
-          j.part_hi = reinterpret_cast<long long*>(j.q.pmax + (j.segs > 1 ? qn * j.segs : 0));
+          j.part_hi = reinterpret_cast<long long*>(j.left + tiles * kPTile * (nt / 32));
           const long long room = (m + g.ws->bytes - reinterpret_cast<unsigned char*>(j.part_hi)) / (128 * nt * 12);
           if (g.ws->counters && nchunks > 1 && tiles <= kSplitTiles) {
             long long best = (tiles + sm_count() - 1) / sm_count() * nchunks;
