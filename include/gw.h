@@ -102,7 +102,8 @@ typedef struct {
   double mu;            /* chemical potential (Ha), used by gw_dyson_G */
   double spin_factor;   /* spin sum of Eq. tilde_P0_tau: 2 for spin-restricted G */
   int precision;        /* gw_precision */
-  int tau_chunk;        /* tau nodes per batch in the contractions; 0 = automatic */
+  int tau_chunk;        /* tau nodes per batch in the contractions; 0 = automatic. In FP64 a bound on their
+                           memory: digits of the tensor-core products share it, with fewer nodes at a time */
   int v_slices;         /* mixed precisions: GW_V_AUTO, GW_V_ALL_PAIRS or GW_V_PER_Q */
   int v_packed;         /* 1: V holds the pairs k1 <= k2 only (layout above). FP64 keeps a full
                            working copy in the context; the mixed precisions unpack the blocks

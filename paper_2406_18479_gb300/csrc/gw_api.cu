@@ -621,16 +621,18 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
     int nt = cfg->tau_chunk > 0 ? cfg->tau_chunk : (int)std::max(1.0, std::floor(4294967296.0 / per_t));
     c->nt = std::min(nt, c->ntau);
     if (cfg->precision == GW_FP64) {
-      // The digits of the contractions take three times their intermediates. An automatic tau batch
-      // shares its memory between both, so that a context needs no more than its intermediates alone
-      // would at the full batch (64 MiB where that is less); a given one gets digits for as much memory
-      // again. More digits than fit are made in pieces, with the same result.
+      // The digits of the contractions take three times their intermediates. Both share the memory that the
+      // intermediates alone would take at the full tau batch, given or automatic (64 MiB where that is less), so the
+      // nodes taken at a time are fewer. More digits than fit are made in pieces, with the same result. A batch
+      // whose digits all fit P(i Omega), which is idle then, keeps its nodes.
       const double dig_t = (double)oz64_bytes(c->naux, c->naux, nk * (int)c->nao2);
-      const double budget = std::max(c->nt * per_t, 67108864.0);
-      // (a sixteenth is left for the partial sums of products that split K)
-      if (cfg->tau_chunk <= 0) c->nt = std::max(1, std::min(c->nt, (int)(budget * 15 / 16 / (per_t + dig_t))));
       const double most = std::max(dig_t, (double)nk * oz64_bytes(c->nao, c->nao, c->naux * c->nao));   // P0's or Sigma's
-      c->oz_bytes = (size_t)std::min(c->nt * most + budget / 16, cfg->tau_chunk > 0 ? budget : std::max(budget - c->nt * per_t, 0.0));
+      const double budget = std::max(c->nt * per_t, 67108864.0);
+      const double pw = std::min(16.0 * nk * c->nwb * c->naux2, 4294967296.0);
+      // (a sixteenth is left for the partial sums of products that split K)
+      if (cfg->tau_chunk <= 0 || pw < c->nt * most)
+        c->nt = std::max(1, std::min(c->nt, (int)(budget * 15 / 16 / (per_t + dig_t))));
+      c->oz_bytes = (size_t)std::min(c->nt * most + budget / 16, std::max(budget - c->nt * per_t, 0.0));
       if ((rc = dev_alloc(c, &c->work, (size_t)c->nt * 2 * nk * c->pair)) != GW_OK) break;
       if (cfg->v_packed && (rc = dev_alloc(c, &c->Vfull, (size_t)nk * nk * c->pair)) != GW_OK) break;
     }
