@@ -131,9 +131,10 @@ struct gw_ctx {
   long long *tab_kkmq = nullptr, *tab_kmqk = nullptr, *tab_gkmq = nullptr;
   double2* work = nullptr;                // contraction intermediates, nt * 2 * nk * pair
   // Digit workspaces of the tensor-core FP64 products. Those of the transforms and of the products
-  // outside the contractions lie in a P array that is not in use (oz_buf): P~ during a transform to
-  // Matsubara, P0(tau) during one to tau, P(i Omega) otherwise; digits of up to kOz64L2Bytes stay in
-  // the 129 MB L2 between the packing and the GEMM. The FP64 contractions have their own (oz_mem).
+  // outside the contractions lie in a P array that is not in use: P~ during a transform to
+  // Matsubara (oz_fwd) and the inversions (oz_inv), P0(tau) during one to tau (oz_back), P(i Omega) otherwise
+  // (oz_w, oz_x); digits of up to kOz64L2Bytes stay in the 129 MB L2 between the packing and the GEMM. The FP64
+  // contractions (oz) take memory of their own (oz_mem) or P(i Omega), whichever is more.
   unsigned char *oz_mem = nullptr, *oz_small = nullptr, *oz_count = nullptr;
   size_t oz_bytes = 0;
   Oz64Ws oz_fwd, oz_back, oz_w, oz_x, oz_inv, oz;
@@ -201,9 +202,10 @@ int dev_alloc(gw_ctx* c, T** p, size_t count) {
   return GW_OK;
 }
 
-// host -> device copy of a table; nothing in a size-only build
+// host -> device copy of a table in the context's stream (which need not wait for the default stream; pageable
+// memory is staged before the call returns); nothing in a size-only build
 void upload(const gw_ctx* c, void* dst, const void* src, size_t bytes) {
-  if (!c->dry) cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+  if (!c->dry) cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream);
 }
 
 int cuda_check(const char* what) {
@@ -667,7 +669,7 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
     {
       if ((rc = dev_alloc(c, &c->oz_small, kOz64SmallBytes)) != GW_OK) break;
       if ((rc = dev_alloc(c, &c->oz_count, oz64_counter_bytes())) != GW_OK) break;
-      if (!c->dry) cudaMemset(c->oz_count, 0, oz64_counter_bytes());
+      if (!c->dry) cudaMemsetAsync(c->oz_count, 0, oz64_counter_bytes(), c->stream);
       // a P array where it is larger than the small buffer
       auto ws = [&](void* p, size_t n) {
         Oz64Ws w;
@@ -698,7 +700,7 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
         c->oz.bytes = c->oz_bytes;
       }
     }
-    if (!c->dry) cudaMemset(c->status, 0, 4 * sizeof(int));
+    if (!c->dry) cudaMemsetAsync(c->status, 0, 4 * sizeof(int), c->stream);
     if (cfg->precision != GW_FP64) {
       MixedDims d;
       d.nk3[0] = cfg->nk[0]; d.nk3[1] = cfg->nk[1]; d.nk3[2] = cfg->nk[2];
@@ -798,20 +800,21 @@ int gw_set_grids(gw_ctx* ctx, const double* tau_host, const gw_c128* Fb_host, co
     return fail(GW_EINVAL, "gw_set_grids: bosonic F and B must map mirrored nodes to mirrored frequencies");
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return cuda_check("gw_set_grids");
   const size_t sb = (size_t)nb * T * sizeof(double2), sf = (size_t)nf * T * sizeof(double2);
-  if (cudaMemcpy(ctx->Fb, Fb_host, sb, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(ctx->Bb, Bb_host, sb, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(ctx->Ff, Ff_host, sf, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(ctx->Bf, Bf_host, sf, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(ctx->wf, omega_f_host, (size_t)nf * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (cudaMemcpyAsync(ctx->Fb, Fb_host, sb, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
+      cudaMemcpyAsync(ctx->Bb, Bb_host, sb, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
+      cudaMemcpyAsync(ctx->Ff, Ff_host, sf, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
+      cudaMemcpyAsync(ctx->Bf, Bf_host, sf, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
+      cudaMemcpyAsync(ctx->wf, omega_f_host, (size_t)nf * sizeof(double), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess)
     return cuda_check("gw_set_grids copy");
   const std::pair<int*, std::vector<int>> exps[] = {{ctx->Fbe, column_exponents(Fb_host, nb, T)}, {ctx->Bbe, column_exponents(Bb_host, T, nb)},
                                                     {ctx->Ffe, column_exponents(Ff_host, nf, T)}, {ctx->Bfe, column_exponents(Bf_host, T, nf)}};
   for (const auto& e : exps)
-    if (cudaMemcpy(e.first, e.second.data(), e.second.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
+    if (cudaMemcpyAsync(e.first, e.second.data(), e.second.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess)
       return cuda_check("gw_set_grids copy");
   std::vector<double> w;
   weights_at_beta(tau_host, T, beta, w);
-  if (cudaMemcpy(ctx->wbeta, w.data(), (size_t)T * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (cudaMemcpyAsync(ctx->wbeta, w.data(), (size_t)T * sizeof(double), cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
+      cudaStreamSynchronize(ctx->stream) != cudaSuccess)      // the caller's arrays may be page-locked
     return cuda_check("gw_set_grids copy");
   return GW_OK;
 }
@@ -1548,8 +1551,8 @@ int gw_synchronize(gw_ctx* ctx) {
   int st[4] = {0, 0, 0, 0};
   cudaMemcpy(st, ctx->status, sizeof(st), cudaMemcpyDeviceToHost);
   if (st[0] || st[1] || st[2] || st[3]) {
-    cudaMemset(ctx->status, 0, sizeof(st));
-    cudaMemset(ctx->oz_count, 0, oz64_counter_bytes());   // a kernel that gave up may have left arrivals behind
+    cudaMemsetAsync(ctx->status, 0, sizeof(st), ctx->stream);
+    cudaMemsetAsync(ctx->oz_count, 0, oz64_counter_bytes(), ctx->stream);   // a kernel that gave up may have left arrivals behind
     if (st[1]) return fail(GW_EDEVTIMEOUT, "a device-side wait gave up (code %d)", st[1]);
     if (st[0]) return fail(GW_EINVAL, "a Dyson matrix was singular");
     return fail(GW_ECUDA, "device status %d %d", st[2], st[3]);

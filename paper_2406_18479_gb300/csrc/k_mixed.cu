@@ -1653,7 +1653,7 @@ int mixed_create(MixedState** out, const MixedDims& d, cudaStream_t stream, int*
         at(E_KMQK) = ((long long)km * nk + k) * s->pair;
       }
     if ((rc = m_alloc(s, &s->rowtabs, t.size(), bytes))) break;
-    if (!dry) cudaMemcpy(s->rowtabs, t.data(), t.size() * sizeof(long long), cudaMemcpyHostToDevice);
+    if (!dry) cudaMemcpyAsync(s->rowtabs, t.data(), t.size() * sizeof(long long), cudaMemcpyHostToDevice, stream);
   } while (false);
   if (rc != GW_OK || dry) {
     mixed_destroy(s);
