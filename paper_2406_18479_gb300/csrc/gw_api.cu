@@ -230,7 +230,7 @@ void free_ctx(gw_ctx* c) {
   delete c;
 }
 
-// Powers of two for the k of a transform's matrix m [rows][cols] (ZGemm::kexp), which keep its outputs with the digits:
+// Powers of two for the k of a transform's matrix m [rows][cols] (as ZGemm::kexp takes them), which keep its outputs with the digits:
 // first rows and columns are brought to a common largest element (a caller's grid may weigh its nodes by any
 // amount), then the columns, halfway, to 1. Fully to 1 the inputs of noise lose (up to 90% of their back transforms
 // left to the FP64 pipe), not at all the bosonic functions of low energy (up to 10%); halfway at most 2% of either,
@@ -239,7 +239,7 @@ std::vector<int> column_exponents(const gw_c128* m, int rows, int cols) {
   std::vector<double> l((size_t)rows * cols), r(rows, 0.0), c(cols, 0.0), h(cols, -1e9);
   double top = 0.0;
   for (size_t i = 0; i < l.size(); ++i) top = std::max(top, l[i] = std::max(std::fabs(m[i].re), std::fabs(m[i].im)));
-  if (!(top > 0.0 && std::isfinite(top))) return std::vector<int>(cols, 0);
+  if (!(top > 0.0 && std::isfinite(top))) return std::vector<int>(cols, 1022);
   for (double& x : l) x = std::max(x > 0.0 ? std::log2(x / top) : -100.0, -100.0);
   for (int it = 0; it < 3; ++it) {
     for (int n = 0; n < rows; ++n) {
@@ -253,7 +253,7 @@ std::vector<int> column_exponents(const gw_c128* m, int rows, int cols) {
   for (int n = 0; n < rows; ++n)
     for (int k = 0; k < cols; ++k) h[k] = std::max(h[k], l[(size_t)n * cols + k] - std::rint(c[k]));
   std::vector<int> e(cols);
-  for (int k = 0; k < cols; ++k) e[k] = (int)std::rint(std::rint(c[k]) + 0.5 * h[k]);
+  for (int k = 0; k < cols; ++k) e[k] = 1022 + (int)std::rint(std::rint(c[k]) + 0.5 * h[k]);
   return e;
 }
 

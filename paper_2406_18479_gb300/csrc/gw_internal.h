@@ -103,7 +103,10 @@ struct ZGemm {
   const Oz64Ws* ws = nullptr;    // digit workspace: with one, products that pay run on the tensor cores
   double unit = 0.0;             // complex multiply-adds of one (k, tau) matrix where a product joins several
   int skip0 = 0, skip1 = 0;      // outputs with m and n both in [skip0, skip1) are not written (K <= 64 and the digits only)
-  const int* kexp = nullptr;     // digits of A(m, k) 2^-kexp[k] and B(n, k) 2^kexp[k] (device, K; the product is the same)
+  // digits of A(m, k) 2^(kexp_a e) and B(n, k) 2^(-kexp_a e), which leaves the product as it is: e = kexp[bi kexp_batch + k]
+  // - 1022 within +-400 (0 where kexp is 0 or 2047); device memory
+  const int* kexp = nullptr;
+  int kexp_batch = 0, kexp_a = -1;
 };
 
 // C = alpha A B^T (+ C) within the error bound of an FP64 sum, K 2^-52 sum |a| |b| per output: on the tensor cores

@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <cstddef>
 
 #include "gw_internal.h"
 
@@ -328,43 +329,61 @@ __global__ void __launch_bounds__(kGjSmallThreads) gj_inverse_small_kernel(doubl
 }
 inline size_t gj_small_smem(int n) { return (size_t)(n * n + 2 * n + 2) * sizeof(double2); }   // of one matrix
 
-// The inversion for larger n, with its n^3 work on the tensor cores. Per panel of B columns this kernel (one
-// block per matrix) factors rows k0.. of the panel (LU with partial pivoting, in shared memory) and lays the
-// panel's step out as one product over the whole matrix (zgemm_oz64),
+// The inversion for larger n, with its n^3 work on the tensor cores. A panel of B columns is laid out as one product
+// over the whole matrix (zgemm_oz64),
 //   A += ap W,   W [B][n] = L11^{-1} ak,  ak: the pivot rows, with the identity in the panel's columns
 //                ap [n][B]: -L21 below the pivot rows, -A_panel U11^{-1} above them, U11^{-1} in them
 // after the rows the pivots interchanged have moved: the pivot rows become D^{-1} A_p (D = L11 U11 the pivot block),
 // the panel -A_panel D^{-1}, the pivot block D^{-1}, the rest A - A_panel D^{-1} A_p. Both triangles are applied
-// by substitution (a thread per row of ap or column of W), never D^{-1}: rounding of W then meets multipliers of at
-// most 1 instead of |A_panel| |D^{-1}|, as in an elimination column by column (with D^{-1} the error grows with
-// cond(D): 1e-3 instead of 1e-9 for column pairs that differ by 1e-6).
-// The digits of a row share one scale. So the B terms of the product are balanced by exact powers of two: row t of W
-// is brought to about 1 and column t of ap takes its size (without: 2e-7 where five rows of a panel are 1e10 times the
-// others). And the triangles keep their diagonals out of it: the panel's column s is L11^{-1} e_s = e_s + small ones,
-// the pivot row r likewise, whose products would meet the small elements of the other operand (a tenth of them left to
-// the FP64 pipe). The diagonal's term, the last kGjTail columns and pivot rows (of few terms), and the pivot block
-// are put into A here; the product adds the rest and spares the block.
-// What bounds the kernel is the chain of a column (search, one division, swap, update: 5 block-wide steps), then
-// the FP64 pipe: B^2/2 complex multiply-adds per row and per column. swp[c]: the row swapped with row c at step c.
+// by substitution, never D^{-1}: rounding of W then meets multipliers of at most 1 instead of |A_panel| |D^{-1}|,
+// as in an elimination column by column (with D^{-1} the error grows with cond(D): 1e-3 instead of 1e-9 for column
+// pairs that differ by 1e-6).
+// The digits of a row share one scale. So the B terms of the product are balanced by exact powers of two (wexp,
+// ZGemm::kexp): row t of W counts as about 1 and column t of ap takes its size (without: 2e-7 where five rows of a panel
+// are 1e10 times the others). And the triangles keep their diagonals out of it: the panel's column s is
+// L11^{-1} e_s = e_s + small ones, the pivot row r likewise, whose products would meet the small elements of the other
+// operand (a tenth of them left to the FP64 pipe). The diagonal's term, the last kGjTail columns and pivot rows (of
+// few terms), and the pivot block are put into A by gj_apply_kernel; the product adds the rest and spares the block.
+//   gj_panel_kernel  one block per matrix: LU of rows k0.. of the panel with partial pivoting, in shared memory. Bound:
+//                    the chain of a column (search, one division, swap, update: 5 block-wide steps)
+//   gj_apply_kernel  a thread per column of W and per row of ap, over all SMs. Bound: the FP64 pipe (B^2/2 complex
+//                    multiply-adds each)
+// One kernel for both, a block per matrix: 24 matrices of 125 took 120 us a panel, now 59 + 54; 81 of 480 239, now
+// 102 + 112; the screened interaction of a 3x3x3 solid (2700 of 200) 89.4 ms, now 82.8.
 constexpr int kGjTail = 4;
+constexpr int kGjApplyThreads = 64;      // two warps: few matrices still reach every SM
+template <int B>
+struct GjPanel {           // of one matrix, in the workspace
+  double2 lu[B][B];        // U11 and the multipliers of L11
+  double2 dinv[B];         // 1 / diagonal of U11
+  int wexp[B];             // biased exponent of the largest |re|, |im| of each row of W
+  int row[2 * B], src[2 * B], cnt;   // the interchanges as one move: row[t] takes what row src[t] held; cnt < 0: singular
+};
 template <int B>
 size_t gj_panel_smem(int n) {
   return (size_t)n * (B + 1) * sizeof(double2);
 }
-constexpr int kGjBalanceMax = 400;       // powers of two of the balance: no over- or underflow of ordinary values
+__device__ __forceinline__ void msub(double2& v, double2 f, double2 r) {   // v -= f r
+  v.x = fma(-f.x, r.x, v.x);
+  v.x = fma(f.y, r.y, v.x);
+  v.y = fma(-f.x, r.y, v.y);
+  v.y = fma(-f.y, r.x, v.y);
+}
+__device__ __forceinline__ double2 neg(double2 v) { return make_double2(-v.x, -v.y); }
+
+// swp[c]: the row swapped with row c at step c
 template <int B>
 __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, long long stride, const int* list, int k0,
-                                                       double2* ap_all, double2* w_all, int* swp_all, int* status) {
+                                                       double2* ap_all, GjPanel<B>* panels, int* swp_all, int* status) {
   extern __shared__ double2 sm[];
   __shared__ long long red_v[8];
   __shared__ int red_i[8];
-  __shared__ int s_p, s_bad, s_cnt;
-  __shared__ int s_swp[B], s_row[2 * B], s_src[2 * B];
-  __shared__ unsigned int s_max[B];        // largest |re|, |im| of a row of W (leading 32 bits)
-  __shared__ double2 s_inv, s_dinv[B], Ui[B][B + 1];   // U11^{-1}
+  __shared__ int s_p, s_bad;
+  __shared__ int s_swp[B];
+  __shared__ double2 s_inv;
   double2* M = base + (long long)(list ? list[blockIdx.x] : (int)blockIdx.x) * stride;
   double2* ap = ap_all + (long long)blockIdx.x * B * n;
-  double2* W = w_all + (long long)blockIdx.x * B * n;
+  GjPanel<B>& out = panels[blockIdx.x];
   int* swp = swp_all + (long long)blockIdx.x * n;
   const int nr = n - k0;                   // rows k0.. of the panel
   double2* P = sm;                         // [nr][B]
@@ -375,14 +394,8 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
     const double den = v.x * v.x + v.y * v.y;
     return make_double2(v.x / den, -v.y / den);
   };
-  auto msub = [](double2& v, double2 f, double2 r) {   // v -= f r
-    v.x = fma(-f.x, r.x, v.x);
-    v.x = fma(f.y, r.y, v.x);
-    v.y = fma(-f.x, r.y, v.y);
-    v.y = fma(-f.y, r.x, v.y);
-  };
   if (tid == 0) s_bad = 0;
-  if (tid < B) s_max[tid] = 0;
+  if (tid < B) out.wexp[tid] = 0;
   for (int e = tid; e < nr * B; e += blockDim.x) {
     const int i = e / B, j = e % B;
     P[e] = j < kb ? M[(long long)(k0 + i) * n + k0 + j] : make_double2(0.0, 0.0);
@@ -412,7 +425,7 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
         if (red_v[w] > bb || (red_v[w] == bb && red_i[w] < ii)) { bb = red_v[w]; ii = red_i[w]; }
       s_p = ii;
       s_swp[j] = k0 + ii;
-      s_inv = s_dinv[j] = inverse(P[ii * B + j]);   // one thread: 256 divisions would cost the FP64 pipe 3k clocks
+      s_inv = out.dinv[j] = inverse(P[ii * B + j]);   // one thread: 256 divisions would cost the FP64 pipe 3k clocks
       if (!(bb > 0)) s_bad = 1;
     }
     __syncthreads();
@@ -445,155 +458,193 @@ __global__ void __launch_bounds__(256) gj_panel_kernel(double2* base, int n, lon
     }
     __syncthreads();
   }
-  if (s_bad) {                             // no step: the product adds nothing to this matrix
-    if (tid == 0) atomicExch(status, 1);
+  if (s_bad) {
+    if (tid == 0) {
+      atomicExch(status, 1);
+      out.cnt = -1;
+    }
     for (int t = tid; t < kb; t += blockDim.x) swp[k0 + t] = k0 + t;
-    for (int e = tid; e < n * B; e += blockDim.x) ap[e] = W[e] = make_double2(0.0, 0.0);
     return;
   }
   if (tid < kb) swp[k0 + tid] = s_swp[tid];
-  if (tid == 0) {   // the swaps as one move: row s_row[t] takes what row s_src[t] held
+  if (tid == 0) {
     int cnt = kb;
-    for (int t = 0; t < kb; ++t) s_row[t] = s_src[t] = k0 + t;
+    for (int t = 0; t < kb; ++t) out.row[t] = out.src[t] = k0 + t;
     for (int j = 0; j < kb; ++j) {
       const int p = s_swp[j];
       int at = -1;
       for (int t = 0; t < cnt; ++t)
-        if (s_row[t] == p) at = t;
+        if (out.row[t] == p) at = t;
       if (at < 0) {
         at = cnt++;
-        s_row[at] = s_src[at] = p;
+        out.row[at] = out.src[at] = p;
       }
-      const int x = s_src[j];
-      s_src[j] = s_src[at];
-      s_src[at] = x;
+      const int x = out.src[j];
+      out.src[j] = out.src[at];
+      out.src[at] = x;
     }
-    s_cnt = cnt;
+    out.cnt = cnt;
+  }
+  for (int e = tid; e < kb * B; e += blockDim.x) out.lu[e / B][e % B] = P[e];
+  for (int e = kb * B + tid; e < nr * B; e += blockDim.x) ap[(long long)k0 * B + e] = neg(P[e]);
+}
+
+// The substitutions go in blocks of 4 unknowns, the vector moving down by 4 registers a block: code that is run once per
+// warp in full (the 120 steps unrolled: 14 KB a triangle) costs more in instruction fetches than in arithmetic.
+template <int B>
+__global__ void __launch_bounds__(kGjApplyThreads) gj_apply_kernel(double2* base, int n, long long stride, const int* list, int k0,
+                                                                   double2* ap_all, double2* w_all, GjPanel<B>* panels) {
+  static_assert(kGjTail == 4 && B % 4 == 0, "the tail is the last block of the substitutions");
+  __shared__ double2 P[B][B + 1], dinv[B], X[kGjApplyThreads][B + 1];
+  __shared__ double2 Ut[4][4], Lt[4][4];   // inverses of the triangles' last blocks
+  __shared__ int s_row[2 * B], s_src[2 * B];
+  double2* M = base + (long long)(list ? list[blockIdx.y] : (int)blockIdx.y) * stride;
+  double2* ap = ap_all + (long long)blockIdx.y * B * n;
+  double2* W = w_all + (long long)blockIdx.y * B * n;
+  GjPanel<B>& in = panels[blockIdx.y];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int kb = min(B, n - k0), tail = (kb - 1) / 4 * 4, n32 = (n + 31) / 32 * 32;
+  const int id = blockIdx.x * kGjApplyThreads + tid;
+  const bool is_col = id < n32;
+  const int at = is_col ? id : id - n32;   // column or row
+  const int cnt = in.cnt;
+  const double2 zero = make_double2(0.0, 0.0);
+  if (cnt < 0) {                           // singular: the product adds nothing to this matrix
+    if (at < n)
+      for (int t = 0; t < B; ++t) (is_col ? W[(long long)t * n + at] : ap[(long long)at * B + t]) = zero;
+    return;
+  }
+  for (int e = tid; e < B * B; e += kGjApplyThreads) P[e / B][e % B] = e / B < kb ? in.lu[e / B][e % B] : zero;
+  if (tid < cnt) {
+    s_row[tid] = in.row[tid];
+    s_src[tid] = in.src[tid];
+  }
+  if (tid < B) dinv[tid] = tid < kb ? in.dinv[tid] : zero;
+  __syncthreads();
+  if (tid < kb - tail) {                   // row tid of Ut
+    for (int c = tid; c < kb - tail; ++c) {
+      double2 x = make_double2(c == tid ? 1.0 : 0.0, 0.0);
+      for (int s = tid; s < c; ++s) msub(x, Ut[tid][s], P[tail + s][tail + c]);
+      Ut[tid][c] = cmul(x, dinv[tail + c]);
+    }
+  } else if (tid >= 32 && tid - 32 < kb - tail) {   // column tid - 32 of Lt
+    const int c = tid - 32;
+    Lt[c][c] = make_double2(1.0, 0.0);
+    for (int a = c + 1; a < kb - tail; ++a) {
+      double2 x = zero;
+      for (int s = c; s < a; ++s) msub(x, P[tail + a][tail + s], Lt[s][c]);
+      Lt[a][c] = x;
+    }
   }
   __syncthreads();
-  const int cnt = s_cnt;
-  // ---- the other columns: pivot rows out, interchanged rows moved; W = L11^{-1} ak
-  unsigned int mx[B];
+  double2 v[B];
+  if (is_col) {
+    // ---- a column: pivot rows out, interchanged rows moved; W = L11^{-1} ak; the pivot rows of A
+    const int col = at;
+    const bool panel = col >= k0 && col < k0 + kb, in_n = col < n, other = in_n && !panel;
 #pragma unroll
-  for (int t = 0; t < B; ++t) mx[t] = 0;
-  for (int col = tid; col < n; col += blockDim.x) {
-    const bool panel = col >= k0 && col < k0 + kb;
-    double2 v[2 * B];
-    if (panel) {
-#pragma unroll
-      for (int t = 0; t < B; ++t) v[t] = make_double2(col - k0 == t ? 1.0 : 0.0, 0.0);
-    } else {
-#pragma unroll
-      for (int t = 0; t < 2 * B; ++t)
-        if (t < cnt) v[t] = M[(long long)s_src[t] * n + col];
-#pragma unroll
-      for (int t = B; t < 2 * B; ++t)
-        if (t < cnt) M[(long long)s_row[t] * n + col] = v[t];
-      if (kb < B) {
-#pragma unroll
-        for (int t = 0; t < B; ++t)
-          if (t >= kb && t < cnt) M[(long long)s_row[t] * n + col] = v[t];
-      }
+    for (int t = 0; t < B; ++t) {
+      v[t] = make_double2(col - k0 == t ? 1.0 : 0.0, 0.0);
+      if (other && t < kb) v[t] = M[(long long)s_src[t] * n + col];
     }
-#pragma unroll
-    for (int t = 0; t < B; ++t)
-      if (t < kb) {
-        double2 x = v[t];
-#pragma unroll
-        for (int s = 0; s < t; ++s) msub(x, P[t * B + s], v[s]);
-        v[t] = x;
-        W[(long long)t * n + col] = x;
-        if (!panel) mx[t] = max(mx[t], (unsigned int)max(__double2hiint(x.x) & 0x7FFFFFFF, __double2hiint(x.y) & 0x7FFFFFFF));
-      }
-  }
-#pragma unroll
-  for (int t = 0; t < B; ++t) {
-    const unsigned int m = __reduce_max_sync(0xffffffffu, mx[t]);
-    if (lane == 0) atomicMax(&s_max[t], m);
-  }
-  __syncthreads();
-  auto size_of = [&](int t) {              // about log2 of the largest element of row t of W
-    const int ex = (int)(s_max[t] >> 20);
-    return ex == 0 || ex == 0x7FF ? 0 : max(-kGjBalanceMax, min(kGjBalanceMax, ex - 1022));
-  };
-  auto pow2 = [](int e) { return __longlong_as_double((long long)(e + 1023) << 52); };
-  const int tail = max(0, kb - kGjTail);
-  // ---- ap: the multipliers below, x U11 = -A_panel (above) or the identity (pivot rows) by substitution; the panel's
-  // part of A: the diagonal's term, all terms of the tail
-  for (int i = tid; i < n; i += blockDim.x) {
-    const bool pivot = i >= k0 && i < k0 + kb;
-    double2 v[B];
-    if (i >= k0 + kb) {
-#pragma unroll
-      for (int t = 0; t < B; ++t) v[t] = make_double2(-P[(i - k0) * B + t].x, -P[(i - k0) * B + t].y);
-    } else {
-#pragma unroll
-      for (int t = 0; t < B; ++t) {
-        v[t] = make_double2(i - k0 == t ? 1.0 : 0.0, 0.0);
-        if (i < k0 && t < kb) {
-          const double2 a = M[(long long)i * n + k0 + t];
-          v[t] = make_double2(-a.x, -a.y);
-        }
-      }
+    if (other) {
+      double2 x[B];
 #pragma unroll
       for (int t = 0; t < B; ++t)
-        if (t < kb) {
-          double2 x = v[t];
+        if (kb + t < cnt) x[t] = M[(long long)s_src[kb + t] * n + col];
 #pragma unroll
-          for (int s = 0; s < t; ++s) msub(x, v[s], P[s * B + t]);
-          v[t] = cmul(x, s_dinv[t]);
-        }
+      for (int t = 0; t < B; ++t)
+        if (kb + t < cnt) M[(long long)s_row[kb + t] * n + col] = x[t];
     }
+    int mine = 0;                          // lane t: of row t
+#pragma unroll 1
+    for (int b = 0; b <= tail; b += 4) {
 #pragma unroll
-    for (int t = 0; t < B; ++t) {
-      const double f = t < kb && !(pivot && (i - k0 >= tail || i - k0 == t)) ? pow2(size_of(t)) : 0.0;
-      ap[(long long)i * B + t] = f != 0.0 ? make_double2(v[t].x * f, v[t].y * f) : make_double2(0.0, 0.0);
-      if (pivot) Ui[i - k0][t] = v[t];
-      if (pivot || t >= kb) continue;
-      double2 x = v[t];
-      if (t >= tail) {
+      for (int s = 0; s < 4; ++s)
 #pragma unroll
-        for (int s = t + 1; s < min(B, t + kGjTail); ++s)
-          if (s < kb) {
-            const double2 w = W[(long long)s * n + k0 + t];
-            msub(x, make_double2(-v[s].x, -v[s].y), w);
+        for (int t = s + 1; t < 4; ++t) msub(v[t], P[b + t][b + s], v[s]);
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        if (b + s >= kb) continue;
+        const int m = other ? max(__double2hiint(v[s].x) & 0x7FFFFFFF, __double2hiint(v[s].y) & 0x7FFFFFFF) >> 20 : 0;
+        const int top = __reduce_max_sync(0xffffffffu, m);
+        if (lane == b + s) mine = top;
+        if (in_n) W[(long long)(b + s) * n + col] = panel && (col - k0 == b + s || col - k0 >= tail) ? zero : v[s];
+        if (other) {
+          double2 x = cmul(dinv[b + s], v[s]);
+          if (b == tail) {
+#pragma unroll
+            for (int t = s + 1; t < 4; ++t)
+              if (b + t < kb) msub(x, neg(Ut[s][t]), v[t]);
           }
+          M[(long long)(k0 + b + s) * n + col] = x;
+        }
       }
-      M[(long long)i * n + k0 + t] = x;
-    }
-  }
-  __syncthreads();
-  if (tid < kb * kb) {                     // the pivot block D^{-1}
-    const int a = tid / kb, c = tid % kb;
-    double2 v = make_double2(0.0, 0.0);
-    for (int t = max(a, c); t < kb; ++t) {
-      const double2 u = Ui[a][t], w = W[(long long)t * n + k0 + c];
-      msub(v, make_double2(-u.x, -u.y), w);
-    }
-    M[(long long)(k0 + a) * n + k0 + c] = v;
-  }
-  __syncthreads();
-  // ---- W scaled, the panel's diagonal and tail out; the pivot rows of A: the diagonal's term, all terms of the tail
-  for (int col = tid; col < n; col += blockDim.x) {
-    const bool panel = col >= k0 && col < k0 + kb;
-    double2 v[B];
 #pragma unroll
-    for (int t = 0; t < B; ++t)
-      if (t < kb) v[t] = W[(long long)t * n + col];
+      for (int g = 4; g < B; g += 4) {
+        if (b + g < B) {
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) msub(v[g + t], P[b + g + t][b + s], v[s]);
+        }
+      }
+#pragma unroll
+      for (int t = 4; t < B; ++t) v[t - 4] = v[t];
+    }
+    if (lane < kb && mine) atomicMax(&in.wexp[lane], mine);
+  } else if (at < n) {
+    // ---- a row: ap (below the pivot rows it is there), x U11 = -A_panel or the identity; the panel of A
+    const int i = at;
+    const bool below = i >= k0 + kb, pivot = i >= k0 && !below;
 #pragma unroll
     for (int t = 0; t < B; ++t) {
-      if (t >= kb) continue;
-      const double f = panel && (col - k0 == t || col - k0 >= tail) ? 0.0 : pow2(-size_of(t));
-      W[(long long)t * n + col] = f != 0.0 ? make_double2(v[t].x * f, v[t].y * f) : make_double2(0.0, 0.0);
-      if (panel) continue;
-      double2 x = cmul(Ui[t][t], v[t]);
-      if (t >= tail) {
-#pragma unroll
-        for (int s = t + 1; s < min(B, t + kGjTail); ++s)
-          if (s < kb) msub(x, make_double2(-Ui[t][s].x, -Ui[t][s].y), v[s]);
-      }
-      M[(long long)(k0 + t) * n + col] = x;
+      v[t] = make_double2(i - k0 == t ? 1.0 : 0.0, 0.0);
+      if (below) v[t] = ap[(long long)i * B + t];
+      else if (!pivot) v[t] = t < kb ? neg(M[(long long)i * n + k0 + t]) : zero;
     }
+#pragma unroll 1
+    for (int b = 0; b < B; b += 4) {
+      if (!below) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          v[s] = cmul(v[s], dinv[b + s]);
+#pragma unroll
+          for (int t = s + 1; t < 4; ++t) msub(v[t], v[s], P[b + s][b + t]);
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const int r = b + s;
+        if (!below) ap[(long long)i * B + r] = r >= kb || (pivot && (i - k0 >= tail || i - k0 == r)) ? zero : v[s];
+        if (pivot) X[tid][r] = v[s];
+        if (pivot || r >= kb) continue;
+        double2 x = v[s];
+        if (b == tail) {
+#pragma unroll
+          for (int t = s + 1; t < 4; ++t)
+            if (b + t < kb) msub(x, neg(v[t]), Lt[t][s]);
+        }
+        M[(long long)i * n + k0 + r] = x;
+      }
+#pragma unroll
+      for (int g = 4; g < B; g += 4) {
+        if (!below && b + g < B) {
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) msub(v[g + t], v[s], P[b + s][b + g + t]);
+        }
+      }
+#pragma unroll
+      for (int t = 4; t < B; ++t) v[t - 4] = v[t];
+    }
+    if (pivot)                             // its row of D^{-1}: y L11 = U11^{-1} row
+      for (int s = kb - 1; s >= 0; --s) {
+        const double2 y = X[tid][s];
+        M[(long long)i * n + k0 + s] = y;
+        for (int t = 0; t < s; ++t) msub(X[tid][t], y, P[s][t]);
+      }
   }
 }
 
@@ -1045,16 +1096,18 @@ bool gj_panel_attr() {
   return ok;
 }
 
-// per matrix: the panel's ap and W, the swaps, and the digits of the product
-size_t gj_side_bytes(int n, int B) { return (size_t)(2 * B * n) * sizeof(double2) + (size_t)n * sizeof(int); }
-size_t gj_group_bytes(int n, int B) { return oz64_bytes(n, n, B) + gj_side_bytes(n, B) + 256; }
+// per matrix: the panel's ap, W and factors, the swaps, and the digits of the product
+template <int B>
+size_t gj_side_bytes(int n) { return (size_t)(2 * B * n) * sizeof(double2) + sizeof(GjPanel<B>) + (size_t)n * sizeof(int); }
+template <int B>
+size_t gj_group_bytes(int n) { return oz64_bytes(n, n, B) + gj_side_bytes<B>(n) + 256; }
 
 // Panels and tensor-core updates of groups of matrices whose digits, pivot rows and swaps fit ws
 template <int B>
 int inverse_panels(double2* base, int n, long long stride, int nbatch, int* status, cudaStream_t st, const int* list,
                    const Oz64Ws& ws) {
   if (!gj_panel_attr<B>()) return fail(GW_ECUDA, "gj_panel: shared memory attribute refused");
-  const int group = (int)std::min<size_t>(nbatch, std::max<size_t>(1, ws.bytes / gj_group_bytes(n, B)));
+  const int group = (int)std::min<size_t>(nbatch, std::max<size_t>(1, ws.bytes / gj_group_bytes<B>(n)));
   const int ngroups = (nbatch + group - 1) / group;
   for (int g = 0; g < ngroups; ++g) {
     const int m0 = (int)((long long)nbatch * g / ngroups), m1 = (int)((long long)nbatch * (g + 1) / ngroups), m = m1 - m0;
@@ -1063,16 +1116,20 @@ int inverse_panels(double2* base, int n, long long stride, int nbatch, int* stat
     const long long pn = (long long)B * n;
     double2* ap = reinterpret_cast<double2*>(ws.mem);
     double2* W = ap + m * pn;
-    int* swp = reinterpret_cast<int*>(W + m * pn);
-    const size_t head = (m * gj_side_bytes(n, B) + 255) / 256 * 256;
+    GjPanel<B>* panels = reinterpret_cast<GjPanel<B>*>(W + m * pn);
+    int* swp = reinterpret_cast<int*>(panels + m);
+    const size_t head = (m * gj_side_bytes<B>(n) + 255) / 256 * 256;
     Oz64Ws rest = ws;
     rest.mem = (unsigned char*)ws.mem + head;
     rest.bytes = ws.bytes - head;
     for (int k0 = 0; k0 < n; k0 += B) {
       const int kb = std::min(B, n - k0);
       prof_begin(SLOT_INVERSE_FP64, st);
-      gj_panel_kernel<B><<<m, 256, gj_panel_smem<B>(n - k0), st>>>(b0, n, stride, l0, k0, ap, W, swp, status);
-      prof_end(SLOT_INVERSE_FP64, st, 4.0 * m * (double)(3 * n - k0) * kb * kb, 32.0 * m * (double)n * (3 * kb));
+      gj_panel_kernel<B><<<m, 256, gj_panel_smem<B>(n - k0), st>>>(b0, n, stride, l0, k0, ap, panels, swp, status);
+      prof_end(SLOT_INVERSE_FP64, st, 4.0 * m * (double)(n - k0) * kb * kb, 32.0 * m * (double)(n - k0) * kb);
+      prof_begin(SLOT_INVERSE_FP64, st);
+      gj_apply_kernel<B><<<dim3((n + 31) / 32, m), kGjApplyThreads, 0, st>>>(b0, n, stride, l0, k0, ap, W, panels);
+      prof_end(SLOT_INVERSE_FP64, st, 8.0 * m * (double)n * kb * kb, 32.0 * m * (double)n * 3 * kb);
       ZGemm z;                               // A += ap W
       z.M = n;
       z.N = n;
@@ -1092,6 +1149,9 @@ int inverse_panels(double2* base, int n, long long stride, int nbatch, int* stat
       z.bc.list = l0;
       z.bc.bs_in = stride;
       z.accumulate = 1;
+      z.kexp = reinterpret_cast<const int*>(reinterpret_cast<const char*>(panels) + offsetof(GjPanel<B>, wexp));
+      z.kexp_batch = (int)(sizeof(GjPanel<B>) / sizeof(int));
+      z.kexp_a = 1;
       z.skip0 = k0;
       z.skip1 = k0 + kb;
       z.slot = SLOT_INVERSE_FP64;
@@ -1117,9 +1177,9 @@ int batched_inverse_fp64(double2* base, int n, long long stride, int nbatch, int
   if (nbatch <= 0) return GW_OK;
   cudaStream_t st = (cudaStream_t)stream;
   if (n >= kGjPanelMinN && n <= kGjPanelMaxN8 && ws && ws->mem) {
-    if (n <= kGjPanelMaxN16 && ws->bytes >= gj_group_bytes(n, 16))
+    if (n <= kGjPanelMaxN16 && ws->bytes >= gj_group_bytes<16>(n))
       return inverse_panels<16>(base, n, stride, nbatch, status_dev, st, list, *ws);
-    if (n > kGjPanelMaxN16 && ws->bytes >= gj_group_bytes(n, 8))
+    if (n > kGjPanelMaxN16 && ws->bytes >= gj_group_bytes<8>(n))
       return inverse_panels<8>(base, n, stride, nbatch, status_dev, st, list, *ws);
   }
   const double flops = 8.0 * (double)n * n * n * nbatch, bytes = 32.0 * (double)n * n * nbatch;

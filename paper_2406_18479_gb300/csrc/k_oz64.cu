@@ -105,8 +105,8 @@ struct Side {
   unsigned long long* pmax = nullptr;   // segs > 1: largest |value| bits of each row and K segment
   unsigned char* mag = nullptr;         // magnitudes max(|re|, |im|) 2^-E, bf16 rounded down, steps of 128 rows x 16 k
   int mtiles = 0;                       // tiles of 128 rows of a packed batch
-  const int* kexp = nullptr;            // element (r, k) counts as x 2^(ksign kexp[k])
-  int ksign = 0;
+  const int* kexp = nullptr;            // element (r, k) counts as x 2^(ksign e) (ZGemm::kexp)
+  int ksign = 0, kbatch = 0;
 };
 
 struct Job {
@@ -149,11 +149,13 @@ __device__ __forceinline__ const double2* side_base(const Side& s, int bo, int b
   return s.src + batch_in(s.b, bi) + (long long)bo * s.b.bs_out;
 }
 
+constexpr int kExpMax = 400;          // of ZGemm::kexp: no over- or underflow of ordinary values
 template <bool KX>
-__device__ __forceinline__ double2 side_elem(const Side& s, const double2* row, int k) {
+__device__ __forceinline__ double2 side_elem(const Side& s, const double2* row, const int* kexp, int k) {
   double2 x = row[side_k(s, k)];
   if (KX) {
-    const double f = __longlong_as_double((long long)(1023 + s.ksign * s.kexp[k]) << 52);
+    const int b = kexp[k], e = b == 0 || b == 2047 ? 0 : max(-kExpMax, min(kExpMax, b - 1022));
+    const double f = __longlong_as_double((long long)(1023 + s.ksign * e) << 52);
     x = make_double2(x.x * f, x.y * f);
   }
   return x;
@@ -204,6 +206,7 @@ struct PackPos {
   long long prow;
   bool row_ok;
   const double2* src;
+  const int* kexp;
   __device__ PackPos(const Side& s, const Job& j, long long t) {
     seg = (int)(t % j.segs);
     t /= j.segs;
@@ -214,6 +217,7 @@ struct PackPos {
     const int r = tile * kRows + row;
     row_ok = r < s.rows;
     src = side_base(s, j.o0 + pb / s.ni, j.i0 + pb % s.ni) + (row_ok ? side_row(s, s.row0 + r) : 0);
+    kexp = s.kexp + (long long)(j.i0 + pb % s.ni) * s.kbatch;
     prow = ((long long)pb * s.tiles + tile) * kRows + row;
     k0 = seg * j.seg_steps;              // k-steps [k0, k1) of the segment
     k1 = min(j.nks, k0 + j.seg_steps);
@@ -230,7 +234,7 @@ __device__ __forceinline__ unsigned long long row_max(const Side& s, const Job& 
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         if (k + u >= kend) break;
-        const double2 x = side_elem<KX>(s, p.src, k + u);
+        const double2 x = side_elem<KX>(s, p.src, p.kexp, k + u);
         mx = max(mx, max((unsigned long long)__double_as_longlong(x.x) & 0x7FFFFFFFFFFFFFFFull,
                          (unsigned long long)__double_as_longlong(x.y) & 0x7FFFFFFFFFFFFFFFull));
       }
@@ -287,7 +291,7 @@ __device__ void pack_tile(const Side& s, const Job& j, long long t) {
     for (int c = 0; c < 4; ++c) {
       const int k = 4 * g + c;
       double2 x = make_double2(0.0, 0.0);
-      if (!zero && k < j.K) x = side_elem<KX>(s, p.src, k);
+      if (!zero && k < j.K) x = side_elem<KX>(s, p.src, p.kexp, k);
       u[2 * c] = digits_of(x.x, E);
       u[2 * c + 1] = digits_of(x.y, E);
       m[c] = magnitude(x, u[2 * c], u[2 * c + 1]);
@@ -1098,7 +1102,8 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
   j.q = p_is_b ? make_side(g.A, g.va, g.ba, no, ni) : make_side(g.B, g.vb, g.bb, no, ni);
   if (g.kexp) {
     j.p.kexp = j.q.kexp = g.kexp;
-    j.p.ksign = p_is_b ? 1 : -1;
+    j.p.kbatch = j.q.kbatch = g.kexp_batch;
+    j.p.ksign = p_is_b ? -g.kexp_a : g.kexp_a;
     j.q.ksign = -j.p.ksign;
   }
   const int pr = p_is_b ? g.N : g.M, qr = p_is_b ? g.M : g.N;
