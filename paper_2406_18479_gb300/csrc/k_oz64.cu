@@ -338,40 +338,136 @@ __device__ __forceinline__ uint32_t skip_bits(const Job& j, int c, int n) {
   return (uint32_t)((1ull << hi) - (1ull << lo));
 }
 
-// The outputs of this CTA's tiles that are left to the FP64 pipe: a group of 256 threads per 32 x 32 complex outputs, the
-// terms in order of k on the FP64 pipe as in zgemm_fp64_kernel. A thread has 2 x 2 outputs and a warp skips those that
-// none of its lanes needs, so a few of them cost the staging of their operands and little arithmetic. Of CTAs that share
-// a tile's K the first takes it. sm: the group's 2 kPlainK rows of 33 elements and the masks.
+// The outputs of this CTA's tiles that are left to the FP64 pipe, every sum in order of k as in zgemm_fp64_kernel.
+// Tiles with a few of them (kFew at most) go into one list, a thread per output; a tile of many goes 32 x 32 at a time, a
+// group of 256 threads each, staged through shared memory, 2 x 2 outputs a thread (a warp skips those that none of its
+// lanes needs). R = P~ V of a molecule (nao = 36, naux = 125), 3e-4 of its outputs left, one in a quarter of the
+// 32 x 32 pieces: 153 us a launch with pieces only, 106 with the list, 62 if nothing were left.
+// Of CTAs that share a tile's K the first takes it. sm: the stages.
 constexpr int kPlainK = 16, kPlainGroups = kEpiWarps / 8;
-constexpr size_t kPlainSmem = 2 * kPlainK * 33 * sizeof(double2) + 256;   // of a group
+constexpr int kFew = 128, kListMax = 8192, kUnitsMax = 16384;        // of a tile; entries; tiles looked over at a time
+constexpr size_t kPlainStage = 2 * kPlainK * 33 * sizeof(double2) + 256;   // of a group
+constexpr size_t kPlainSmem = kPlainGroups * kPlainStage + kListMax * 8 + kUnitsMax * 4 + 16;
 template <int NT>
-__device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, const uint32_t* map, int map_sh, int group, int tid,
-                                            unsigned char* sm) {
-  double2(*Ps)[33] = reinterpret_cast<double2(*)[33]>(sm);
+__device__ __noinline__ void plain_tiles(const Job& j, int ksplit, const uint32_t* map, int map_sh, int tid, unsigned char* sm) {
+  constexpr int kThreads = 32 * kEpiWarps, kWords = NT / 32;
+  const int group = tid >> 8, gid = tid & 255, warp = tid >> 5, lane = tid & 31;
+  unsigned char* stage = sm + group * kPlainStage;
+  double2(*Ps)[33] = reinterpret_cast<double2(*)[33]>(stage);
   double2(*Qs)[33] = Ps + kPlainK;
   uint32_t* s_left = reinterpret_cast<uint32_t*>(Qs + kPlainK);         // left columns of each row; whether any
+  int2* list = reinterpret_cast<int2*>(sm + kPlainGroups * kPlainStage);   // outputs: tile, row * 64 + column
+  int* many = reinterpret_cast<int*>(list + kListMax);                  // tiles with many
+  int* counts = many + kUnitsMax;                                       // of list and many
   auto sync = [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + group) : "memory"); };
+  auto sync_all = [&] { asm volatile("bar.sync 3, %0;" ::"n"(kThreads) : "memory"); };
   constexpr int kSub = 2 * (NT / 32);                 // 32 x 32 pieces of a GEMM tile
   const int per_batch = j.p.tiles * j.q.tiles, total = per_batch * j.no * j.ni * ksplit;
-  const int tx = tid & 15, ty = tid >> 4;
-  int own = 0;
+  const int owned = (total - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  auto mac = [](double2& s, double2 x, double2 y) {
+    s.x = fma(-x.y, y.y, fma(x.x, y.x, s.x));
+    s.y = fma(x.y, y.x, fma(x.x, y.y, s.y));
+  };
+  auto put = [&](int bo, int bi, int a, int c, double2 v) {              // output of P row a, Q row c
+    const int aq = div_by(a, j.cp_div), cq = div_by(c, j.cq_div);
+    double2* at = j.C + batch_in(j.bc, bi) + (long long)bo * j.bc.bs_out + (long long)aq * j.cp_out +
+                  (long long)(a - aq * j.cp_div.d) * j.cp_in + (long long)cq * j.cq_out + (long long)(c - cq * j.cq_div.d) * j.cq_in;
+    double2 x = make_double2(j.alpha * v.x, j.alpha * v.y);
+    if (j.accumulate) {
+      const double2 old = *at;
+      x.x += old.x;
+      x.y += old.y;
+    }
+    *at = x;
+  };
 #pragma unroll 1
-  for (int unit = blockIdx.x; unit < total; unit += gridDim.x, ++own) {
-    if (!(map[own >> map_sh >> 5] >> (own >> map_sh & 31) & 1)) continue;
-    const int tile = unit / ksplit;
-    if (unit != tile * ksplit) continue;
-    const int b = tile / per_batch, w = tile - b * per_batch, o = b / j.ni, i = b - o * j.ni;
-    const int pt = w / j.q.tiles, qt = w - pt * j.q.tiles;
+  for (int own0 = 0; own0 < owned; own0 += kUnitsMax) {
+    if (tid < 2) counts[tid] = 0;
+    sync_all();
+    // ---- a warp per tile: its outputs into the list, or the tile among those with many
 #pragma unroll 1
-    for (int sub = group; sub < kSub; sub += kPlainGroups) {
+    for (int own = own0 + warp; own < min(owned, own0 + kUnitsMax); own += kEpiWarps) {
+      if (!(map[own >> map_sh >> 5] >> (own >> map_sh & 31) & 1)) continue;
+      const int unit = blockIdx.x + own * gridDim.x, tile = unit / ksplit;
+      if (unit != tile * ksplit) continue;
+      const int pt = tile % per_batch / j.q.tiles;
+      uint32_t w[2 * kWords];
+      int n = 0;
+#pragma unroll
+      for (int u = 0; u < 2 * kWords; ++u) {
+        const int word = u * 32 + lane;
+        w[u] = pt * kPTile + word / kWords < j.p.rows ? j.left[(long long)tile * kPTile * kWords + word] : 0u;
+        n += __popc(w[u]);
+      }
+      int before = n;                      // outputs of the lanes up to this one
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += x;
+      }
+      const int all = __shfl_sync(0xffffffffu, before, 31);
+      if (all == 0) continue;
+      int first = kListMax;
+      if (all <= kFew) {
+        if (lane == 0) first = atomicAdd(&counts[0], all);
+        first = __shfl_sync(0xffffffffu, first, 0);
+      }
+      if (first + all > kListMax) {        // no room, or many
+        if (lane == 0) many[atomicAdd(&counts[1], 1)] = tile;
+        for (int e = first + lane; e < kListMax && e < first + all; e += 32) list[e] = make_int2(-1, 0);
+        continue;
+      }
+      int at = first + before - n;
+#pragma unroll
+      for (int u = 0; u < 2 * kWords; ++u)
+        for (uint32_t x = w[u]; x; x &= x - 1) {
+          const int word = u * 32 + lane;
+          list[at++] = make_int2(tile, word / kWords * 64 + word % kWords * 32 + __ffs(x) - 1);
+        }
+    }
+    sync_all();
+    // ---- the list, a thread per output, 4 k in flight
+    const int listed = min(counts[0], kListMax);
+#pragma unroll 1
+    for (int e = tid; e < listed; e += kThreads) {
+      const int2 x = list[e];
+      if (x.x < 0) continue;
+      const int b = x.x / per_batch, w = x.x - b * per_batch, o = b / j.ni, i = b - o * j.ni;
+      const int pt = w / j.q.tiles, qt = w - pt * j.q.tiles, bo = j.o0 + o, bi = j.i0 + i;
+      const int a = j.p.row0 + pt * kPTile + x.y / 64, c = j.q.row0 + qt * NT + x.y % 64;
+      const double2* A = side_base(j.p, bo, bi) + side_row(j.p, a);
+      const double2* B = side_base(j.q, bo, bi) + side_row(j.q, c);
+      double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 1
+      for (int k0 = 0; k0 < j.K; k0 += 4) {
+        double2 p[4], q[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k0 + k < j.K) {
+            p[k] = A[side_k(j.p, k0 + k)];
+            q[k] = B[side_k(j.q, k0 + k)];
+          }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k0 + k < j.K) mac(acc, p[k], q[k]);
+      }
+      put(bo, bi, a, c, acc);
+    }
+    // ---- the tiles with many
+    const int tx = gid & 15, ty = gid >> 4, nmany = counts[1];
+#pragma unroll 1
+    for (int piece = group; piece < nmany * kSub; piece += kPlainGroups) {
+      const int tile = many[piece / kSub], sub = piece % kSub;
+      const int b = tile / per_batch, w = tile - b * per_batch, o = b / j.ni, i = b - o * j.ni;
+      const int pt = w / j.q.tiles, qt = w - pt * j.q.tiles;
       const int p0 = (sub & 1) * 32, q0 = (sub >> 1) * 32;        // of the tile
       const int np = min(32, j.p.rows - pt * kPTile - p0), nq = min(32, j.q.rows - qt * NT - q0);
       if (np <= 0 || nq <= 0) continue;
       sync();
-      if (tid < 32) {
-        s_left[tid] = tid < np ? j.left[((long long)tile * kPTile + p0 + tid) * (NT / 32) + q0 / 32] : 0u;
-        const bool any = __any_sync(0xffffffffu, s_left[tid] != 0);
-        if (tid == 0) s_left[32] = any;
+      if (gid < 32) {
+        s_left[gid] = gid < np ? j.left[((long long)tile * kPTile + p0 + gid) * kWords + q0 / 32] : 0u;
+        const bool any = __any_sync(0xffffffffu, s_left[gid] != 0);
+        if (gid == 0) s_left[32] = any;
       }
       sync();
       if (!s_left[32]) continue;
@@ -381,8 +477,7 @@ __device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, const uint
       for (int u = 0; u < 2; ++u)
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
-          const int r = 2 * tx + u, c = 2 * ty + v;
-          need[u][v] = s_left[r] >> c & 1;
+          need[u][v] = s_left[2 * tx + u] >> (2 * ty + v) & 1;
           acc[u][v] = make_double2(0.0, 0.0);
         }
       const int bo = j.o0 + o, bi = j.i0 + i;
@@ -394,7 +489,7 @@ __device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, const uint
       for (int k0 = 0; k0 < j.K; k0 += kPlainK) {
         sync();
 #pragma unroll
-        for (int e = tid; e < 32 * kPlainK; e += 256) {
+        for (int e = gid; e < 32 * kPlainK; e += 256) {
           const int rp = pk ? e / kPlainK : e % 32, kp = pk ? e % kPlainK : e / 32;
           const int rq = qk ? e / kPlainK : e % 32, kq = qk ? e % kPlainK : e / 32;
           Ps[kp][rp] = rp < np && k0 + kp < j.K ? A[side_row(j.p, pr + rp) + side_k(j.p, k0 + kp)] : make_double2(0.0, 0.0);
@@ -407,34 +502,19 @@ __device__ __forceinline__ void plain_tiles(const Job& j, int ksplit, const uint
 #pragma unroll
           for (int v = 0; v < 2; ++v) {
             if (!need[u][v]) continue;
-            double2 s = acc[u][v];
+            double2 x = acc[u][v];
 #pragma unroll 4
-            for (int k = 0; k < kn; ++k) {
-              const double2 x = Ps[k][2 * tx + u], y = Qs[k][2 * ty + v];
-              s.x = fma(-x.y, y.y, fma(x.x, y.x, s.x));
-              s.y = fma(x.y, y.x, fma(x.x, y.y, s.y));
-            }
-            acc[u][v] = s;
+            for (int k = 0; k < kn; ++k) mac(x, Ps[k][2 * tx + u], Qs[k][2 * ty + v]);
+            acc[u][v] = x;
           }
       }
-      double2* C = j.C + batch_in(j.bc, bi) + (long long)bo * j.bc.bs_out;
 #pragma unroll
       for (int u = 0; u < 2; ++u)
 #pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          if (!need[u][v]) continue;
-          const int a = pr + 2 * tx + u, aq = div_by(a, j.cp_div), c = qr + 2 * ty + v, cq = div_by(c, j.cq_div);
-          double2* at = C + (long long)aq * j.cp_out + (long long)(a - aq * j.cp_div.d) * j.cp_in + (long long)cq * j.cq_out +
-                        (long long)(c - cq * j.cq_div.d) * j.cq_in;
-          double2 x = make_double2(j.alpha * acc[u][v].x, j.alpha * acc[u][v].y);
-          if (j.accumulate) {
-            const double2 old = *at;
-            x.x += old.x;
-            x.y += old.y;
-          }
-          *at = x;
-        }
+        for (int v = 0; v < 2; ++v)
+          if (need[u][v]) put(bo, bi, pr + 2 * tx + u, qr + 2 * ty + v, acc[u][v]);
     }
+    sync_all();
   }
 }
 
@@ -449,7 +529,7 @@ struct Oz64Shape {
   static constexpr int kThreads = 64 + 32 * kEpiWarps;          // producer, MMA, epilogue warps
   static constexpr size_t kSmem = 128 + (size_t)kStages * kStageBytes + 512;
   static_assert(kSmem <= 232448, "stages exceed shared memory");
-  static_assert(kPlainGroups * kPlainSmem <= (size_t)kStages * kStageBytes, "plain_tiles works in the stages");
+  static_assert(kPlainSmem <= (size_t)kStages * kStageBytes, "plain_tiles works in the stages");
 };
 
 // K-major operand without swizzle: 8 x 16-byte core matrices, 128 bytes between the two k halves
@@ -981,10 +1061,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) oz64_gemm_kernel(const
   __syncthreads();
   tc_fence_after();
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
-  if (!*abort_flag && warp >= 2) {
-    const int t = threadIdx.x - 64;
-    plain_tiles<NT>(j, ksplit, map, map_sh, t >> 8, t & 255, smem + (t >> 8) * kPlainSmem);
-  }
+  if (!*abort_flag && warp >= 2 && __any_sync(0xffffffffu, map[lane] != 0)) plain_tiles<NT>(j, ksplit, map, map_sh, threadIdx.x - 64, smem);
 }
 
 int sm_count() {

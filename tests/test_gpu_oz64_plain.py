@@ -107,3 +107,33 @@ def test_non_finite_rows(case, bad):
     assert not np.isfinite(s[:, 1]).any()
     keep = [t for t in range(ntau) if t != 1]
     assert np.array_equal(s[:, keep], clean_s[:, keep])
+
+
+def test_more_left_outputs_than_a_list_holds():
+    """Some rows of V beyond the digit range in every tile, over a hundred tiles a CTA: outputs in the list, those
+    that find no room in it, against plain complex128 products on the device."""
+    from paper_2406_18479_gb300 import gw
+    nk, nao, naux, ntau = 8, 26, 104, 80
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    c = lambda *s: torch.view_as_complex(torch.randn(s + (2,), dtype=torch.float64, device="cuda", generator=gen))   # noqa: E731
+    V, G = c(nk, nk, naux, nao, nao), c(nk, ntau, nao, nao)
+    V[:, :, :, 0, :] *= 1e148
+    ctx = gw.gw_create((2, 2, 2), nao, naux, ntau, 10.0)
+    gw.gw_set_coulomb(ctx, V)
+    P = torch.full(ctx.shapes()["Pt"], float("nan"), dtype=torch.complex128, device="cuda")
+    gw.gw_polarization(ctx, G, P)
+    gw.gw_synchronize(ctx)
+    gw.gw_check_guards(ctx)
+    ctx.destroy()
+    for q, t in ((0, 3), (5, 0), (7, 39)):
+        ref, mag = 0, 0
+        for k in range(nk):
+            p = k ^ q                                            # k + q on a mesh of twos
+            f = lambda x, y: (x @ y).reshape(naux, -1)           # noqa: E731
+            g = lambda x, y: (x @ y).transpose(1, 2).reshape(naux, -1)   # noqa: E731
+            ref = ref - 2.0 / nk * f(V[k, p], G[p, t]) @ g(V[p, k], G[k, ntau - 1 - t]).T
+            m = lambda x: torch.complex(x.abs(), torch.zeros_like(x.real))    # noqa: E731
+            mag = mag + 2.0 / nk * (f(m(V[k, p]), m(G[p, t])) @ g(m(V[p, k]), m(G[k, ntau - 1 - t])).T).real
+        bound = 2 * (2 * nao + nk * nao * nao + 4) * 2.0 ** -52 * mag
+        assert bool(((P[q, t] - ref).abs() <= bound).all())
