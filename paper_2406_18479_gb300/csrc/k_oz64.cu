@@ -103,8 +103,9 @@ struct Side {
   unsigned char* dst = nullptr;
   double* scale = nullptr;              // per packed row: 2^(E - 34), NaN: no digit form
   unsigned long long* pmax = nullptr;   // segs > 1: largest |value| bits of each row and K segment
-  unsigned char* mag = nullptr;         // magnitudes max(|re|, |im|) 2^-E, bf16 rounded down, steps of 128 rows x 16 k
-  int mtiles = 0;                       // tiles of 128 rows of a packed batch
+  // magnitudes max(|re|, |im|) 2^-E, bf16 rounded down: tiles of 128 rows (the last of what is left, in eights), steps of 16 k
+  unsigned char* mag = nullptr;
+  int mtiles = 0;                       // tiles of a packed batch
   const int* kexp = nullptr;            // element (r, k) counts as x 2^(ksign e) (ZGemm::kexp)
   int ksign = 0, kbatch = 0;
 };
@@ -133,6 +134,12 @@ struct Job {
   uint32_t* left = nullptr;             // [tile][64 rows of P][NT / 32]: bit c: column c is left to plain_tiles
   int* status = nullptr;
 };
+
+// bytes of one step of tile t of the magnitudes; where the tile begins
+__device__ __forceinline__ int mag_step(const Side& s, int t) { return min(kMagTile, (s.rows - t * kMagTile + 7) / 8 * 8) * (2 * kMagK); }
+__device__ __forceinline__ unsigned char* mag_tile(const Side& s, int nms, int batch, int t) {
+  return s.mag + (long long)nms * (2 * kMagK) * ((long long)batch * ((s.rows + 7) / 8 * 8) + (long long)t * kMagTile);
+}
 
 __device__ __forceinline__ long long side_row(const Side& s, int r) {
   const int rq = div_by(r, s.rdiv);
@@ -280,9 +287,9 @@ __device__ void pack_tile(const Side& s, const Job& j, long long t) {
   // the padding rows of the last tile stay unwritten: a row of digits meets only its own row of the output
   if (!p.row_ok) return;
   const int mrow = p.tile * kRows + p.row;
-  unsigned char* mag = s.mag + ((long long)p.pb * s.mtiles + mrow / kMagTile) * j.nms * (long long)kMagStep +
-                       (mrow % kMagTile >> 3) * 256 + (mrow & 7) * 16;
-  auto mag_at = [&](int g) { return reinterpret_cast<uint2*>(mag + (long long)(g >> 2) * kMagStep + (g >> 1 & 1) * 128 + (g & 1) * 8); };
+  const int mstep = mag_step(s, mrow / kMagTile);
+  unsigned char* mag = mag_tile(s, j.nms, p.pb, mrow / kMagTile) + (mrow % kMagTile >> 3) * 256 + (mrow & 7) * 16;
+  auto mag_at = [&](int g) { return reinterpret_cast<uint2*>(mag + (long long)(g >> 2) * mstep + (g >> 1 & 1) * 128 + (g & 1) * 8); };
   if (p.k1 == j.nks && (j.nks & 1) && p.grp < 2) *mag_at(2 * j.nks + p.grp) = make_uint2(0u, 0u);   // half a step beyond K
   for (int g = 2 * p.k0 + p.grp; g < 2 * p.k1; g += kGroups) {
     unsigned long long u[8];
@@ -604,6 +611,8 @@ __device__ __forceinline__ double to_fp64(long long hi, uint32_t lo, int e) {
 // so from below), two tiles in flight. Long K in two passes: 512 of its k spread evenly, which is enough for every output
 // of most tiles, then all of it for the other tiles (P0 of a 2x2x2 solid, 13 tiles of K = 5408: 50 us for all of it).
 // Bound: launch and copy latency; 1/70 of the digit MMAs and 1/30 of their bytes, and one load and compare an output.
+// Steps lie behind one another in shared memory as in global memory; where a tile has fewer than 128 rows an MMA reads on
+// into the next ones, for rows and columns that are not there.
 constexpr int kMagStages = 3, kMagPer = 4;           // stages, steps of a stage
 constexpr int kMagFirst = 8;                         // stages of a first pass (512 k)
 constexpr int kMagThreads = 192;                     // producer, MMA, four epilogue warps
@@ -671,24 +680,16 @@ __global__ void __launch_bounds__(kMagThreads) oz64_bound_kernel(const __grid_co
         for (int tile = blockIdx.x; tile < total && !*abort_flag; tile += gridDim.x, ++own) {
           if (pass && !(map[own >> map_sh >> 5] >> (own >> map_sh & 31) & 1)) continue;
           const int b = tile / per_batch, w = tile - b * per_batch, pt = w / j.q.mtiles, qt = w - pt * j.q.mtiles;
-          const unsigned char* a = j.p.mag + ((long long)packed(j.p, b, j.ni) * j.p.mtiles + pt) * j.nms * (long long)kMagStep;
-          const unsigned char* q = j.q.mag + ((long long)packed(j.q, b, j.ni) * j.q.mtiles + qt) * j.nms * (long long)kMagStep;
-          const uint32_t pb = min(kMagTile, (j.p.rows - pt * kMagTile + 7) / 8 * 8) * (2 * kMagK);   // bytes of a step that hold rows
-          const uint32_t qb = min(kMagTile, (j.q.rows - qt * kMagTile + 7) / 8 * 8) * (2 * kMagK);
+          const unsigned char* a = mag_tile(j.p, j.nms, packed(j.p, b, j.ni), pt);
+          const unsigned char* q = mag_tile(j.q, j.nms, packed(j.q, b, j.ni), qt);
+          const int pb = mag_step(j.p, pt), qb = mag_step(j.q, qt);
           for (int i = 0; i < ns; ++i, ++step) {
             const int st = step % kMagStages, s = stage_at(i), nk = steps_of(s);
             if (!mbar_wait(&empty[st], ((step / kMagStages) & 1) ^ 1, abort_flag, j.status, 25)) break;
             uint8_t* sa = smem + (size_t)st * 2 * kHalf;
             mbar_expect_tx(&full[st], nk * (pb + qb));
-            if (pb + qb == 2 * kMagStep) {
-              bulk_load(sa, a + (long long)s * kHalf, nk * kMagStep, &full[st]);
-              bulk_load(sa + kHalf, q + (long long)s * kHalf, nk * kMagStep, &full[st]);
-            } else {     // only the 8-row groups that hold rows (small matrices: a quarter of the reads)
-              for (int k = 0; k < nk; ++k) {
-                bulk_load(sa + k * kMagStep, a + (long long)s * kHalf + k * kMagStep, pb, &full[st]);
-                bulk_load(sa + kHalf + k * kMagStep, q + (long long)s * kHalf + k * kMagStep, qb, &full[st]);
-              }
-            }
+            bulk_load(sa, a + (long long)s * kMagPer * pb, nk * pb, &full[st]);
+            bulk_load(sa + kHalf, q + (long long)s * kMagPer * qb, nk * qb, &full[st]);
           }
         }
       }
@@ -698,6 +699,7 @@ __global__ void __launch_bounds__(kMagThreads) oz64_bound_kernel(const __grid_co
         int own = 0;
         for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x, ++own) {
           if (pass && !(map[own >> map_sh >> 5] >> (own >> map_sh & 31) & 1)) continue;
+          const int w = tile % per_batch, pb = mag_step(j.p, w / j.q.mtiles), qb = mag_step(j.q, w % j.q.mtiles);
           const uint32_t buf = n & 1;
           if (!mbar_wait(&acc_empty[buf], ((n >> 1) & 1) ^ 1, abort_flag, j.status, 26)) { ok = false; break; }
           ++n;
@@ -708,7 +710,7 @@ __global__ void __launch_bounds__(kMagThreads) oz64_bound_kernel(const __grid_co
             tc_fence_after();
             const uint64_t sa = desc0 + (uint64_t)((st * 2 * kHalf) >> 4);
             for (int k = 0; k < nk; ++k)
-              mma_bf16(tmem + buf * kMagTile, sa + (uint64_t)(k * kMagStep >> 4), sa + (uint64_t)((kHalf + k * kMagStep) >> 4),
+              mma_bf16(tmem + buf * kMagTile, sa + (uint64_t)(k * pb >> 4), sa + (uint64_t)((kHalf + k * qb) >> 4),
                        idesc_bf16(kMagTile, false), i == 0 && k == 0 ? 0u : 1u);
             mma_commit(&empty[st]);
           }
@@ -1156,7 +1158,7 @@ size_t oz64_bytes(long long p_rows, long long q_rows, int K) {
   // digit tiles (64-row Q tiles bound the padding) and scales; magnitudes; a bit for every output
   const long long extra = 8 + (nks >= 2 * kSegSteps ? 8 * kMaxSegs : 0), mag = (nks + 1) / 2 * 2 * kMagK;
   return (size_t)(up(p_rows, kPTile) * (nks * 512 + extra) + up(q_rows, 64) * (nks * 256 + extra) +
-                  (up(p_rows, kMagTile) + up(q_rows, kMagTile)) * mag + up(p_rows, kPTile) * up(q_rows, 64) / 8 + 1024);
+                  (up(p_rows, 8) + up(q_rows, 8)) * mag + up(p_rows, kPTile) * up(q_rows, 64) / 8 + 1024);
 }
 
 // Where digits pay: below 8 complex k most of a k-step is padding, and tiny products (under 2^13
@@ -1209,8 +1211,8 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
   const long long row_extra = 8 + (j.nks >= 2 * kSegSteps ? 8 * kMaxSegs : 0);
   const long long pb = (long long)j.nks * 512 + row_extra, qb = (long long)j.nks * 256 + row_extra, mb = j.nms * 2LL * kMagK;
   const long long W = (long long)g.ws->bytes - 1024;
-  auto p_bytes = [&](long long r) { return up(r, kPTile) * pb + up(r, kMagTile) * mb; };
-  auto q_bytes = [&](long long r) { return up(r, nt) * qb + up(r, kMagTile) * mb; };
+  auto p_bytes = [&](long long r) { return up(r, kPTile) * pb + up(r, 8) * mb; };
+  auto q_bytes = [&](long long r) { return up(r, nt) * qb + up(r, 8) * mb; };
   auto need = [&](long long prow, long long qrow, long long o, long long i) {
     return p_bytes(prow) * (j.p.dep_o ? o : 1) * (j.p.dep_i ? i : 1) + q_bytes(qrow) * (j.q.dep_o ? o : 1) * (j.q.dep_i ? i : 1) +
            o * i * (up(prow, kPTile) * up(qrow, nt) / 8);
@@ -1253,8 +1255,8 @@ int zgemm_oz64(const ZGemm& g, void* stream, bool* done) {
           j.p.dst = m;
           j.q.dst = m + pn * j.nks * 512;
           j.p.mag = j.q.dst + qn * j.nks * 256;
-          j.q.mag = j.p.mag + (long long)j.p.no * j.p.ni * j.p.mtiles * j.nms * kMagStep;
-          j.p.scale = reinterpret_cast<double*>(j.q.mag + (long long)j.q.no * j.q.ni * j.q.mtiles * j.nms * kMagStep);
+          j.q.mag = j.p.mag + (long long)j.p.no * j.p.ni * up(j.p.rows, 8) * mb;
+          j.p.scale = reinterpret_cast<double*>(j.q.mag + (long long)j.q.no * j.q.ni * up(j.q.rows, 8) * mb);
           j.q.scale = j.p.scale + pn;
           // long rows are packed in segments where the row tiles alone leave SMs idle (8 blocks an SM)
           const long long blocks = (long long)j.p.no * j.p.ni * j.p.tiles + (long long)j.q.no * j.q.ni * j.q.tiles;
