@@ -120,6 +120,7 @@ using namespace gwi;
 struct gw_ctx {
   gw_config cfg{};
   cudaStream_t stream = nullptr;
+  bool digits_on_top = false;             // create_ctx
   bool dry = false;                       // size-only build: count bytes, allocate and copy nothing
   int nk = 0, nao = 0, naux = 0, ntau = 0, nwb = 0, nwf = 0, nt = 1;
   long long nao2 = 0, naux2 = 0, pair = 0;
@@ -625,16 +626,17 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
     if (cfg->precision == GW_FP64) {
       // The digits of the contractions take three times their intermediates. Both share the memory that the
       // intermediates alone would take at the full tau batch, given or automatic (64 MiB where that is less), so the
-      // nodes taken at a time are fewer. More digits than fit are made in pieces, with the same result. A batch
+      // nodes taken at a time are fewer (digits_on_top: as much again for the digits). More digits than fit are made in pieces, with the same result. A batch
       // whose digits all fit P(i Omega), which is idle then, keeps its nodes.
       const double dig_t = (double)oz64_bytes(c->naux, c->naux, nk * (int)c->nao2);
       const double most = std::max(dig_t, (double)nk * oz64_bytes(c->nao, c->nao, c->naux * c->nao));   // P0's or Sigma's
       const double budget = std::max(c->nt * per_t, 67108864.0);
       const double pw = std::min(16.0 * nk * c->nwb * c->naux2, 4294967296.0);
       // (a sixteenth is left for the partial sums of products that split K)
-      if (cfg->tau_chunk <= 0 || pw < c->nt * most)
+      const bool on_top = c->digits_on_top && cfg->tau_chunk > 0;
+      if (!on_top && (cfg->tau_chunk <= 0 || pw < c->nt * most))
         c->nt = std::max(1, std::min(c->nt, (int)(budget * 15 / 16 / (per_t + dig_t))));
-      c->oz_bytes = (size_t)std::min(c->nt * most + budget / 16, std::max(budget - c->nt * per_t, 0.0));
+      c->oz_bytes = (size_t)std::min(c->nt * most + budget / 16, std::max(budget - (on_top ? 0.0 : c->nt * per_t), 0.0));
       if ((rc = dev_alloc(c, &c->work, (size_t)c->nt * 2 * nk * c->pair)) != GW_OK) break;
       if (cfg->v_packed && (rc = dev_alloc(c, &c->Vfull, (size_t)nk * nk * c->pair)) != GW_OK) break;
     }
@@ -722,10 +724,11 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
 
 CtxInfo ctx_info(const gw_ctx* c) { return CtxInfo{c->stream, c->nk, c->ntau, c->nao, c->nwf, c->cfg.mu}; }
 
-size_t job_device_bytes(const gw_config* cfg) {
+size_t job_device_bytes(const gw_config* cfg, bool digits_on_top) {
   if (!config_ok(cfg)) return 0;
   gw_ctx c;
   c.dry = true;
+  c.digits_on_top = digits_on_top;
   if (ctx_build(&c, cfg) != GW_OK) return 0;
   const size_t nk = (size_t)cfg->nk[0] * cfg->nk[1] * cfg->nk[2], nao2 = (size_t)cfg->nao * cfg->nao;
   // V, H (and an overlap of its size), G and the Sigma output of the job, and the loop's buffers
@@ -736,16 +739,13 @@ size_t job_device_bytes(const gw_config* cfg) {
          scgw_device_bytes(cfg, &o);
 }
 
-}  // namespace gwi
-
-extern "C" {
-
-int gw_create(gw_ctx** out, const gw_config* cfg, void* cuda_stream) {
+int create_ctx(gw_ctx** out, const gw_config* cfg, void* cuda_stream, bool digits_on_top) {
   if (!out || !cfg) return fail(GW_EINVAL, "gw_create: null argument");
   *out = nullptr;
   if (!config_ok(cfg)) return fail(GW_EINVAL, "gw_create: configuration out of range");
   gw_ctx* c = new gw_ctx();
   c->stream = (cudaStream_t)cuda_stream;
+  c->digits_on_top = digits_on_top;
   const int rc = ctx_build(c, cfg);
   if (rc != GW_OK) {
     free_ctx(c);
@@ -754,6 +754,12 @@ int gw_create(gw_ctx** out, const gw_config* cfg, void* cuda_stream) {
   *out = c;
   return GW_OK;
 }
+
+}  // namespace gwi
+
+extern "C" {
+
+int gw_create(gw_ctx** out, const gw_config* cfg, void* cuda_stream) { return create_ctx(out, cfg, cuda_stream, false); }
 
 int gw_destroy(gw_ctx* ctx) {
   if (!ctx) return GW_OK;

@@ -36,6 +36,7 @@ struct gw_batch {
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   std::vector<cudaEvent_t> ev;           // fork event, one join event per stream
   std::vector<const gw_c128*> V;
+  std::vector<char> planned;             // the batch chose the system's tau batch, by its bytes with digits on top
   std::vector<int> max_chunk;            // largest tau batch within each system's budget share
   // captured graph and the pointers it was captured with
   cudaGraphExec_t exec = nullptr;
@@ -82,11 +83,12 @@ void fit_tau_batches(gw_batch* b, size_t budget) {
   for (int i = 0; i < b->n; ++i) {
     gw_config t = b->cfg[i];
     t.tau_chunk = t.ntau;
-    need[i] = (double)job_device_bytes(&t);
+    need[i] = (double)job_device_bytes(&t, b->cfg[i].tau_chunk == 0);
     total += need[i];
   }
   const double scale = total > 0.0 ? std::min(1.0, (double)budget / total) : 1.0;
   b->max_chunk.assign(b->n, 0);
+  b->planned.assign(b->n, 0);
   for (int i = 0; i < b->n; ++i) {
     gw_config& c = b->cfg[i];
     if (c.tau_chunk != 0) {
@@ -98,13 +100,14 @@ void fit_tau_batches(gw_batch* b, size_t budget) {
     for (int d = 1; d <= c.ntau; ++d) {
       gw_config t = c;
       t.tau_chunk = (c.ntau + d - 1) / d;
-      const size_t bytes = job_device_bytes(&t);
+      const size_t bytes = job_device_bytes(&t, true);
       if (bytes != 0 && (double)bytes <= share) {
         chosen = t.tau_chunk;
         break;
       }
     }
     c.tau_chunk = chosen;
+    b->planned[i] = 1;
     b->max_chunk[i] = chosen;
   }
 }
@@ -120,7 +123,7 @@ int create_contexts(gw_batch* b) {
   for (int i = 0; i < b->n; ++i) {
     if (b->ctx[i]) gw_destroy(b->ctx[i]);
     b->ctx[i] = nullptr;
-    GW_TRY_BATCH(gw_create(&b->ctx[i], &b->cfg[i], b->streams[b->lane[i]]));
+    GW_TRY_BATCH(create_ctx(&b->ctx[i], &b->cfg[i], b->streams[b->lane[i]], b->planned[i]));
     if (b->V[i]) GW_TRY_BATCH(gw_set_coulomb(b->ctx[i], b->V[i]));
   }
   drop_graph(b);
@@ -350,7 +353,7 @@ int gw_batch_autotune(gw_batch* b, const gw_c128* const* G_dev, gw_c128* const* 
     *ms = 1e30f;
     cudaStream_t s = b->streams[b->lane[i]];
     gw_ctx* ctx = nullptr;
-    if (gw_create(&ctx, &cfg, s) != GW_OK) return GW_OK;   // a candidate that does not fit is skipped
+    if (create_ctx(&ctx, &cfg, s, b->planned[i]) != GW_OK) return GW_OK;   // a candidate that does not fit is skipped
     if (gw_set_coulomb(ctx, b->V[i]) == GW_OK && gw_sigma_eval(ctx, G_dev[i], Sig_dev[i]) == GW_OK &&
         cudaEventRecord(e0, s) == cudaSuccess && gw_sigma_eval(ctx, G_dev[i], Sig_dev[i]) == GW_OK &&
         cudaEventRecord(e1, s) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess)
@@ -364,7 +367,7 @@ int gw_batch_autotune(gw_batch* b, const gw_c128* const* G_dev, gw_c128* const* 
     const gw_config &x = b->cfg[i], &y = b->cfg[j];
     return std::equal(x.nk, x.nk + 3, y.nk) && x.nao == y.nao && x.naux == y.naux && x.ntau == y.ntau &&
            x.precision == y.precision && x.v_slices == y.v_slices && x.v_packed == y.v_packed &&
-           x.slice_pass == y.slice_pass && b->max_chunk[i] == b->max_chunk[j];
+           x.slice_pass == y.slice_pass && b->max_chunk[i] == b->max_chunk[j] && b->planned[i] == b->planned[j];
   };
   std::vector<int> done;
   int rc = GW_OK;

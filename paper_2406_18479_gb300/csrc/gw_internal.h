@@ -40,7 +40,10 @@ struct NvtxRange {
 // Device bytes of one scGW job: its context's workspaces (counted by running the
 // context build in size-only mode) plus V, H, G and two Sigma buffers. 0 for an
 // invalid configuration.
-size_t job_device_bytes(const gw_config* cfg);
+size_t job_device_bytes(const gw_config* cfg, bool digits_on_top = false);
+// gw_create; digits_on_top: an FP64 context takes the digits of a given tau batch on top of its intermediates, for a
+// caller that counts its bytes (job_device_bytes with the same flag) against a budget of its own
+int create_ctx(gw_ctx** out, const gw_config* cfg, void* cuda_stream, bool digits_on_top);
 
 // ---- kernel timing and launch counting (gw_api.cu)
 //
