@@ -1005,7 +1005,7 @@ namespace {
 // The exchange term as two digit products over all (k, k') of a group of k: X = V^{kk'} gamma^{k'} and
 // its contraction with V^{k'k} over (Q, b), the partial sums over k' (and pieces of Q) reduced in order.
 // The FP64 pipe takes 16 nao^3 flops per (k, k', Q): 36.2 ms on the 3x3x3 solid at nao = 26 (41 GFLOP);
-// this way 12.1, half of it packing. Below 2^26 multiply-adds in all (half a millisecond on the FP64
+// this way 13.1, half of it packing. Below 2^26 multiply-adds in all (half a millisecond on the FP64
 // pipe) the six launches and their long packed rows cost more than they save. X and, with a packed
 // V, the unpacked blocks lie in P~ and P0 (not in use outside an evaluation), which hold them for at
 // least one k where ntau naux >= 2 nao^2; the same rule for a full V keeps the two layouts' results

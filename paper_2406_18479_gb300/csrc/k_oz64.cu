@@ -27,8 +27,8 @@
 // Bound: the L2 reads of the digit tiles at long K (48 KB per k-step of a 128 x 64 tile, 5.5 TB/s), the
 // epilogue's three FP64 operations an output at short K. 27 TFLOP/s of complex products at long K (R of a
 // molecule, nao = 45) and 16 where the output is as large as the work (transforms), against 0.7..1.1 on
-// the FP64 pipe. P0 of a 2x2x2 solid (nao = 26, naux = 104, 80 nodes): 313 -> 21.3 ms; Sigma of a molecule
-// (nao = 45): 76.9 -> 5.1 ms; the two transforms of a 3x3x3 solid (naux = 200, 100 nodes): 198 -> 19 ms with
+// the FP64 pipe. P0 of a 2x2x2 solid (nao = 26, naux = 104, 80 nodes): 313 -> 21.9 ms; Sigma of a molecule
+// (nao = 45): 76.9 -> 5.3 ms; the two transforms of a 3x3x3 solid (naux = 200, 100 nodes): 198 -> 19 ms with
 // their packing. Error against 64-bit references on these: 2e-16 and 4e-16 (FP64 pipe: 3e-15 and 6e-15).
 //
 // Rows with a non-finite element, or whose scale lies outside 2^+-480 (where the scaled product
@@ -609,7 +609,7 @@ __device__ __forceinline__ double to_fp64(long long hi, uint32_t lo, int e) {
 
 // S of every output: magnitudes of 128 rows of P times 128 rows of Q, summed over K in one FP32 accumulator (truncated,
 // so from below), two tiles in flight. Long K in two passes: 512 of its k spread evenly, which is enough for every output
-// of most tiles, then all of it for the other tiles (P0 of a 2x2x2 solid, 13 tiles of K = 5408: 50 us for all of it).
+// of most tiles, then all of it for the other tiles (P0 of a 2x2x2 solid, 13 tiles of K = 5408: 10 us, 50 for all of it).
 // Bound: launch and copy latency; 1/70 of the digit MMAs and 1/30 of their bytes, and one load and compare an output.
 // Steps lie behind one another in shared memory as in global memory; where a tile has fewer than 128 rows an MMA reads on
 // into the next ones, for rows and columns that are not there.
