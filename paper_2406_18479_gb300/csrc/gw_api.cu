@@ -126,6 +126,7 @@ struct gw_ctx {
   long long nao2 = 0, naux2 = 0, pair = 0;
   double2 *Fb = nullptr, *Bb = nullptr, *Ff = nullptr, *Bf = nullptr;
   int *Fbe = nullptr, *Bbe = nullptr, *Ffe = nullptr, *Bfe = nullptr;   // powers of two of their columns (ZGemm::kexp)
+  int* vexp = nullptr;                    // FP64: sizes of V per auxiliary function (ZGemm::kexp of R)
   double* wf = nullptr;                   // fermionic frequencies (device)
   long long* tabs = nullptr;              // 6 tables [nq][nk]
   long long *tab_kkpq = nullptr, *tab_kpqk = nullptr, *tab_gkpq = nullptr;
@@ -223,7 +224,7 @@ int cuda_check(const char* what) {
 void free_ctx(gw_ctx* c) {
   if (!c) return;
   mixed_destroy(c->mixed);
-  void* ptrs[] = {c->Fb, c->Bb, c->Ff, c->Bf, c->Fbe, c->Bbe, c->Ffe, c->Bfe, c->wf, c->tabs, c->mq_dev, c->wlist, c->wlist_q, c->work, c->P0t, c->Pw,
+  void* ptrs[] = {c->Fb, c->Bb, c->Ff, c->Bf, c->Fbe, c->Bbe, c->Ffe, c->Bfe, c->vexp, c->wf, c->tabs, c->mq_dev, c->wlist, c->wlist_q, c->work, c->P0t, c->Pw,
                   c->Pt, c->dyson_ws, c->status, c->maxdiff, c->nonfinite, c->wbeta, c->gamma, c->rho,
                   c->xinf, c->scal, c->gw_w, c->heff, c->gf2_ws, c->Vfull, c->cw_tmp, c->oz_mem, c->oz_small, c->oz_count};
   for (void* p : ptrs)
@@ -370,6 +371,11 @@ int self_energy_fp64(gw_ctx* c, const double2* G, const double2* Pt, double2* Si
         g.ba.bs_out = c->naux2;
         g.B = c->V; g.vb.rs_in = 1; g.vb.ks_in = nao2; g.bb.tab = c->tab_kmqk + (long long)q * nk;
         g.C = Rbuf; g.vc.rs_in = nao2; g.vc.ks_in = 1; g.bc.bs_in = pair; g.bc.bs_out = (long long)nk * pair;
+        // P~ is near a multiple of the identity where screening is strong, while V falls with Q': unbalanced, the large
+        // elements of V meet the small ones of P~ (nao = 52, naux = 400 solid: most outputs left to the FP64 pipe, R
+        // of an evaluation 89 ms, balanced 30; 26 without any check)
+        g.kexp = c->vexp;
+        g.kexp_a = 1;
         g.slot = SLOT_R_FP64;
         g.ws = &c->oz;
         GW_TRY(zgemm_fp64(g, c->stream));
@@ -638,6 +644,7 @@ int ctx_build(gw_ctx* c, const gw_config* cfg) {
         c->nt = std::max(1, std::min(c->nt, (int)(budget * 15 / 16 / (per_t + dig_t))));
       c->oz_bytes = (size_t)std::min(c->nt * most + budget / 16, std::max(budget - (on_top ? 0.0 : c->nt * per_t), 0.0));
       if ((rc = dev_alloc(c, &c->work, (size_t)c->nt * 2 * nk * c->pair)) != GW_OK) break;
+      if ((rc = dev_alloc(c, &c->vexp, (size_t)c->naux)) != GW_OK) break;
       if (cfg->v_packed && (rc = dev_alloc(c, &c->Vfull, (size_t)nk * nk * c->pair)) != GW_OK) break;
     }
     if ((rc = dev_alloc(c, &c->P0t, (size_t)nk * c->ntau * c->naux2)) != GW_OK) break;
@@ -846,6 +853,8 @@ int gw_set_coulomb(gw_ctx* ctx, const gw_c128* V_dev) {
     ctx->Vp = nullptr;
     if (ctx->mixed) GW_TRY(mixed_set_coulomb(ctx->mixed, V));
   }
+  // (of V as it is now: V changed in place later keeps its results, more of them by way of the FP64 pipe)
+  if (!ctx->mixed) GW_TRY(aux_exponents_fp64(ctx->V, (long long)ctx->nk * ctx->nk, ctx->naux, (int)ctx->nao2, ctx->vexp, ctx->stream));
   ctx->coulomb = true;
   return GW_OK;
 }

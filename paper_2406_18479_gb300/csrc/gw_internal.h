@@ -179,6 +179,8 @@ struct VPairs {
   int fixed = -1;   // >= 0: the pairs (fixed, 0..nk-1), then (0..nk-1, fixed)
   int k1[4] = {0, 0, 0, 0}, k2[4] = {0, 0, 0, 0};
 };
+// out[Q] (device, naux ints): as ZGemm::kexp takes it, of the elements of V[blocks][naux][nao2]
+int aux_exponents_fp64(const double2* V, long long blocks, int naux, int nao2, int* out, void* stream);
 inline long long packed_pairs(int nk) { return (long long)nk * (nk + 1) / 2; }
 int unpack_v_fp64(const double2* Vp, int nk, int nao, long long pair, const VPairs& L, int nblocks, double2* dst,
                   void* stream);

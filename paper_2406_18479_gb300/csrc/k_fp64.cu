@@ -834,6 +834,22 @@ __device__ __forceinline__ double2 v_load(const double2* V, int k1, int k2, int 
 // dst[b] = V^{k1 k2} (full layout [naux][nao][nao]) from the packed V, for the blocks b of a list:
 // pairs decoded from full-layout offsets tab[b] = (k1 nk + k2) pair, or every pair in order
 // (all = 1), or up to four given pairs.
+// out[Q] = the largest biased exponent of |re|, |im| of V[block][Q][nao2] over all blocks (out zero before). Bound: HBM, V
+// read once.
+__global__ void __launch_bounds__(256) aux_exponents_kernel(const double2* __restrict__ V, long long blocks, int naux, int nao2,
+                                                            int* out) {
+  for (long long s = blockIdx.x; s < blocks * naux; s += gridDim.x) {
+    const double2* v = V + s * nao2;
+    int m = 0;
+    for (int e = threadIdx.x; e < nao2; e += blockDim.x) {
+      const double2 x = v[e];
+      m = max(m, max(__double2hiint(x.x) & 0x7FFFFFFF, __double2hiint(x.y) & 0x7FFFFFFF) >> 20);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(&out[s % naux], m);
+  }
+}
+
 __global__ void unpack_v_kernel(const double2* __restrict__ Vp, int nk, int nao, long long pair, VPairs L,
                                 int nblocks, double2* __restrict__ dst) {
   const long long n2 = (long long)nao * nao;
@@ -1353,6 +1369,15 @@ int exchange_fp64(const double2* V, const double2* gamma, double2* part, double2
            32.0 * (double)nk * nk * naux * n2);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "exchange launch: %s", cudaGetErrorString(e));
+}
+
+int aux_exponents_fp64(const double2* V, long long blocks, int naux, int nao2, int* out, void* stream) {
+  cudaMemsetAsync(out, 0, (size_t)naux * sizeof(int), (cudaStream_t)stream);
+  prof_begin(SLOT_ELEMENTWISE, (cudaStream_t)stream);
+  aux_exponents_kernel<<<(unsigned)std::min<long long>(blocks * naux, 8 * 152), 256, 0, (cudaStream_t)stream>>>(V, blocks, naux, nao2, out);
+  prof_end(SLOT_ELEMENTWISE, (cudaStream_t)stream, 0.0, 16.0 * (double)blocks * naux * nao2);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? GW_OK : fail(GW_ECUDA, "aux_exponents launch: %s", cudaGetErrorString(e));
 }
 
 int unpack_v_fp64(const double2* Vp, int nk, int nao, long long pair, const VPairs& L, int nblocks, double2* dst,
